@@ -43,83 +43,338 @@ __device__ __forceinline__ float epilogue(const Epi& e, int m, int n, float v) {
     return v;
 }
 
-template <int BM, int BN, int BK, int NT>
-__device__ __forceinline__ void load_tiles(const Seg& s, int m0, int n0, int k0, int M, int N,
-                                           float (*As)[BM + 4], float (*Bs)[BN + 4]) {
-    const int tid = threadIdx.x;
-#pragma unroll
-    for (int r = 0; r < (BM * BK) / NT; ++r) {
-        const int e = tid + r * NT;
-        int mm, kk;
-        if (s.sak == 1) { mm = e / BK; kk = e % BK; } else { mm = e % BM; kk = e / BM; }
-        const int m = m0 + mm, k = k0 + kk;
-        As[kk][mm] = (m < M && k < s.K) ? __ldg(s.A + (int64_t)m * s.sam + (int64_t)k * s.sak) : 0.0f;
-    }
-#pragma unroll
-    for (int r = 0; r < (BN * BK) / NT; ++r) {
-        const int e = tid + r * NT;
-        int kk, nn;
-        if (s.sbn == 1) { kk = e / BN; nn = e % BN; } else { kk = e % BK; nn = e / BK; }
-        const int n = n0 + nn, k = k0 + kk;
-        Bs[kk][nn] = (n < N && k < s.K) ? __ldg(s.B + (int64_t)k * s.sbk + (int64_t)n * s.sbn) : 0.0f;
-    }
+// One 4-byte (or 16-byte) asynchronous copy global -> shared; bytes beyond `src` are zeros.
+__device__ __forceinline__ void cp_async4(uint32_t dst, const float* src, bool in) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(in ? 4 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async16(uint32_t dst, const float* src, int bytes) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void cp_async_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-// C tile [BM x BN] per block, [TM x TN] per thread (rows ty + i*BM/TM, columns
-// tx + j*BN/TN).  Every output sums its products in increasing k (segment 0, then
-// segment 1) with one FMA each, whatever the tile shape, so all tiles give the same bits.
+// d = a * b + d on two packed floats, each rounded as one FMA
+__device__ __forceinline__ void ffma2(uint64_t& d, uint64_t a, uint64_t b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ uint64_t swap2(uint64_t v) {
+    uint64_t r;
+    asm("{\n .reg .b32 lo, hi;\n mov.b64 {lo, hi}, %1;\n mov.b64 %0, {hi, lo};\n}" : "=l"(r) : "l"(v));
+    return r;
+}
+
+// Asynchronous copies of the BK x R operand tiles of one segment, element (k, r) of a tile to
+// dst[k * PITCH + r], from P(r, k) = P[r * sr + k * sk]; rows r0 + r >= rows and columns k >= K
+// read as zero.  Each thread's source pointer, its step between copies and which of its copies
+// lie inside the rows are worked out once per segment, so a tile costs an add and a copy each
+// (the address arithmetic per element had been two thirds of the issued instructions).
+//  - kTrans, k contiguous (activations, weights [n][k]): the tile is transposed on the way by
+//    4-byte copies, a warp taking 8 k x 4 rows: whole 32-byte sectors in, 32 different banks out;
+//  - kVec, rows contiguous (sr = 1) on 16-byte boundaries (the operands of the weight gradients,
+//    the weights of the data gradients): 16-byte copies;
+//  - kAny, other strides: 4-byte copies along r.
+enum { kTrans = 0, kVec = 1, kAny = 2 };
+template <int R, int BK, int PITCH, int NT> struct Loader {
+    static constexpr int KG = BK / 8;                           // kTrans: 8-column groups
+    static constexpr int RSTEP = 4 * (NT / 32) / KG;            // rows between a thread's copies
+    static constexpr int NTR = R / RSTEP;
+    static constexpr int KSTEP = NT / (R / 4);                  // kVec: columns between copies
+    static constexpr int NVEC = BK / KSTEP;
+    static_assert((NT / 32) % KG == 0 && R % RSTEP == 0 && NT % (R / 4) == 0 && BK % KSTEP == 0 && NTR <= 32,
+                  "copies must divide evenly");
+    const float* p;         // this thread's element of the tile at k = 0 (kAny: the segment)
+    int64_t step, sr, sk;
+    uint32_t dst, rows_in;  // byte offset in the tile; kTrans: which copies are inside, kVec: bytes, kAny: rows left
+    int k, K, mode;
+    __device__ __forceinline__ void init(const float* P, int64_t sr_, int64_t sk_, int r0, int rows, int K_) {
+        const int tid = threadIdx.x;
+        sr = sr_; sk = sk_; K = K_;
+        mode = sk == 1 ? kTrans : ((sr == 1 && (sk & 3) == 0 && (reinterpret_cast<uintptr_t>(P) & 15u) == 0) ? kVec : kAny);
+        if (mode == kTrans) {
+            const int w = tid >> 5, lane = tid & 31;
+            k = (w % KG) * 8 + (lane & 7);
+            const int r = (w / KG) * 4 + (lane >> 3);
+            p = P + (int64_t)(r0 + r) * sr + k;
+            step = (int64_t)RSTEP * sr;
+            dst = 4u * (uint32_t)(k * PITCH + r);
+            rows_in = 0;
+#pragma unroll
+            for (int i = 0; i < NTR; ++i) rows_in |= (uint32_t)(r0 + r + i * RSTEP < rows) << i;
+        } else if (mode == kVec) {
+            k = tid / (R / 4);
+            const int r = (tid % (R / 4)) * 4;
+            p = P + (int64_t)k * sk + r0 + r;
+            step = (int64_t)KSTEP * sk;
+            dst = 4u * (uint32_t)(k * PITCH + r);
+            rows_in = 4u * (uint32_t)min(max(rows - r0 - r, 0), 4);
+        } else {
+            k = 0; step = 0; dst = 0;
+            p = P + (int64_t)r0 * sr;
+            rows_in = (uint32_t)max(rows - r0, 0);
+        }
+    }
+    // the tile of columns k0 .. k0 + BK - 1 (a copy outside the matrix reads no bytes)
+    __device__ __forceinline__ void start(uint32_t base, int k0) const {
+        if (mode == kTrans) {
+            const float* q = p + k0;
+            const bool kin = k0 + k < K;
+            const uint32_t in = kin ? rows_in : 0u;
+#pragma unroll
+            for (int i = 0; i < NTR; ++i) {
+                cp_async4(base + dst + 4u * (uint32_t)(i * RSTEP), q, (in >> i) & 1u);
+                q += step;
+            }
+        } else if (mode == kVec) {
+            const float* q = p + (int64_t)k0 * sk;
+#pragma unroll
+            for (int i = 0; i < NVEC; ++i) {
+                cp_async16(base + dst + 4u * (uint32_t)(i * KSTEP * PITCH), q, k0 + k + i * KSTEP < K ? (int)rows_in : 0);
+                q += step;
+            }
+        } else {
+#pragma unroll 4
+            for (int e = threadIdx.x; e < BK * R; e += NT) {
+                const int kk = e / R, rr = e % R;
+                const bool in = (uint32_t)rr < rows_in && k0 + kk < K;
+                cp_async4(base + 4u * (uint32_t)(kk * PITCH + rr), in ? p + (int64_t)rr * sr + (int64_t)(k0 + kk) * sk : p,
+                          in);
+            }
+        }
+    }
+};
+
+// four consecutive outputs (m, n .. n + 3), all inside the matrix, every row 16-byte aligned
+__device__ __forceinline__ void epilogue_store4(const Epi& e, int m, int n, const float4 b, float4 v) {
+    if (e.bias) { v.x += b.x; v.y += b.y; v.z += b.z; v.w += b.w; }
+    if (e.res) {
+        const float4 r = *reinterpret_cast<const float4*>(e.res + (int64_t)m * e.ldr + n);
+        v.x += r.x; v.y += r.y; v.z += r.z; v.w += r.w;
+    }
+    if (e.relu) { v.x = fmaxf(v.x, 0.0f); v.y = fmaxf(v.y, 0.0f); v.z = fmaxf(v.z, 0.0f); v.w = fmaxf(v.w, 0.0f); }
+    if (e.mask) {
+        const float4 q = *reinterpret_cast<const float4*>(e.mask + (int64_t)m * e.ldm + n);
+        if (!(q.x > 0.0f)) v.x = 0.0f;
+        if (!(q.y > 0.0f)) v.y = 0.0f;
+        if (!(q.z > 0.0f)) v.z = 0.0f;
+        if (!(q.w > 0.0f)) v.w = 0.0f;
+    }
+    *reinterpret_cast<float4*>(e.C + (int64_t)m * e.ldc + n) = v;
+}
+__device__ __forceinline__ bool aligned16(const float* p, int64_t ld) {
+    return ((reinterpret_cast<uintptr_t>(p) & 15u) | (uint64_t)(ld & 3)) == 0;
+}
+
+// C tile [BM x BN] per block, [TM x TN] per thread: thread (ty, tx) of the (BM / TM) x
+// (BN / TN) grid has rows in groups of four and the columns tx * TN .. + TN - 1, so a warp
+// covers a strip of few columns, and a warp whose strip lies beyond the tile's columns skips
+// the arithmetic (the column tiles of a matrix are equally wide, in whole strips).
+// Bound: the FP32 FMA rate (75 TFLOP/s measured for packed or scalar FMAs from registers);
+// this kernel reaches 37 on 155,648 rows, 60 with its operand copies and barriers left out.
+// The products are packed pairs of FMAs, half the issue slots of scalar ones: row pair
+// (a0, a1) against column pair (b0, b1) and against (b1, b0) gives the 2 x 2 outputs with one
+// swap per column pair (duplicating each a instead cost two moves per row and 5 % of the
+// time).  STAGES operand tiles are in flight as asynchronous copies.
+// 20,011 rows through the network's 23 layers: 3.08 ms with scalar FMAs and a load, barrier,
+// compute, barrier loop; 1.73 ms now.  A 4,096-row 64 x 64 render: 0.92 -> 0.56 ms; a training
+// step of 1,000 rows (its weight gradients: 28 blocks over K = 1,000): 3.73 -> 1.41 ms.
+// Every output sums its products in increasing k (segment 0, then segment 1) with one FMA
+// each, whatever the tile shape, so all tiles give the same bits.
 // With splits > 1, block z takes the z-th contiguous run of the K tiles and writes its
 // partial sums to ws[z][m][n]; k_splitk_epi adds them in z order and applies the epilogue.
+template <int BM, int BN, int BK, int TM, int TN> struct GemmCfg {
+    static constexpr int RY = BM / TM, CX = BN / TN, NT = RY * CX;
+    static constexpr int PA = BM + 4, PB = BN + 4;
+    static constexpr int STAGE = BK * (PA + PB);                      // floats
+    static constexpr int FIT = 48 * 1024 / (STAGE * 4);
+    static constexpr int STAGES = FIT > 4 ? 4 : FIT;
+    static constexpr int STRIP = (32 / RY) * TN;                      // columns of a warp
+    // blocks per SM the registers are held to (the fastest of those tried for each tile)
+    static constexpr int BLOCKS = TM * TN == 64 ? (NT == 256 ? 2 : 3) : (BN == 64 && TN == 8 ? 4 : (BN == 64 ? 3 : 5));
+    static_assert(TM % 4 == 0 && TN % 4 == 0 && (RY == 8 || RY == 16) && STAGES >= 3, "vector reads, whole strips, three stages");
+};
+
 template <int BM, int BN, int BK, int TM, int TN>
-__global__ void __launch_bounds__((BM / TM) * (BN / TN))
-k_gemm(int M_host, const int* __restrict__ M_dev, int N, Seg s0, Seg s1, int nseg, Epi e, int splits,
-       float* __restrict__ ws) {
-    constexpr int NT = (BM / TM) * (BN / TN), CX = BN / TN, RY = BM / TM;
-    static_assert((BM * BK) % NT == 0 && (BN * BK) % NT == 0, "tile loads must divide evenly");
-    const int M = M_dev ? *M_dev : M_host;
-    const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
-    if (m0 >= M) return;
-    __shared__ float As[BK][BM + 4];
-    __shared__ float Bs[BK][BN + 4];
-    const int tx = threadIdx.x % CX, ty = threadIdx.x / CX;
-    float acc[TM][TN] = {};
+__device__ __forceinline__ void gemm_tile(float* sm, int M, int Mws, int N, int m0, int n0, int n1, int z,
+                                          const Seg& s0, const Seg& s1, int nseg, const Epi& e, int splits,
+                                          float* __restrict__ ws) {
+    using C = GemmCfg<BM, BN, BK, TM, TN>;
+    constexpr int NT = C::NT, PA = C::PA, PB = C::PB, ST = C::STAGES;
+    const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(sm);
+    // lane -> (ty, tx): bits 1-3 (1-4) are ty, the others tx.  A 16-byte shared-memory read of a
+    // warp whose address depends on both of a lane's two lowest bits takes four passes, else two
+    // (measured for every such map), so neither operand's address may hold both.
+    const int lane = threadIdx.x & 31;
+    const int ty = (lane >> 1) % C::RY;
+    const int tx = (int)(threadIdx.x / 32) * (32 / C::RY) + (C::RY == 16 ? lane & 1 : (lane & 1) | (lane >> 4) << 1);
     const int T0 = (s0.K + BK - 1) / BK;
     const int T = T0 + (nseg > 1 ? (s1.K + BK - 1) / BK : 0);
     const int per = (T + splits - 1) / splits;
-    const int tb = (int)blockIdx.z * per, te = min(T, tb + per);
-    for (int t = tb; t < te; ++t) {
-        const bool first = t < T0;
-        const Seg& s = first ? s0 : s1;
-        const int k0 = (first ? t : t - T0) * BK;
-        load_tiles<BM, BN, BK, NT>(s, m0, n0, k0, M, N, As, Bs);
+    const int tb = z * per, nt = max(0, min(T, tb + per) - tb);
+    const bool live = n0 + (int)(threadIdx.x / 32) * C::STRIP < n1;   // warp-uniform
+    uint64_t acc[TM][TN / 2];
+#pragma unroll
+    for (int i = 0; i < TM; ++i)
+#pragma unroll
+        for (int j = 0; j < TN / 2; ++j) acc[i][j] = 0ull;
+    Loader<BM, BK, PA, NT> la;
+    Loader<BN, BK, PB, NT> lb;
+    bool second = tb >= T0;
+    auto segment = [&](const Seg& s) {
+        la.init(s.A, s.sam, s.sak, m0, M, s.K);
+        lb.init(s.B, s.sbn, s.sbk, n0, N, s.K);
+    };
+    segment(second ? s1 : s0);
+    auto start = [&](int it) {
+        if (it < nt) {
+            const int t = tb + it;
+            if (!second && t >= T0) { second = true; segment(s1); }
+            const int k0 = (second ? t - T0 : t) * BK;
+            const uint32_t d = sbase + 4u * (uint32_t)((it % ST) * C::STAGE);
+            la.start(d, k0);
+            lb.start(d + 4u * (BK * PA), k0);
+        }
+        cp_async_commit();
+    };
+    for (int it = 0; it < ST - 1; ++it) start(it);
+    for (int it = 0; it < nt; ++it) {
+        cp_async_wait<ST - 2>();
         __syncthreads();
+        start(it + ST - 1);
+        if (!live) continue;
+        const float* As = sm + (it % ST) * C::STAGE + 4 * ty;
+        const float* Bs = sm + (it % ST) * C::STAGE + BK * PA + tx * TN;
 #pragma unroll
         for (int kk = 0; kk < BK; ++kk) {
-            float a[TM], b[TN];
+            uint64_t a[TM / 2], b[TN / 2];
 #pragma unroll
-            for (int i = 0; i < TM; ++i) a[i] = As[kk][ty + RY * i];
+            for (int i = 0; i < TM / 4; ++i)
+                *reinterpret_cast<ulonglong2*>(a + 2 * i) =
+                    *reinterpret_cast<const ulonglong2*>(As + kk * PA + 4 * C::RY * i);
 #pragma unroll
-            for (int j = 0; j < TN; ++j) b[j] = Bs[kk][tx + CX * j];
+            for (int j = 0; j < TN / 4; ++j)
+                *reinterpret_cast<ulonglong2*>(b + 2 * j) = *reinterpret_cast<const ulonglong2*>(Bs + kk * PB + 4 * j);
+#pragma unroll
+            for (int j = 0; j < TN / 2; ++j) {
+                const uint64_t bs = swap2(b[j]);
+#pragma unroll
+                for (int i = 0; i < TM / 2; ++i) {
+                    ffma2(acc[2 * i][j], a[i], b[j]);
+                    ffma2(acc[2 * i + 1][j], a[i], bs);
+                }
+            }
+        }
+    }
+    if (!live) return;
+    // acc[2p][q] = (C(2p, 2q), C(2p + 1, 2q + 1)), acc[2p + 1][q] = (C(2p, 2q + 1), C(2p + 1, 2q))
+    auto val = [&](int i, int j) {
+        const uint64_t v = acc[(i & ~1) + ((i ^ j) & 1)][j / 2];
+        return __uint_as_float((uint32_t)(i & 1 ? v >> 32 : v));
+    };
+    auto row_of = [&](int i) { return m0 + 4 * C::RY * (i / 4) + 4 * ty + (i & 3); };
+    const int nc = n0 + tx * TN;
+    if (splits > 1) {
+#pragma unroll
+        for (int i = 0; i < TM; ++i) {
+            const int m = row_of(i);
+            if (m >= M) continue;
+#pragma unroll
+            for (int j = 0; j < TN; ++j)
+                if (nc + j < n1) ws[((int64_t)z * Mws + m) * N + nc + j] = val(i, j);
+        }
+        return;
+    }
+    const bool vec = aligned16(e.C, e.ldc) && (!e.res || aligned16(e.res, e.ldr)) &&
+                     (!e.mask || (e.mcs == 1 && aligned16(e.mask, e.ldm))) && (!e.bias || aligned16(e.bias, 0));
+#pragma unroll
+    for (int j0 = 0; j0 < TN; j0 += 4) {
+        if (vec && nc + j0 + 3 < n1) {
+            const float4 b = e.bias ? *reinterpret_cast<const float4*>(e.bias + nc + j0) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int i = 0; i < TM; ++i)
+                if (row_of(i) < M)
+                    epilogue_store4(e, row_of(i), nc + j0, b, make_float4(val(i, j0), val(i, j0 + 1), val(i, j0 + 2), val(i, j0 + 3)));
+        } else {
 #pragma unroll
             for (int i = 0; i < TM; ++i)
 #pragma unroll
-                for (int j = 0; j < TN; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+                for (int j = j0; j < j0 + 4; ++j)
+                    if (row_of(i) < M && nc + j < n1)
+                        e.C[(int64_t)row_of(i) * e.ldc + nc + j] = epilogue(e, row_of(i), nc + j, val(i, j));
+        }
+    }
+}
+
+// columns [n0, n1) of column tile `x` of `tiles` equally wide ones (whole strips)
+__device__ __forceinline__ void column_range(int N, int tiles, int strip, int x, int& n0, int& n1) {
+    const int w = ((N + tiles - 1) / tiles + strip - 1) / strip * strip;
+    n0 = x * w;
+    n1 = min(N, n0 + w);
+}
+
+template <int BM, int BN, int BK, int TM, int TN>
+__global__ void __launch_bounds__(GemmCfg<BM, BN, BK, TM, TN>::NT, GemmCfg<BM, BN, BK, TM, TN>::BLOCKS)
+k_gemm(int M_host, const int* __restrict__ M_dev, int N, const __grid_constant__ Seg s0, const __grid_constant__ Seg s1,
+       int nseg, const __grid_constant__ Epi e, int splits, float* __restrict__ ws) {
+    using C = GemmCfg<BM, BN, BK, TM, TN>;
+    __shared__ __align__(16) float sm[C::STAGES * C::STAGE];
+    const int M = M_dev ? *M_dev : M_host;
+    const int m0 = blockIdx.y * BM;
+    int n0, n1;
+    column_range(N, (int)gridDim.x, C::STRIP, (int)blockIdx.x, n0, n1);
+    if (m0 >= M || n0 >= n1) return;
+    gemm_tile<BM, BN, BK, TM, TN>(sm, M, M_host, N, m0, n0, n1, (int)blockIdx.z, s0, s1, nseg, e, splits, ws);
+}
+
+// N = 1 (the output layer): one thread per row sums its K products in increasing k with one
+// FMA each, as a k_gemm output does; the block's 64 rows pass through shared memory in pieces
+// of 40 columns so the loads are coalesced.
+constexpr int kDotRows = 64, kDotK = 40;
+__global__ void __launch_bounds__(256) k_rowdot(int M_host, const int* __restrict__ M_dev,
+                                                const __grid_constant__ Seg s, const __grid_constant__ Epi e) {
+    __shared__ float As[2][kDotK][kDotRows + 1];
+    const int M = M_dev ? *M_dev : M_host;
+    const int m0 = blockIdx.x * kDotRows;
+    if (m0 >= M) return;
+    const int T = (s.K + kDotK - 1) / kDotK;
+    auto start = [&](int t) {
+        if (t < T) {
+            for (int i = threadIdx.x; i < kDotRows * kDotK; i += 256) {
+                const int kk = i % kDotK, mm = i / kDotK;
+                const bool in = m0 + mm < M && t * kDotK + kk < s.K;
+                cp_async4((uint32_t)__cvta_generic_to_shared(&As[t & 1][kk][mm]),
+                          in ? s.A + (int64_t)(m0 + mm) * s.sam + (int64_t)(t * kDotK + kk) * s.sak : s.A, in);
+            }
+        }
+        cp_async_commit();
+    };
+    float acc = 0.0f;
+    start(0);
+    for (int t = 0; t < T; ++t) {
+        start(t + 1);
+        cp_async_wait<1>();
+        __syncthreads();
+        if (threadIdx.x < kDotRows) {
+            const int kn = min(kDotK, s.K - t * kDotK);
+#pragma unroll 8
+            for (int kk = 0; kk < kn; ++kk)
+                acc = fmaf(As[t & 1][kk][threadIdx.x], __ldg(s.B + (int64_t)(t * kDotK + kk) * s.sbk), acc);
         }
         __syncthreads();
     }
-#pragma unroll
-    for (int i = 0; i < TM; ++i) {
-        const int m = m0 + ty + RY * i;
-        if (m >= M) continue;
-#pragma unroll
-        for (int j = 0; j < TN; ++j) {
-            const int n = n0 + tx + CX * j;
-            if (n >= N) continue;
-            if (splits > 1)
-                ws[((int64_t)blockIdx.z * M_host + m) * N + n] = acc[i][j];
-            else
-                e.C[(int64_t)m * e.ldc + n] = epilogue(e, m, n, acc[i][j]);
-        }
+    const int m = m0 + (int)threadIdx.x;
+    if (threadIdx.x < kDotRows && m < M) e.C[(int64_t)m * e.ldc] = epilogue(e, m, 0, acc);
+}
+
+// K = 1 (the output layer's data gradient): C(m, n) = epilogue(a(m) b(n))
+__global__ void k_outer(int M, int N, const __grid_constant__ Seg s, const __grid_constant__ Epi e) {
+    const int64_t total = (int64_t)M * N;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+        // a column-major mask is read along m
+        const int m = e.mcs == 1 ? (int)(i / N) : (int)(i % M), n = e.mcs == 1 ? (int)(i % N) : (int)(i / M);
+        e.C[(int64_t)m * e.ldc + n] =
+            epilogue(e, m, n, fmaf(__ldg(s.A + (int64_t)m * s.sam), __ldg(s.B + (int64_t)n * s.sbn), 0.0f));
     }
 }
 
@@ -187,12 +442,13 @@ Epi epi(float* C, int64_t ldc, const float* bias = nullptr, int relu = 0,
 // ---- tile shapes and the autotuner ----------------------------------------------------
 struct TileShape { int bm, bn, bk, tm, tn; };
 constexpr TileShape kTiles[] = {
-    {64, 64, 16, 4, 4},    // the default (no tuning)
-    {128, 64, 16, 8, 4},
-    {64, 128, 16, 4, 8},
+    {64, 64, 16, 4, 8},    // the default (no tuning)
+    {128, 64, 16, 8, 8},
+    {64, 128, 16, 8, 8},
     {128, 128, 8, 8, 8},
-    {32, 64, 16, 2, 4},
-    {128, 32, 16, 8, 2},
+    {32, 64, 16, 4, 4},
+    {128, 32, 16, 8, 4},
+    {32, 128, 16, 4, 8},
 };
 constexpr int kNumTiles = sizeof(kTiles) / sizeof(kTiles[0]);
 constexpr int kSplits[] = {1, 2, 4, 8, 16, 32};
@@ -202,7 +458,7 @@ template <int BM, int BN, int BK, int TM, int TN>
 void launch_tile(int M, const int* M_dev, int N, const Seg& s0, const Seg& s1, int nseg, const Epi& e,
                  int splits, float* ws, cudaStream_t s) {
     dim3 grid((N + BN - 1) / BN, (M + BM - 1) / BM, splits);
-    k_gemm<BM, BN, BK, TM, TN><<<grid, (BM / TM) * (BN / TN), 0, s>>>(M, M_dev, N, s0, s1, nseg, e, splits, ws);
+    k_gemm<BM, BN, BK, TM, TN><<<grid, GemmCfg<BM, BN, BK, TM, TN>::NT, 0, s>>>(M, M_dev, N, s0, s1, nseg, e, splits, ws);
 }
 
 rpnn_status launch_gemm(int tile, int splits, int M, const int* M_dev, int N, const Seg& s0, const Seg& s1,
@@ -210,12 +466,13 @@ rpnn_status launch_gemm(int tile, int splits, int M, const int* M_dev, int N, co
     const TileShape& t = kTiles[tile];
     if ((M + t.bm - 1) / t.bm > 65535) { set_error("GEMM with %d rows exceeds the grid limit", M); return RPNN_ERR_ARG; }
     switch (tile) {
-        case 0: launch_tile<64, 64, 16, 4, 4>(M, M_dev, N, s0, s1, nseg, e, splits, ws, s); break;
-        case 1: launch_tile<128, 64, 16, 8, 4>(M, M_dev, N, s0, s1, nseg, e, splits, ws, s); break;
-        case 2: launch_tile<64, 128, 16, 4, 8>(M, M_dev, N, s0, s1, nseg, e, splits, ws, s); break;
+        case 0: launch_tile<64, 64, 16, 4, 8>(M, M_dev, N, s0, s1, nseg, e, splits, ws, s); break;
+        case 1: launch_tile<128, 64, 16, 8, 8>(M, M_dev, N, s0, s1, nseg, e, splits, ws, s); break;
+        case 2: launch_tile<64, 128, 16, 8, 8>(M, M_dev, N, s0, s1, nseg, e, splits, ws, s); break;
         case 3: launch_tile<128, 128, 8, 8, 8>(M, M_dev, N, s0, s1, nseg, e, splits, ws, s); break;
-        case 4: launch_tile<32, 64, 16, 2, 4>(M, M_dev, N, s0, s1, nseg, e, splits, ws, s); break;
-        default: launch_tile<128, 32, 16, 8, 2>(M, M_dev, N, s0, s1, nseg, e, splits, ws, s); break;
+        case 4: launch_tile<32, 64, 16, 4, 4>(M, M_dev, N, s0, s1, nseg, e, splits, ws, s); break;
+        case 5: launch_tile<128, 32, 16, 8, 4>(M, M_dev, N, s0, s1, nseg, e, splits, ws, s); break;
+        default: launch_tile<32, 128, 16, 4, 8>(M, M_dev, N, s0, s1, nseg, e, splits, ws, s); break;
     }
     RPNN_CHECK_LAUNCH();
     if (splits > 1) {
@@ -302,6 +559,17 @@ rpnn_status tune(Ctx& c, const GemmKey& key, int M, const int* M_dev, int N, con
 rpnn_status gemm(Ctx* c, int M, const int* M_dev, int N, const Seg& s0, const Seg* s1, const Epi& e,
                  cudaStream_t s) {
     if (M <= 0 || N <= 0) return RPNN_OK;
+    if (N == 1 && !s1) {
+        k_rowdot<<<(M + kDotRows - 1) / kDotRows, 256, 0, s>>>(M, M_dev, s0, e);
+        RPNN_CHECK_LAUNCH();
+        return RPNN_OK;
+    }
+    if (s0.K == 1 && !s1 && !M_dev) {
+        const int64_t b = ((int64_t)M * N + 255) / 256;
+        k_outer<<<(unsigned)std::min<int64_t>(b, 152 * 8), 256, 0, s>>>(M, N, s0, e);
+        RPNN_CHECK_LAUNCH();
+        return RPNN_OK;
+    }
     GemmChoice ch{0, 1, 0.0f, 0.0f};
     const Seg& s1r = s1 ? *s1 : s0;
     const int nseg = s1 ? 2 : 1;

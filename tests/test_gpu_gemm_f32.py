@@ -1,0 +1,48 @@
+"""The FP32 GEMM behind the plain MLPs (and the FP32 network) at tile edges: odd widths and row
+counts, rows on 4-, 8- and 16-byte boundaries, one-column and one-row outputs, inner sizes
+below and above the split threshold, tuned and untuned.  Weights, inputs and gradients are
+positive, so every sum has positive terms and each result's relative error is at most the
+number of its roundings (the inner sizes it passed through, a few per layer more) times
+2^-24, against FP64 torch autograd."""
+import numpy as np
+import pytest
+
+from paper_1709_05418_gb300 import workloads as W
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def reference(widths, params, x, dout):
+    p = params.double().requires_grad_(True)
+    h, prev, off = x.double(), x.shape[1], 0
+    for w in list(widths) + [1]:
+        h = torch.relu(h @ p[off:off + w * prev].reshape(w, prev).t() + p[off + w * prev:off + w * prev + w])
+        off += w * prev + w
+        prev = w
+    (h[:, 0] * dout.double()).sum().backward()
+    return h[:, 0].detach(), p.grad
+
+
+@pytest.mark.parametrize("tuned", [False, True])
+@pytest.mark.parametrize("widths,din", [((200, 200), 226), ((1, 33, 130), 51), ((64, 7), 2400), ((257,), 18)])
+@pytest.mark.parametrize("q", [1, 63, 65, 129, 1100])
+def test_dense_at_tile_edges(widths, din, q, tuned):
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_1709_05418_gb300 import api
+    ctx = api.Context()
+    ctx.set_autotune(tuned)
+    g = torch.Generator().manual_seed(q + din)
+    params = torch.from_numpy(np.abs(W.dense_he_init(widths, din, seed=3, bias=0.1))).cuda()
+    x = (torch.rand((q, din), generator=g) + 0.1).cuda()
+    dout = (torch.rand(q, generator=g) + 0.1).cuda()
+    out, grad = reference(widths, params, x, dout)
+    inner = [din] + list(widths)
+    fwd = (sum(inner) + 4 * len(inner)) * 2.0 ** -24
+    bwd = (2 * sum(inner) + q + 8 * len(inner)) * 2.0 ** -24
+    got = ctx.dense_forward(widths, params, x).double()
+    assert float(((got - out).abs() / out).max()) <= fwd
+    got = ctx.dense_backward(widths, params, x, dout).double()
+    assert float(((got - grad).abs() / grad).max()) <= bwd
+    ctx.close()
