@@ -448,7 +448,8 @@ static rpnn_status render_impl(Ctx* c, int32_t vol, const rpnn_render_desc* desc
     rpnn_render_desc rd0 = *desc;                   // the primary pass carries light 0
     for (int a = 0; a < 3; ++a) rd0.light_dir[a] = lights[a];
     rd0.light_E = lights[3 * nl];
-    const bool queries = net || nl > 1;             // shading points are listed for the network or extra lights
+    const bool path = desc->mode == RPNN_MODE_PATH;
+    const bool queries = net || path || nl > 1;     // shading points are listed for the network, paths or extra lights
     const int64_t P = (int64_t)desc->width * desc->height * desc->spp;
     const bool f32 = desc->precision == RPNN_F32;
     const bool fp8 = desc->precision == RPNN_FP8E4M3;
@@ -460,7 +461,7 @@ static rpnn_status render_impl(Ctx* c, int32_t vol, const rpnn_render_desc* desc
     const int64_t CH = std::min<int64_t>(P, c->chunk_rows > 0 ? c->chunk_rows : kChunkRows);
     const int nchunks = (int)((P + CH - 1) / CH);
     st = c->sample_val.reserve(P * sizeof(float));
-    if (!st) st = c->q_count.reserve((1 + nchunks) * sizeof(int));
+    if (!st) st = c->q_count.reserve((2 + nchunks) * sizeof(int));
     if (!st) st = c->light.reserve(lights.size() * sizeof(float));
     if (queries) {
         if (!st) st = c->q_x.reserve(P * 3 * sizeof(float));
@@ -492,13 +493,18 @@ static rpnn_status render_impl(Ctx* c, int32_t vol, const rpnn_render_desc* desc
     // and environment next-event kernels
     RPNN_CUDA_TRY(cudaMemcpyAsync(c->light.p, lights.data(), lights.size() * sizeof(float), cudaMemcpyHostToDevice, s));
     const float* ldir = c->light.as<float>();
-    RPNN_CUDA_TRY(cudaMemsetAsync(qc, 0, sizeof(int), s));
+    RPNN_CUDA_TRY(cudaMemsetAsync(qc, 0, 2 * sizeof(int), s));
     {
         NvtxRange stage("primary");
         st = launch_primary(*c, vv, rd0, c->sample_val.as<float>(), queries ? c->q_x.as<float>() : nullptr,
                             queries ? c->q_d.as<float>() : nullptr, queries ? c->q_ps.as<uint32_t>() : nullptr,
                             queries ? qc : nullptr, nullptr, nullptr, nullptr, nullptr, s);
         if (st) return st;
+        if (path) {
+            st = launch_paths(*c, vv, rd0, c->q_x.as<float>(), c->q_d.as<float>(), c->q_ps.as<uint32_t>(), qc, qc + 1,
+                              c->sample_val.as<float>(), s);
+            if (st) return st;
+        }
         if (nl > 1) {
             st = launch_nee_env(*c, vv, rd0, c->q_x.as<float>(), c->q_d.as<float>(), c->q_ps.as<uint32_t>(), qc, P,
                                 ldir, ldir + 3 * nl, 1, nl, c->sample_val.as<float>(), s);

@@ -66,7 +66,7 @@ __device__ __forceinline__ void duff_basis(float3 n, float3& b1, float3& b2) {
 
 // Henyey-Greenstein phase function of the cosine between propagation directions.
 __device__ __forceinline__ float hg_eval(float g, float ct) {
-    const float den = 1.0f + g * g - 2.0f * g * ct;
+    const float den = __fmaf_rn(-2.0f * g, ct, __fmaf_rn(g, g, 1.0f));
     return (1.0f - g * g) / (4.0f * kPi * den * sqrtf(den));
 }
 
@@ -142,7 +142,7 @@ __device__ __forceinline__ bool box_clip(const float ext[3], float3 o, float3 d,
 
 // Raw-grid density (trilinear, voxel centres, zero outside) for free-flight sampling.
 __device__ __forceinline__ float raw_density(const VolumeView& v, float3 p) {
-    const float u[3] = {p.x * v.inv_h0 - 0.5f, p.y * v.inv_h0 - 0.5f, p.z * v.inv_h0 - 0.5f};
+    const float u[3] = {__fmaf_rn(p.x, v.inv_h0, -0.5f), __fmaf_rn(p.y, v.inv_h0, -0.5f), __fmaf_rn(p.z, v.inv_h0, -0.5f)};
     int i[3];
     float f[3];
 #pragma unroll
@@ -176,10 +176,10 @@ struct BrickWalk {
 
 __device__ __forceinline__ void walk_axis(float o, float d, float t0, float bs, int nb, int& b, int& s, float& tn,
                                           float& td) {
-    b = (int)floorf((o + t0 * d) / bs);
+    b = (int)floorf(__fmaf_rn(t0, d, o) / bs);
     b = min(max(b, 0), nb - 1);
-    if (d > 0.0f) { s = 1; tn = ((float)(b + 1) * bs - o) / d; td = bs / d; }
-    else if (d < 0.0f) { s = -1; tn = ((float)b * bs - o) / d; td = -bs / d; }
+    if (d > 0.0f) { s = 1; tn = __fmaf_rn((float)(b + 1), bs, -o) / d; td = bs / d; }
+    else if (d < 0.0f) { s = -1; tn = __fmaf_rn((float)b, bs, -o) / d; td = -bs / d; }
     else { s = 0; tn = INFINITY; td = INFINITY; }
 }
 
@@ -247,31 +247,10 @@ __device__ __forceinline__ int delta_track(const VolumeView& v, float3 o, float3
     return -1;
 }
 
-// Delta tracking against the global majorant (one block per tentative collision: x for
-// the exponential step, y for the real/null decision), for the path tracer's bounces,
-// which start inside the medium where the bricks hold nearly the global majorant anyway.
-// The medium behind a first bounce has extinction v.dscale * mu_t (the chopped
-// Lorenz-Mie medium; 1 otherwise): the majorant's rate scales, the real/null ratio not.
-__device__ __forceinline__ int delta_track_global(const VolumeView& v, float3 o, float3 d, const Rng& rng,
-                                                  uint32_t& ctr, float3& x) {
-    float t0, t1;
-    if (v.majorant <= 0.0f || !box_clip(v.ext, o, d, t0, t1)) return 0;
-    const float maj_s = v.majorant * v.dscale;
-    float t = t0;
-    for (uint32_t n = 0; n < v.track_cap; ++n) {
-        const float4 xi = rng.draw(ctr++);
-        t -= logf(1.0f - xi.x) / maj_s;
-        if (t >= t1) return 0;
-        const float3 p = o + t * d;
-        if (xi.y * v.majorant < raw_density(v, p)) { x = p; return 1; }
-    }
-    return -1;
-}
-
 // Ratio-tracking transmittance from o along d to the grid boundary over the same walk:
 // one block (x -> optical depth) per tentative collision, T *= 1 - mu_t / mu_b there.
-// Light travels through the medium of extinction v.dscale * mu_t (see delta_track_global):
-// each brick's rate is v.dscale * mu_b, the ratio unchanged.
+// Light travels through the medium of extinction v.dscale * mu_t (the chopped Lorenz-Mie
+// medium; 1 otherwise): each brick's rate is v.dscale * mu_b, the ratio unchanged.
 __device__ __forceinline__ float ratio_track(const VolumeView& v, float3 o, float3 d, const Rng& rng,
                                              uint32_t& ctr, bool& capped) {
     float t0, t1;
@@ -314,33 +293,6 @@ __device__ __forceinline__ float nee(const VolumeView& v, bool first, float3 x, 
                                      const Rng& rng, uint32_t& ctr, bool& capped) {
     const float T = ratio_track(v, x, wl, rng, ctr, capped);
     return E * phase_eval(v, first ? v.lm : v.lmc, dot3(d, wl)) * T;
-}
-
-// One path estimate of L_i at vertex x reached along tracing direction d: phase
-// sampling, delta tracking to the next collision, survival with probability albedo,
-// NEE there, repeat.  Draw order per bounce: direction block, tracking blocks,
-// survival block, shadow blocks.  x is the path's first bounce (full phase function);
-// everything after it uses the medium behind the first bounce (v.lmc, v.dscale,
-// v.albedo_c), which is the volume's own unless its Lorenz-Mie function is chopped.
-__device__ __forceinline__ float path_Li(const VolumeView& v, float3 x, float3 d, float3 wl, float E,
-                                         const Rng& rng, bool& capped) {
-    uint32_t ctr = 0;
-    float L = 0.0f;
-    for (int b = 0; b < kBounceCap; ++b) {
-        float4 xi = rng.draw(ctr++);
-        const float3 nd = phase_sample(v, b == 0 ? v.lm : v.lmc, d, xi.x, xi.y);
-        float3 nx;
-        const int hit = delta_track_global(v, x, nd, rng, ctr, nx);
-        if (hit < 0) { capped = true; return L; }
-        if (hit == 0) return L;
-        xi = rng.draw(ctr++);
-        if (!(xi.x < v.albedo_c)) return L;
-        L += nee(v, false, nx, nd, wl, E, rng, ctr, capped);
-        x = nx;
-        d = nd;
-    }
-    capped = true;
-    return L;
 }
 
 __device__ __forceinline__ void raise_status(uint32_t* status, uint32_t bits) {

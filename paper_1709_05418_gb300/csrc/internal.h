@@ -292,6 +292,10 @@ rpnn_status launch_scatter_composite(Ctx& c, const rpnn_render_desc& rd, float a
                                      float* sample_val, float* image, bool with_g,
                                      cudaStream_t s, const int* g_off = nullptr,
                                      const int* g_total = nullptr);
+// Path mode: adds the path-traced L_i of the *qcount shading points to their samples (which hold
+// L_d) and multiplies by the albedo; *next: the work counter, zero before the launch.
+rpnn_status launch_paths(Ctx& c, const VolumeView& vv, const rpnn_render_desc& rd, const float* qx, const float* qd,
+                         const uint32_t* qps, const int* qcount, int* next, float* sample_val, cudaStream_t s);
 // Environment lighting: next-event estimates towards lights j0..n-1 (device dirs [n][3],
 // irradiances E [n]) of the *qcount (<= max_q) shading points, added to their samples.
 rpnn_status launch_nee_env(Ctx& c, const VolumeView& vv, const rpnn_render_desc& rd, const float* qx,

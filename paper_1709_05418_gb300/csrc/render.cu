@@ -3,13 +3,14 @@
 //
 // k_primary: one thread per pixel sample.  Pinhole ray with Philox pixel jitter, delta
 // tracking to the first real collision (the visible point), next-event estimation of
-// the direct in-scattering with a ratio-tracked shadow ray, and either (RPNN mode) an
-// appended shading query for the descriptor + network stages, or (path mode) a
-// path-traced estimate of the indirect part.  Queries are compacted with one atomic per
+// the direct in-scattering with a ratio-tracked shadow ray, and an appended shading query
+// for the descriptor + network stages (RPNN mode) or for k_paths, which adds a path-traced
+// estimate of the indirect part (path mode).  Queries are compacted with one atomic per
 // warp so the list stays in pixel order within a warp.
 #include <vector>
 
 #include "common.cuh"
+#include "paths.cuh"
 
 namespace rpnn {
 
@@ -94,10 +95,8 @@ k_primary(const VolumeView v_, const RenderArgs a_, int64_t P_, float* __restric
             const float3 wl = f3(a.wl[0], a.wl[1], a.wl[2]);
             uint32_t c2 = 0;
             Ld = nee(v, true, x, d, wl, a.E, make_rng(a.seed, pixel, s, kDomShadow), c2, capped);
-            float Li = 0.0f;
-            if (a.mode == RPNN_MODE_PATH)
-                Li = path_Li(v, x, d, wl, a.E, make_rng(a.seed, pixel, s, kDomPath), capped);
-            val = v.albedo * (Ld + Li);
+            // path mode: k_paths adds L_i and multiplies by the albedo
+            val = a.mode == RPNN_MODE_PATH ? Ld : v.albedo * Ld;
         }
         if (capped) raise_status(status, kStatIterLimit);
         if (sample_val) sample_val[ps] = val;
@@ -237,96 +236,223 @@ __device__ __forceinline__ float warp_scan(float v, int lane) {
     return v;
 }
 
-// Training records (Sec. 5.1); one warp per record.  Lane 0 samples the record (direction,
-// origin on the bounding sphere's cross-section, free flight by delta tracking with
-// retries, light direction) and the warp traces its label paths 32 at a time, path j on
-// lane j % 32 with path j's own random stream.  After each round the stopping rule is
-// evaluated at every path count of the round in order -- n >= n_min and
-// 1.96 s / sqrt(n) <= rel_ci * mean -- from FP32 prefix sums of L and L^2 over the round
-// added to Kahan-compensated running totals; the first count that meets it (or n_max)
-// ends the record and its label is the mean of its first n paths.
-__global__ void __launch_bounds__(128)
+// Indirect part of a path-traced render (Sec. 4.4's reference): the shading points are dealt to
+// the lanes of a resident grid as they finish their paths; sample value = albedo (L_d + L_i),
+// L_d left there by k_primary.  `lanes`: lanes of a warp that take paths -- fewer than 32 when
+// the grid has more lanes than there are paths, where latency sets the time and fewer lanes
+// wait for one another.
+struct RenderPaths {
+    const VolumeView& v;
+    const RenderArgs& a;
+    const float *qx, *qd;
+    const uint32_t* qps;
+    const int* qcount;
+    int* next;
+    float* sample_val;
+    uint32_t* status;
+    int total, lanes;
+    uint32_t ps;
+    __device__ __forceinline__ int fetch(bool want, float3& x, float3& d, Rng& rng) {
+        const int lane = threadIdx.x & 31;
+        const bool take = want && lane < lanes;
+        const unsigned m = __ballot_sync(0xffffffffu, take);
+        int base = 0;
+        if (m && lane == __ffs(m) - 1) base = atomicAdd(next, __popc(m));
+        base = __shfl_sync(0xffffffffu, base, m ? __ffs(m) - 1 : 0);
+        const int i = base + __popc(m & ((1u << lane) - 1u));
+        if (!take || i >= total) return -1;
+        ps = qps[i];
+        x = f3(qx[3 * i], qx[3 * i + 1], qx[3 * i + 2]);
+        d = f3(qd[3 * i], qd[3 * i + 1], qd[3 * i + 2]);
+        rng = make_rng(a.seed, ps / (uint32_t)a.spp, ps % (uint32_t)a.spp, kDomPath);
+        return 1;
+    }
+    __device__ __forceinline__ void finish(float L, bool capped) {
+        sample_val[ps] = v.albedo * (sample_val[ps] + L);
+        if (capped) raise_status(status, kStatIterLimit);
+    }
+    __device__ __forceinline__ bool stopped() const { return false; }
+    __device__ __forceinline__ bool keep() const { return false; }
+    __device__ __forceinline__ void gave_up() { raise_status(status, kStatTimeout); }
+};
+
+constexpr int kPathBlocks = 5;       // blocks of 128 threads per SM
+__global__ void __launch_bounds__(128, kPathBlocks)
+k_paths(const VolumeView v, const RenderArgs a, const float* __restrict__ qx, const float* __restrict__ qd,
+        const uint32_t* __restrict__ qps, const int* __restrict__ qcount, int* next, float* sample_val,
+        uint32_t* status) {
+    const int total = *qcount, warps = (int)(gridDim.x * (blockDim.x >> 5));
+    const int lanes = min(32, max(1, (total + warps - 1) / warps));
+    RenderPaths src{v, a, qx, qd, qps, qcount, next, sample_val, status, total, lanes, 0};
+    trace_paths(v, f3(a.wl[0], a.wl[1], a.wl[2]), a.E, src);
+}
+
+// Training records (Sec. 5.1).  k_record_start, one thread per record, samples it: direction,
+// origin on the bounding sphere's cross-section, free flight by delta tracking with retries,
+// light direction (npaths = -1: no collision found in kRecordAttempts tries).
+__global__ void __launch_bounds__(32)
+k_record_start(const VolumeView v, int64_t first, int64_t n, uint64_t seed, float* __restrict__ xo,
+               float* __restrict__ dout, float* __restrict__ wlo, float* __restrict__ label,
+               int* __restrict__ npaths, uint32_t* status) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const uint32_t rec = (uint32_t)(first + i);
+    float3 x = f3(0.f, 0.f, 0.f), d = f3(0.f, 0.f, 1.f);
+    int found = 0;
+    const float ext[3] = {v.ext[0], v.ext[1], v.ext[2]};
+    const float3 C = f3(0.5f * ext[0], 0.5f * ext[1], 0.5f * ext[2]);
+    const float R = 0.5f * sqrtf(ext[0] * ext[0] + ext[1] * ext[1] + ext[2] * ext[2]);
+    for (uint32_t att = 0; att < (uint32_t)kRecordAttempts && !found; ++att) {
+        const float4 xi = make_rng(seed, rec, att, kDomRecord).draw(0);
+        const float cz = 1.0f - 2.0f * xi.x;
+        float sp, cp;
+        sincosf(2.0f * kPi * xi.y, &sp, &cp);
+        const float sz = sqrtf(fmaxf(0.0f, 1.0f - cz * cz));
+        d = f3(sz * cp, sz * sp, cz);
+        float3 b1, b2;
+        duff_basis(d, b1, b2);
+        const float rr = R * sqrtf(xi.z);
+        float s2, c2;
+        sincosf(2.0f * kPi * xi.w, &s2, &c2);
+        const float3 o = C + (rr * c2) * b1 + (rr * s2) * b2 + (-2.0f * R) * d;
+        uint32_t ctr = 0;
+        const int h = delta_track(v, o, d, make_rng(seed, rec, att, kDomRecTrack), ctr, x);
+        if (h < 0) raise_status(status, kStatIterLimit);
+        found = h == 1;
+    }
+    const float4 xi = make_rng(seed, rec, 0, kDomLight).draw(0);
+    const float cz = 1.0f - 2.0f * xi.x;
+    float sp, cp;
+    sincosf(2.0f * kPi * xi.y, &sp, &cp);
+    const float sz = sqrtf(fmaxf(0.0f, 1.0f - cz * cz));
+    if (!found) raise_status(status, kStatIterLimit);
+    xo[3 * i] = x.x; xo[3 * i + 1] = x.y; xo[3 * i + 2] = x.z;
+    dout[3 * i] = d.x; dout[3 * i + 1] = d.y; dout[3 * i + 2] = d.z;
+    wlo[3 * i] = sz * cp; wlo[3 * i + 1] = sz * sp; wlo[3 * i + 2] = cz;
+    label[i] = 0.0f;
+    npaths[i] = found ? 0 : -1;
+}
+
+// The label paths of one record, shared by the warps of its block.  Path j has its own random
+// stream and its estimate goes to slot j % kRing of a ring in shared memory; lanes take path
+// indices in order as they finish, at most kRing ahead of the first round of 32 paths that is
+// not complete.  Warp 0 evaluates the complete rounds in order: the stopping rule at every path
+// count -- n >= n_min and 1.96 s / sqrt(n) <= rel_ci * mean -- from FP32 prefix sums of L and
+// L^2 over the round added to Kahan-compensated running totals; the first count that meets it
+// (or n_max) ends the record and its label is the mean of its first n paths.
+// A slot holds the estimate's bits or kEmpty (a NaN no estimate has); cap: a loop of the path
+// reached its cap.
+constexpr int kRing = 512;
+constexpr uint32_t kEmpty = 0xffffffffu;
+struct RecordRing {
+    uint32_t slot[kRing];
+    unsigned char cap[kRing];
+    int next, base, done;
+};
+struct LabelPaths {
+    RecordRing& r;
+    float3 x0, d0;
+    uint64_t seed;
+    uint32_t rec;
+    float rel_ci;
+    int n_min, n_max;
+    uint32_t* status;
+    int j;                       // this lane's path, -1: none
+    KahanF S, Q;                 // warp 0: running sums of L and L^2
+    float mean;
+    int np;
+    __device__ __forceinline__ void rounds() {
+        const int lane = threadIdx.x & 31;
+        volatile RecordRing& vr = r;
+        for (;;) {
+            const int base = vr.base, jj = base + lane;
+            const uint32_t bits = jj < n_max ? vr.slot[jj % kRing] : 0u;
+            if (__any_sync(0xffffffffu, bits == kEmpty)) return;
+            __threadfence_block();
+            if (jj < n_max && vr.cap[jj % kRing]) {
+                raise_status(status, kStatIterLimit);
+                vr.cap[jj % kRing] = 0;
+            }
+            const float L = __uint_as_float(bits);
+            const float pS = warp_scan(L, lane), pQ = warp_scan(L * L, lane);
+            const float cnt = (float)(jj + 1);
+            const float s_j = S.with(pS), q_j = Q.with(pQ);
+            const float m_j = s_j / cnt;
+            const float var = fmaxf(q_j - s_j * m_j, 0.0f) / fmaxf(cnt - 1.0f, 1.0f);
+            const float hw = 1.96f * sqrtf(var / cnt);
+            const bool stop = jj < n_max &&
+                              ((jj + 1 >= n_min && jj > 0 && m_j > 0.0f && hw <= rel_ci * m_j) || jj + 1 == n_max);
+            const uint32_t hit = __ballot_sync(0xffffffffu, stop);
+            if (hit) {
+                const int f = __ffs(hit) - 1;
+                mean = __shfl_sync(0xffffffffu, m_j, f);
+                np = base + f + 1;
+                vr.done = 1;
+                return;
+            }
+            S.add(__shfl_sync(0xffffffffu, pS, 31));
+            Q.add(__shfl_sync(0xffffffffu, pQ, 31));
+            vr.slot[jj % kRing] = kEmpty;
+            __threadfence_block();                 // slots are free before base says so
+            __syncwarp();
+            if (lane == 0) vr.base = base + 32;
+            __syncwarp();
+        }
+    }
+    __device__ __forceinline__ int fetch(bool want, float3& x, float3& d, Rng& rng) {
+        const int lane = threadIdx.x & 31;
+        volatile RecordRing& vr = r;
+        if (threadIdx.x < 32 && !vr.done) rounds();
+        const bool claim = want && j < 0;
+        const unsigned m = __ballot_sync(0xffffffffu, claim);
+        int first = 0;
+        if (m && lane == __ffs(m) - 1) first = atomicAdd(&r.next, __popc(m));
+        first = __shfl_sync(0xffffffffu, first, m ? __ffs(m) - 1 : 0);
+        if (claim) j = first + __popc(m & ((1u << lane) - 1u));
+        if (!want || j >= n_max) return -1;
+        const int base = vr.base;
+        __threadfence_block();
+        if (j >= base + kRing) return 0;
+        x = x0; d = d0;
+        rng = make_rng(seed, rec, (uint32_t)j, kDomLabel);
+        return 1;
+    }
+    __device__ __forceinline__ void finish(float L, bool capped) {
+        volatile RecordRing& vr = r;
+        if (capped) vr.cap[j % kRing] = 1;
+        __threadfence_block();                     // the flag is there before the estimate
+        vr.slot[j % kRing] = __float_as_uint(L);
+        j = -1;
+    }
+    __device__ __forceinline__ bool stopped() const {
+        volatile RecordRing& vr = r;
+        return __any_sync(0xffffffffu, vr.done != 0);
+    }
+    __device__ __forceinline__ bool keep() const { return threadIdx.x < 32; }
+    __device__ __forceinline__ void gave_up() { raise_status(status, kStatTimeout); }
+};
+
+__global__ void __launch_bounds__(128, 5)
 k_records(const VolumeView v, int64_t first, int64_t n, uint64_t seed, float rel_ci, int n_min,
-          int n_max, float* __restrict__ xo, float* __restrict__ dout, float* __restrict__ wlo,
+          int n_max, const float* __restrict__ xo, const float* __restrict__ dout, const float* __restrict__ wlo,
           float* __restrict__ label, int* __restrict__ npaths, uint32_t* status) {
-    const int lane = threadIdx.x & 31;
-    const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t i = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); i < n; i += nwarps) {
-        const uint32_t rec = (uint32_t)(first + i);
-        float3 x = f3(0.f, 0.f, 0.f), d = f3(0.f, 0.f, 1.f);
-        int found = 0;
-        if (lane == 0) {
-            const float ext[3] = {v.ext[0], v.ext[1], v.ext[2]};
-            const float3 C = f3(0.5f * ext[0], 0.5f * ext[1], 0.5f * ext[2]);
-            const float R = 0.5f * sqrtf(ext[0] * ext[0] + ext[1] * ext[1] + ext[2] * ext[2]);
-            for (uint32_t att = 0; att < (uint32_t)kRecordAttempts && !found; ++att) {
-                const float4 xi = make_rng(seed, rec, att, kDomRecord).draw(0);
-                const float cz = 1.0f - 2.0f * xi.x;
-                float sp, cp;
-                sincosf(2.0f * kPi * xi.y, &sp, &cp);
-                const float sz = sqrtf(fmaxf(0.0f, 1.0f - cz * cz));
-                d = f3(sz * cp, sz * sp, cz);
-                float3 b1, b2;
-                duff_basis(d, b1, b2);
-                const float rr = R * sqrtf(xi.z);
-                float s2, c2;
-                sincosf(2.0f * kPi * xi.w, &s2, &c2);
-                const float3 o = C + (rr * c2) * b1 + (rr * s2) * b2 + (-2.0f * R) * d;
-                uint32_t ctr = 0;
-                const int h = delta_track(v, o, d, make_rng(seed, rec, att, kDomRecTrack), ctr, x);
-                if (h < 0) raise_status(status, kStatIterLimit);
-                found = h == 1;
-            }
+    __shared__ RecordRing ring;
+    for (int64_t i = blockIdx.x; i < n; i += gridDim.x) {
+        if (npaths[i] < 0) {                       // no collision: label 0, no paths
+            __syncthreads();
+            if (threadIdx.x == 0) npaths[i] = 0;
+            continue;
         }
-        found = __shfl_sync(0xffffffffu, found, 0);
-        x = f3(__shfl_sync(0xffffffffu, x.x, 0), __shfl_sync(0xffffffffu, x.y, 0), __shfl_sync(0xffffffffu, x.z, 0));
-        d = f3(__shfl_sync(0xffffffffu, d.x, 0), __shfl_sync(0xffffffffu, d.y, 0), __shfl_sync(0xffffffffu, d.z, 0));
-        float3 wl;
-        {
-            const float4 xi = make_rng(seed, rec, 0, kDomLight).draw(0);
-            const float cz = 1.0f - 2.0f * xi.x;
-            float sp, cp;
-            sincosf(2.0f * kPi * xi.y, &sp, &cp);
-            const float sz = sqrtf(fmaxf(0.0f, 1.0f - cz * cz));
-            wl = f3(sz * cp, sz * sp, cz);
-        }
-        float mean = 0.0f;
-        int np = 0;
-        bool capped = false;
-        if (found) {
-            KahanF S, Q;                               // running sums of L and L^2
-            for (int base = 0; base < n_max; base += 32) {
-                const int j = base + lane;
-                float L = 0.0f;
-                if (j < n_max) L = path_Li(v, x, d, wl, 1.0f, make_rng(seed, rec, (uint32_t)j, kDomLabel), capped);
-                const float pS = warp_scan(L, lane), pQ = warp_scan(L * L, lane);
-                const float cnt = (float)(j + 1);
-                const float s_j = S.with(pS), q_j = Q.with(pQ);
-                const float m_j = s_j / cnt;
-                const float var = fmaxf(q_j - s_j * m_j, 0.0f) / fmaxf(cnt - 1.0f, 1.0f);
-                const float hw = 1.96f * sqrtf(var / cnt);
-                const bool stop = j < n_max && ((j + 1 >= n_min && j > 0 && m_j > 0.0f && hw <= rel_ci * m_j) ||
-                                                j + 1 == n_max);
-                const uint32_t hit = __ballot_sync(0xffffffffu, stop);
-                if (hit) {
-                    const int f = __ffs(hit) - 1;
-                    mean = __shfl_sync(0xffffffffu, m_j, f);
-                    np = base + f + 1;
-                    break;
-                }
-                S.add(__shfl_sync(0xffffffffu, pS, 31));
-                Q.add(__shfl_sync(0xffffffffu, pQ, 31));
-            }
-        } else if (lane == 0) {
-            raise_status(status, kStatIterLimit);
-        }
-        if (__any_sync(0xffffffffu, capped) && lane == 0) raise_status(status, kStatIterLimit);
-        if (lane == 0) {
-            xo[3 * i] = x.x; xo[3 * i + 1] = x.y; xo[3 * i + 2] = x.z;
-            dout[3 * i] = d.x; dout[3 * i + 1] = d.y; dout[3 * i + 2] = d.z;
-            wlo[3 * i] = wl.x; wlo[3 * i + 1] = wl.y; wlo[3 * i + 2] = wl.z;
-            label[i] = mean;
-            npaths[i] = np;
+        for (int k = threadIdx.x; k < kRing; k += blockDim.x) { ring.slot[k] = kEmpty; ring.cap[k] = 0; }
+        if (threadIdx.x == 0) { ring.next = 0; ring.base = 0; ring.done = 0; }
+        __syncthreads();
+        LabelPaths src{ring, f3(xo[3 * i], xo[3 * i + 1], xo[3 * i + 2]), f3(dout[3 * i], dout[3 * i + 1], dout[3 * i + 2]),
+                       seed, (uint32_t)(first + i), rel_ci, n_min, n_max, status, -1, KahanF(), KahanF(), 0.0f, 0};
+        trace_paths(v, f3(wlo[3 * i], wlo[3 * i + 1], wlo[3 * i + 2]), 1.0f, src);
+        __syncthreads();                           // every warp has left the ring
+        if (threadIdx.x == 0) {
+            label[i] = src.mean;
+            npaths[i] = src.np;
         }
     }
 }
@@ -430,6 +556,14 @@ rpnn_status launch_scatter_composite(Ctx& c, const rpnn_render_desc& rd, float a
     return RPNN_OK;
 }
 
+rpnn_status launch_paths(Ctx& c, const VolumeView& vv, const rpnn_render_desc& rd, const float* qx, const float* qd,
+                         const uint32_t* qps, const int* qcount, int* next, float* sample_val, cudaStream_t s) {
+    k_paths<<<(unsigned)(c.num_sms * kPathBlocks), 128, 0, s>>>(vv, make_args(rd), qx, qd, qps, qcount, next, sample_val,
+                                                                c.status.as<uint32_t>());
+    RPNN_CHECK_LAUNCH();
+    return RPNN_OK;
+}
+
 rpnn_status launch_nee_env(Ctx& c, const VolumeView& vv, const rpnn_render_desc& rd, const float* qx,
                            const float* qd, const uint32_t* qps, const int* qcount, int64_t max_q, const float* dirs,
                            const float* E, int j0, int n, float* sample_val, cudaStream_t s) {
@@ -490,10 +624,15 @@ rpnn_status launch_chunk_counts(Ctx& c, const int* count, int64_t rows, int n, i
 rpnn_status launch_records(Ctx& c, const VolumeView& vv, int64_t first, int64_t n, uint64_t seed,
                            float rel_ci, int n_min, int n_max, float* x, float* d, float* wl,
                            float* label, int* npaths, cudaStream_t s) {
-    // one warp per record, four per block; at most a few waves of blocks (grid-stride)
-    const int64_t blocks = std::min<int64_t>((n + 3) / 4, (int64_t)c.num_sms * 16);
-    k_records<<<(unsigned)blocks, 128, 0, s>>>(vv, first, n, seed, rel_ci, n_min, n_max, x, d, wl,
-                                               label, npaths, c.status.as<uint32_t>());
+    k_record_start<<<(unsigned)((n + 31) / 32), 32, 0, s>>>(vv, first, n, seed, x, d, wl, label, npaths,
+                                                            c.status.as<uint32_t>());
+    RPNN_CHECK_LAUNCH();
+    // a block per record (grid-stride beyond the grid limit); few records get more warps each
+    // so that the chip is full
+    const int64_t want = (int64_t)c.num_sms * 20;          // resident warps
+    const int warps = n * 1 >= want ? 1 : (n * 2 >= want ? 2 : 4);
+    k_records<<<(unsigned)std::min<int64_t>(n, 1 << 30), 32 * warps, 0, s>>>(
+        vv, first, n, seed, rel_ci, n_min, n_max, x, d, wl, label, npaths, c.status.as<uint32_t>());
     RPNN_CHECK_LAUNCH();
     return RPNN_OK;
 }
