@@ -7,9 +7,10 @@
 // 32 lanes per instruction: every loop ends with its longest lane.  Here each lane is a state
 // machine and the warp runs one step of all lanes at a time: a step is one tentative
 // collision, of a free flight (global majorant) or of a shadow ray (brick majorants), whose
-// random block, logarithm and density lookup both kinds share.  What happens once per bounce
-// (a new direction, survival and the shadow ray's set-up, the next path for a lane that ended
-// one) waits until several lanes need it (kEventLanes) or as many lanes wait as run.
+// random block, logarithm and density lookup both kinds share; a shadow ray crosses at most
+// kWalkSteps bricks a step.  What happens once per bounce (the end of a shadow ray, survival
+// and the next shadow ray's set-up, a new direction, the next path for a lane that ended one)
+// waits, each of the two kinds by itself, until kEventLanes lanes need it or as many as run.
 // The arithmetic whose contraction the compiler would otherwise choose by the code around it
 // (positions, the optical depth spent, the phase cosine) is written out with one rounding
 // sequence.  Every path does the arithmetic and the draws of its own stream in the order direction block,
@@ -22,7 +23,8 @@
 
 namespace rpnn {
 
-constexpr int kEventLanes = 8;
+constexpr int kEventLanes = 11;               // 5 to 18 lanes, 3 to 6 bricks: within 5 % of one another
+constexpr int kWalkSteps = 4;
 constexpr uint32_t kPathPolls = 1u << 24;     // bound on a warp's polls for other warps' results
 
 // Source of paths and sink of estimates for trace_paths:
@@ -33,10 +35,11 @@ constexpr uint32_t kPathPolls = 1u << 24;     // bound on a warp's polls for oth
 //   void gave_up()                   the bound on polls was reached
 template <class Src>
 __device__ __forceinline__ void trace_paths(const VolumeView& v, const float3 wl, const float E, Src& src) {
-    enum { kFetch, kTurn, kHit, kFly, kShadow, kWait, kDone };
+    enum { kHit, kFetch, kEnd, kExit, kTurn, kFly, kShadow, kWait, kDone };
     int state = kFetch, b = 0;
     float3 x = f3(0.f, 0.f, 0.f), d = f3(0.f, 0.f, 1.f);
     float t = 0.0f, t1 = 0.0f, L = 0.0f, T = 1.0f, te = 0.0f, mu_b = 0.0f;
+    float tau = -1.0f;                  // shadow ray: optical depth left to spend, < 0: draw first
     uint32_t ctr = 0, n = 0, polls = 0;
     Rng rng = make_rng(0, 0, 0, 0);
     BrickWalk w{};
@@ -44,16 +47,8 @@ __device__ __forceinline__ void trace_paths(const VolumeView& v, const float3 wl
     const float maj_s = v.majorant * v.dscale;
     // the point at t along e from x
     auto at = [&](const float3 e) { return f3(__fmaf_rn(t, e.x, x.x), __fmaf_rn(t, e.y, x.y), __fmaf_rn(t, e.z, x.z)); };
-    auto end = [&]() { src.finish(L, capped); state = kFetch; };
-    // next-event estimate of the vertex x from the shadow ray's transmittance; next bounce
-    auto nee_done = [&]() {
-        const float ct = __fmaf_rn(d.z, wl.z, __fmaf_rn(d.x, wl.x, __fmul_rn(d.y, wl.y)));
-        L = __fmaf_rn(__fmul_rn(E, phase_eval(v, v.lmc, ct)), T, L);
-        ++b;
-        state = kTurn;
-    };
-    // the shadow ray's brick at t; false once it has left the grid or reached its cap
     auto brick = [&]() { te = walk_exit(w, t1); mu_b = walk_majorant(v, w); };
+    // the shadow ray into its next brick; false once it has left the grid or reached its cap
     auto advance = [&]() {
         if (te >= t1) return false;
         t = te;
@@ -64,19 +59,21 @@ __device__ __forceinline__ void trace_paths(const VolumeView& v, const float3 wl
     };
     for (;;) {
         const int run = __popc(__ballot_sync(0xffffffffu, state == kFly || state == kShadow));
-        const int ev = __popc(__ballot_sync(0xffffffffu, state <= kHit));
-        if (run == 0 && ev == 0 && !__any_sync(0xffffffffu, state == kWait) && !src.keep()) break;
+        const int hits = __popc(__ballot_sync(0xffffffffu, state == kHit));
+        const int turns = __popc(__ballot_sync(0xffffffffu, state > kHit && state <= kTurn));
+        if (run + hits + turns == 0 && !__any_sync(0xffffffffu, state == kWait) && !src.keep()) break;
         if (src.stopped()) break;
-        if (run == 0 || ev >= kEventLanes || ev >= run) {
+        const bool do_hits = hits >= min(kEventLanes, run), do_turns = turns >= min(kEventLanes, run);
+        if (do_hits && hits) {
             if (state == kHit) {
                 const float4 xi = rng.draw(ctr++);
                 float t0;
                 if (!(xi.x < v.albedo_c)) {
-                    end();
+                    state = kEnd;
                 } else {
                     T = 1.0f;
                     if (v.majorant <= 0.0f || !box_clip(v.ext, x, wl, t0, t1)) {
-                        nee_done();
+                        state = kExit;
                     } else {
                         walk_init(v, x, wl, t0, w);
                         t = t0;
@@ -84,10 +81,24 @@ __device__ __forceinline__ void trace_paths(const VolumeView& v, const float3 wl
                         brick();
                         bool in = true;
                         while (in && !(mu_b > 0.0f)) in = advance();    // empty bricks spend nothing
-                        if (in) state = kShadow;
-                        else nee_done();
+                        state = in ? kShadow : kExit;
+                        tau = -1.0f;
                     }
                 }
+            }
+            continue;
+        }
+        if (do_turns && (turns || run == 0)) {
+            if (state == kExit) {
+                // next-event estimate of the vertex x from the shadow ray's transmittance; next bounce
+                const float ct = __fmaf_rn(d.z, wl.z, __fmaf_rn(d.x, wl.x, __fmul_rn(d.y, wl.y)));
+                L = __fmaf_rn(__fmul_rn(E, phase_eval(v, v.lmc, ct)), T, L);
+                ++b;
+                state = kTurn;
+            }
+            if (state == kEnd) {
+                src.finish(L, capped);
+                state = kFetch;
             }
             const int got = src.fetch(state == kFetch || state == kWait, x, d, rng);
             if (state == kFetch || state == kWait) {
@@ -97,61 +108,62 @@ __device__ __forceinline__ void trace_paths(const VolumeView& v, const float3 wl
             if (state == kTurn) {
                 if (b >= kBounceCap) {
                     capped = true;
-                    end();
+                    state = kEnd;
                 } else {
                     const float4 xi = rng.draw(ctr++);
                     d = phase_sample(v, b == 0 ? v.lm : v.lmc, d, xi.x, xi.y);
                     float t0;
-                    if (v.majorant <= 0.0f || !box_clip(v.ext, x, d, t0, t1)) end();
-                    else { t = t0; n = 0; state = kFly; }
+                    const bool in = v.majorant > 0.0f && box_clip(v.ext, x, d, t0, t1);
+                    state = in ? kFly : kEnd;
+                    if (in) { t = t0; n = 0; }
                 }
             }
-            if (run == 0 && !__any_sync(0xffffffffu, state < kWait)) {
+            if (run == 0 && turns == 0 && !__any_sync(0xffffffffu, state < kWait)) {
                 // only waiting for other warps of the block
                 if (++polls >= kPathPolls) { src.gave_up(); break; }
                 __nanosleep(200);
             }
             continue;
         }
-        const bool fly = state == kFly, shadow = state == kShadow;
+        const bool fly = state == kFly;
         bool look = false;
-        float3 p = x;
         float xy = 0.0f;
-        if (fly || shadow) {
+        if (fly || (state == kShadow && tau < 0.0f)) {
             const float4 xi = rng.draw(ctr++);
             const float lg = logf(1.0f - xi.x);
             xy = xi.y;
+            tau = -lg;
             if (fly) {
                 t -= lg / maj_s;
-                if (t >= t1) end();
-                else { p = at(d); look = true; }
-            } else {
-                float tau = -lg;
-                bool in = true;
-                while (in) {
-                    if (mu_b > 0.0f) {
-                        const float mu_s = mu_b * v.dscale;
-                        const float seg = __fmul_rn(mu_s, __fsub_rn(te, t));
-                        if (tau < seg) {
-                            t += tau / mu_s;
-                            break;
-                        }
-                        tau = __fsub_rn(tau, seg);
+                look = t < t1;
+                if (!look) state = kEnd;
+            }
+        }
+        if (state == kShadow) {
+            for (int k = 0; k < kWalkSteps; ++k) {
+                if (mu_b > 0.0f) {
+                    const float mu_s = mu_b * v.dscale;
+                    const float seg = __fmul_rn(mu_s, __fsub_rn(te, t));
+                    if (tau < seg) {
+                        t += tau / mu_s;
+                        look = true;
+                        break;
                     }
-                    in = advance();
+                    tau = __fsub_rn(tau, seg);
                 }
-                if (in) { p = at(wl); look = true; }
-                else nee_done();
+                if (!advance()) { state = kExit; break; }
             }
         }
         if (look) {
+            const float3 p = at(fly ? d : wl);
             const float mu = raw_density(v, p);
             if (fly) {
                 if (xy * v.majorant < mu) { x = p; state = kHit; }
-                else if (++n >= v.track_cap) { capped = true; end(); }
+                else if (++n >= v.track_cap) { capped = true; state = kEnd; }
             } else {
                 T *= 1.0f - mu / mu_b;
-                if (++n >= v.track_cap) { capped = true; nee_done(); }
+                tau = -1.0f;
+                if (++n >= v.track_cap) { capped = true; state = kExit; }
             }
         }
     }
