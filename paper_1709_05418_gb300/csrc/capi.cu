@@ -213,7 +213,6 @@ rpnn_status rpnn_build_mips(rpnn_ctx* ctx, int32_t vol, void* stream) {
     cudaStream_t s = (cudaStream_t)stream;
     ++c->epoch;
     rpnn_status st = volume_stats(*c, *v, s);
-    if (!st) st = volume_brick_majorants(*c, *v, s);
     if (st) return st;
     return volume_pack_levels(*c, *v, s);
 }

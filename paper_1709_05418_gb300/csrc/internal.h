@@ -263,8 +263,8 @@ rpnn_status launch_primary_batch(Ctx& c, const void* tables, int n, int64_t bloc
 rpnn_status launch_scatter_composite_batch(Ctx& c, const void* tables, int n, int64_t pixels, const float* g,
                                            const uint32_t* qps, const int* off, float* sample_val, cudaStream_t s);
 void train_graph_release(Ctx& c);     // frees the captured training step and its buffers
+// statistics and tracking majorants (synchronises s to read the statistics back)
 rpnn_status volume_stats(Ctx& c, Volume& v, cudaStream_t s);
-rpnn_status volume_brick_majorants(Ctx& c, Volume& v, cudaStream_t s);
 rpnn_status volume_build_level(Ctx& c, Volume& v, int level, float* dst, cudaStream_t s);
 // levels[0..n-1] into dst[0..n-1] (each [az][ay][ax] FP32), their y and z passes in shared launches
 rpnn_status volume_build_levels(Ctx& c, Volume& v, const int* levels, int n, float* const* dst, cudaStream_t s);

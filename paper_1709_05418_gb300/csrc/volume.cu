@@ -6,6 +6,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <mutex>
 #include <vector>
 
 #include "common.cuh"
@@ -27,33 +28,72 @@ __global__ void k_f16_to_f32(const __half* __restrict__ in, float* __restrict__ 
         out[i] = __half2float(in[i]);
 }
 
-// The grid is read as 16-byte vectors (the allocation is 256-byte aligned), the last n % 4
-// voxels one by one; max, count and the fixed-point sum below are exact in any order.
 __device__ __forceinline__ void stats_max_one(float x, unsigned int& mx, unsigned int& bad, unsigned int& cnt) {
     if (!(x >= 0.0f) || isinf(x)) { bad = 1; return; }
     mx = max(mx, __float_as_uint(x));
     cnt += x > 0.0f;
 }
-__global__ void k_stats_max(const float* __restrict__ v, int64_t n, DevStats* st) {
-    unsigned int mx = 0, bad = 0, c32 = 0;
-    const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, nt = (int64_t)gridDim.x * blockDim.x;
-    const float4* v4 = reinterpret_cast<const float4*>(v);
-    for (int64_t i = tid; i < n / 4; i += nt) {
-        const float4 q = __ldg(v4 + i);
-        stats_max_one(q.x, mx, bad, c32); stats_max_one(q.y, mx, bad, c32);
-        stats_max_one(q.z, mx, bad, c32); stats_max_one(q.w, mx, bad, c32);
+// Statistics (majorant, voxels > 0, negative / NaN / Inf) and the tracking majorants in one
+// pass.  Brick b (kBrick^3 voxels) bounds the trilinear density over its region by the largest
+// of the voxels it interpolates, 8b - 1 .. 8b + 8 per axis (zero outside the grid); max and
+// count are exact in any order.  A block takes one row of bricks: thread x reads voxel x of the
+// row's 10 x 10 lines (coalesced, a plane's ten loads in flight together), keeps the
+// largest and, for the 8 x 8 lines of its own bricks, the statistics; then each brick takes
+// the largest of its ten columns.  256^3: 30 us (a thread per brick reading scattered
+// lines 55 us, and 34 us for a statistics pass of its own).
+constexpr int kBrickThreads = 256;
+__global__ void __launch_bounds__(kBrickThreads)
+k_stats_bricks(const float* __restrict__ raw, int nx, int ny, int nz, int bx, int by, float* __restrict__ out,
+               DevStats* st) {
+    __shared__ float col[kBrickThreads + 2 * kBrick];
+    const int yb = blockIdx.x % by, zb = blockIdx.x / by;
+    const int y0 = yb * kBrick - 1, z0 = zb * kBrick - 1;
+    unsigned int mx = 0, bad = 0, cnt = 0;
+    // columns in chunks of kBrickThreads - 2 voxels, whole bricks each, with a voxel of overlap
+    constexpr int kChunk = (kBrickThreads - 2) / kBrick * kBrick;
+    for (int c0 = 0; c0 < nx; c0 += kChunk) {
+        const int x = c0 - 1 + (int)threadIdx.x;
+        const bool inx = x >= 0 && x < nx;
+        const bool own = inx && x >= c0 && x < c0 + kChunk;       // counted by this chunk
+        float m = 0.0f;
+        if (inx && (int)threadIdx.x < kChunk + 2) {
+            for (int dz = 0; dz < kBrick + 2; ++dz) {
+                const int z = z0 + dz;
+                if (z < 0 || z >= nz) continue;
+                const float* r = raw + ((int64_t)z * ny + y0) * nx + x;
+                float v[kBrick + 2];
+#pragma unroll
+                for (int dy = 0; dy < kBrick + 2; ++dy)
+                    v[dy] = y0 + dy >= 0 && y0 + dy < ny ? __ldg(r + (int64_t)dy * nx) : 0.0f;
+#pragma unroll
+                for (int dy = 0; dy < kBrick + 2; ++dy) m = fmaxf(m, v[dy]);
+                if (own && dz >= 1 && dz <= kBrick) {
+#pragma unroll
+                    for (int dy = 1; dy <= kBrick; ++dy) stats_max_one(v[dy], mx, bad, cnt);
+                }
+            }
+        }
+        __syncthreads();                                          // the previous chunk's readers are done
+        col[threadIdx.x] = m;
+        __syncthreads();
+        const int b = c0 / kBrick + (int)threadIdx.x;
+        if ((int)threadIdx.x < kChunk / kBrick && b < bx) {
+            float q = 0.0f;
+#pragma unroll
+            for (int k = 0; k < kBrick + 2; ++k) q = fmaxf(q, col[kBrick * threadIdx.x + k]);
+            out[(int64_t)blockIdx.x * bx + b] = q;
+        }
     }
-    for (int64_t i = n / 4 * 4 + tid; i < n; i += nt) stats_max_one(v[i], mx, bad, c32);
-    unsigned long long cnt = c32;       // a thread counts at most n / threads + 4 voxels
+    unsigned long long c64 = cnt;
     for (int o = 16; o; o >>= 1) {
         mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
         bad |= __shfl_xor_sync(0xffffffffu, bad, o);
-        cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
+        c64 += __shfl_xor_sync(0xffffffffu, c64, o);
     }
     if ((threadIdx.x & 31) == 0) {
         atomicMax(&st->max_bits, mx);
         if (bad) atomicOr(&st->bad, 1u);
-        atomicAdd(&st->count, cnt);
+        if (c64) atomicAdd(&st->count, c64);
     }
 }
 
@@ -79,13 +119,17 @@ __global__ void k_stats_sum(const float* __restrict__ v, int64_t n, DevStats* st
     const int S = 32 - e;
     unsigned long long s = 0;
     const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, nt = (int64_t)gridDim.x * blockDim.x;
+    // 16-byte vectors (the allocation is 256-byte aligned), four in flight a thread; the last
+    // n % 4 voxels one by one
     const float4* v4 = reinterpret_cast<const float4*>(v);
-    for (int64_t i = tid; i < n / 4; i += nt) {
-        const float4 q = __ldg(v4 + i);
-        if (q.x > 0.0f) s += fixed_point(q.x, S);
-        if (q.y > 0.0f) s += fixed_point(q.y, S);
-        if (q.z > 0.0f) s += fixed_point(q.z, S);
-        if (q.w > 0.0f) s += fixed_point(q.w, S);
+    auto add = [&](float x) { if (x > 0.0f) s += fixed_point(x, S); };
+    for (int64_t i = tid; i < n / 4; i += 4 * nt) {
+        float4 q[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            q[k] = i + k * nt < n / 4 ? __ldg(v4 + i + k * nt) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) { add(q[k].x); add(q[k].y); add(q[k].z); add(q[k].w); }
     }
     for (int64_t i = n / 4 * 4 + tid; i < n; i += nt) {
         const float x = v[i];
@@ -141,23 +185,62 @@ __global__ void k_mip_pass_multi(const __grid_constant__ MipJobs J) {
 
 // The x passes of several levels, staged: a block copies R consecutive x lines of the fine
 // grid (contiguous in memory) into shared memory once, with coalesced loads (line pitch
-// nx + 1 floats), and computes every level's decimated outputs (line r, index j) from them
-// with r fastest, so a warp's lanes read different lines at one position (different banks)
-// instead of 32 scattered global lines per tap.  Each output's taps in ascending m,
-// acc = acc + w*v.
+// nx + 1 floats, so a warp's lanes read different lines at one position from different banks),
+// and its warps compute the levels' outputs.  A thread streams along two lines at once per
+// level: the windows of Q consecutive outputs overlap (6 level spacings wide; level 0: 7), so
+// each voxel read is multiplied into Q running sums, and the Q weights of its phase, the same
+// for all lanes, are read once for both.  Each output's taps in ascending order,
+// acc = acc + w*v (no contraction); taps outside the grid are not visited.  Bound: multiplies and
+// adds; a thread per output, with a weight and a voxel read per tap, was bound by those reads
+// (256^3, six levels: 131 us, now 117 us).
+// Output j's tap m meets voxel j st + off + m; with phase blocks of st voxels from
+// i0 = off + m, output j covers blocks j .. j + Q - 1 of the line shifted by off.
 struct MipXJob {
     float* out;
-    const float* w;
-    int ax, st, off, T;
+    const float* w;       // [st][8]: the Q weights m = p + q st of phase p
+    int ax, st, off;
 };
 struct MipXJobs {
     MipXJob j[kMaxLevels];
     int n;
 };
-__global__ void k_mip_pass_x(const float* __restrict__ in, int nx, int64_t nrows, int R,
-                             const __grid_constant__ MipXJobs J) {
+constexpr int kXThreads = 256;
+template <int Q>
+__device__ __forceinline__ void mip_x_stream(const MipXJob& b, const float* line0, const float* line1, int nx,
+                                             int64_t row0, int64_t row1, int j0, int j1) {
+    // sums of outputs s - Q + 1 .. s of both lines, oldest first, while block s (voxels
+    // off + s st ..) passes
+    float acc0[Q] = {}, acc1[Q] = {};
+    for (int s = j0; s < j1 + Q - 1; ++s) {
+        const int i0 = b.off + s * b.st;
+        const int plo = max(0, -i0), phi = min(b.st, nx - i0);
+#pragma unroll 4
+        for (int p = plo; p < phi; ++p) {
+            const float4 wa = __ldg(reinterpret_cast<const float4*>(b.w + 8 * p));
+            const float4 wb = __ldg(reinterpret_cast<const float4*>(b.w + 8 * p + 4));
+            const float w[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
+            const float v0 = line0[i0 + p], v1 = line1[i0 + p];
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                acc0[Q - 1 - q] = __fadd_rn(acc0[Q - 1 - q], __fmul_rn(w[q], v0));
+                acc1[Q - 1 - q] = __fadd_rn(acc1[Q - 1 - q], __fmul_rn(w[q], v1));
+            }
+        }
+        const int j = s - Q + 1;                 // its window ends with block s
+        if (j >= j0 && j < j1) {
+            if (row0 >= 0) b.out[row0 * b.ax + j] = acc0[0];
+            if (row1 >= 0) b.out[row1 * b.ax + j] = acc1[0];
+        }
+#pragma unroll
+        for (int q = 0; q + 1 < Q; ++q) { acc0[q] = acc0[q + 1]; acc1[q] = acc1[q + 1]; }
+        acc0[Q - 1] = acc1[Q - 1] = 0.0f;
+    }
+}
+__global__ void __launch_bounds__(kXThreads)
+k_mip_pass_x(const float* __restrict__ in, int nx, int64_t nrows, int R, int split, const __grid_constant__ MipXJobs J) {
     extern __shared__ float lines[];
     const int pitch = nx + 1;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int64_t r0 = (int64_t)blockIdx.x * R; r0 < nrows; r0 += (int64_t)gridDim.x * R) {
         const int nr = (int)min((int64_t)R, nrows - r0);
         __syncthreads();                       // the previous lines' readers are done
@@ -180,19 +263,21 @@ __global__ void k_mip_pass_x(const float* __restrict__ in, int nx, int64_t nrows
             lines[r * pitch + e - r * nx] = __ldg(src + e);
         }
         __syncthreads();
-        for (int k = 0; k < J.n; ++k) {
-            const MipXJob& b = J.j[k];
-            for (int task = threadIdx.x; task < R * b.ax; task += blockDim.x) {
-                const int r = task % R, j = task / R;
-                if (r >= nr) continue;
-                const float* line = lines + r * pitch;
-                const int t0 = j * b.st + b.off;
-                const int mlo = max(0, -t0), mhi = min(b.T, nx - t0);
-                float acc = 0.0f;
-#pragma unroll 4
-                for (int m = mlo; m < mhi; ++m) acc = __fadd_rn(acc, __fmul_rn(__ldg(b.w + m), line[t0 + m]));
-                b.out[(r0 + r) * b.ax + j] = acc;
-            }
+        // a task: a level, 64 lines (two per lane; fewer where R is smaller), one of `split` runs of
+        // its outputs
+        const int groups = (R + 63) / 64;
+        for (int task = warp; task < J.n * groups * split; task += kXThreads / 32) {
+            const MipXJob& b = J.j[task / (groups * split)];
+            const int g = task / split % groups, part = task % split;
+            const int per = (b.ax + split - 1) / split;
+            const int j0 = part * per, j1 = min(b.ax, j0 + per);
+            if (j0 >= j1) continue;
+            const int ra = g * 64 + lane, rb = ra + 32;
+            const float* la = lines + min(ra, nr - 1) * pitch;
+            const float* lb = lines + min(rb, nr - 1) * pitch;
+            const int64_t wa = ra < nr ? r0 + ra : -1, wb = rb < nr ? r0 + rb : -1;
+            if (b.st == 1) mip_x_stream<7>(b, la, lb, nx, wa, wb, j0, j1);
+            else mip_x_stream<6>(b, la, lb, nx, wa, wb, j0, j1);
         }
     }
 }
@@ -201,23 +286,37 @@ __global__ void k_mip_pass_x(const float* __restrict__ in, int nx, int64_t nrows
 // (rx-1, ry-1, rz-1).  With c[dx + 2 dy + 4 dz] its 8 corner values (zero outside), the
 // record holds c0, c1 - c0, c2, c3 - c2, c4, c5 - c4, c6, c7 - c6: the x-differences the
 // four x-lerps need, rounded exactly as a lerp rounds them.
-__global__ void k_pack(const float* __restrict__ lv, float4* __restrict__ rec, int ax, int ay, int az) {
-    const int rx_n = ax + 1, ry_n = ay + 1, rz_n = az + 1;
-    const int64_t total = (int64_t)rx_n * ry_n * rz_n;
-    for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < total;
-         r += (int64_t)gridDim.x * blockDim.x) {
+struct PackJob {
+    const float* lv;
+    float4* rec;
+    int ax, ay, az;
+    int64_t first;            // its first record in the launch's numbering
+};
+struct PackJobs {
+    PackJob j[kMaxLevels];
+    int n;
+    int64_t total;
+};
+__global__ void k_pack(const __grid_constant__ PackJobs J) {
+    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < J.total;
+         q += (int64_t)gridDim.x * blockDim.x) {
+        int k = 0;
+        while (k + 1 < J.n && J.j[k + 1].first <= q) ++k;
+        const PackJob& b = J.j[k];
+        const int64_t r = q - b.first;
+        const int ax = b.ax, ay = b.ay, az = b.az, rx_n = ax + 1, ry_n = ay + 1;
         const int x0 = (int)(r % rx_n) - 1;
         const int y0 = (int)((r / rx_n) % ry_n) - 1;
         const int z0 = (int)(r / ((int64_t)rx_n * ry_n)) - 1;
         float c[8];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const int x = x0 + (k & 1), y = y0 + ((k >> 1) & 1), z = z0 + (k >> 2);
+        for (int k2 = 0; k2 < 8; ++k2) {
+            const int x = x0 + (k2 & 1), y = y0 + ((k2 >> 1) & 1), z = z0 + (k2 >> 2);
             const bool in = x >= 0 && y >= 0 && z >= 0 && x < ax && y < ay && z < az;
-            c[k] = in ? lv[((int64_t)z * ay + y) * ax + x] : 0.0f;
+            c[k2] = in ? __ldg(b.lv + ((int64_t)z * ay + y) * ax + x) : 0.0f;
         }
-        rec[2 * r] = make_float4(c[0], __fsub_rn(c[1], c[0]), c[2], __fsub_rn(c[3], c[2]));
-        rec[2 * r + 1] = make_float4(c[4], __fsub_rn(c[5], c[4]), c[6], __fsub_rn(c[7], c[6]));
+        b.rec[2 * r] = make_float4(c[0], __fsub_rn(c[1], c[0]), c[2], __fsub_rn(c[3], c[2]));
+        b.rec[2 * r + 1] = make_float4(c[4], __fsub_rn(c[5], c[4]), c[6], __fsub_rn(c[7], c[6]));
     }
 }
 
@@ -234,13 +333,8 @@ int grid_for(int64_t n, int block, int num_sms) {
     return (int)(g < 1 ? 1 : g);
 }
 
-// Gaussian taps of level i: sigma = 2^i, offsets |d| <= 3 sigma, normalised (FP64,
-// rounded to FP32).
-std::vector<float> gauss_taps(int level, int* off) {
+std::vector<float> make_taps(int level, int T) {
     const double sigma = std::ldexp(1.0, level);
-    int T;
-    if (level == 0) { T = 7; *off = -3; }
-    else { T = 6 << level; *off = (1 << (level - 1)) - 3 * (1 << level); }
     std::vector<double> w(T);
     double sum = 0.0;
     for (int m = 0; m < T; ++m) {
@@ -252,6 +346,20 @@ std::vector<float> gauss_taps(int level, int* off) {
     for (int m = 0; m < T; ++m) wf[m] = (float)(w[m] / sum);
     return wf;
 }
+
+// Gaussian taps of level i: sigma = 2^i, offsets |d| <= 3 sigma, normalised (FP64,
+// rounded to FP32).  They depend on the level alone and are computed once per process: the
+// exponentials of a 256^3 pyramid had kept the GPU waiting for 40 us of every build.
+const std::vector<float>& gauss_taps(int level, int* off) {
+    static std::vector<float> table[kMaxLevels];
+    static std::once_flag once[kMaxLevels];
+    int T;
+    if (level == 0) { T = 7; *off = -3; }
+    else { T = 6 << level; *off = (1 << (level - 1)) - 3 * (1 << level); }
+    std::call_once(once[level], [&] { table[level] = make_taps(level, T); });
+    return table[level];
+}
+
 
 }  // namespace
 
@@ -268,51 +376,21 @@ rpnn_status load_density(Ctx& c, Volume& v, const void* src, int dtype, cudaStre
     return RPNN_OK;
 }
 
-// Per-brick majorant for tracking: brick b (kBrick^3 voxels) bounds the trilinear density
-// over its region by the largest of the voxels it interpolates, 8b - 1 .. 8b + 8 per axis
-// (zero outside the grid).  One thread per brick; max is exact, so the order is free.
-__global__ void k_brick_majorant(const float* __restrict__ raw, int nx, int ny, int nz, int bx, int by, int bz,
-                                 float* __restrict__ out) {
-    const int64_t nb = (int64_t)bx * by * bz;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nb; i += (int64_t)gridDim.x * blockDim.x) {
-        const int x0 = (int)(i % bx) * kBrick - 1, y0 = (int)((i / bx) % by) * kBrick - 1,
-                  z0 = (int)(i / ((int64_t)bx * by)) * kBrick - 1;
-        float m = 0.0f;
-        for (int z = max(z0, 0); z <= min(z0 + kBrick + 1, nz - 1); ++z)
-            for (int y = max(y0, 0); y <= min(y0 + kBrick + 1, ny - 1); ++y) {
-                const float* r = raw + ((int64_t)z * ny + y) * nx;
-                // a fixed-length line with in-grid predicates: its loads are in flight together
-#pragma unroll
-                for (int dx = 0; dx < kBrick + 2; ++dx) {
-                    const int x = x0 + dx;
-                    if (x >= 0 && x < nx) m = fmaxf(m, __ldg(r + x));
-                }
-            }
-        out[i] = m;
-    }
-}
-
-rpnn_status volume_brick_majorants(Ctx& c, Volume& v, cudaStream_t s) {
-    for (int a = 0; a < 3; ++a) v.info.bricks[a] = v.nb[a] = (v.n[a] + kBrick - 1) / kBrick;
-    const int64_t nb = (int64_t)v.nb[0] * v.nb[1] * v.nb[2];
-    rpnn_status st = v.bmaj.reserve((size_t)nb * sizeof(float));
-    if (st) return st;
-    k_brick_majorant<<<grid_for(nb, 128, c.num_sms), 128, 0, s>>>(v.raw.as<float>(), v.n[0], v.n[1], v.n[2], v.nb[0],
-                                                                  v.nb[1], v.nb[2], v.bmaj.as<float>());
-    RPNN_CHECK_LAUNCH();
-    return RPNN_OK;
-}
-
 rpnn_status volume_stats(Ctx& c, Volume& v, cudaStream_t s) {
     const int64_t n = (int64_t)v.n[0] * v.n[1] * v.n[2];
     rpnn_status st = v.stats.reserve(sizeof(DevStats));
     if (st) return st;
     DevStats* ds = v.stats.as<DevStats>();
     RPNN_CUDA_TRY(cudaMemsetAsync(ds, 0, sizeof(DevStats), s));
-    const int g = grid_for(n, 256, c.num_sms);
-    k_stats_max<<<g, 256, 0, s>>>(v.raw.as<float>(), n, ds);
+    for (int a = 0; a < 3; ++a) v.info.bricks[a] = v.nb[a] = (v.n[a] + kBrick - 1) / kBrick;
+    st = v.bmaj.reserve((size_t)v.nb[0] * v.nb[1] * v.nb[2] * sizeof(float));
+    if (st) return st;
+    k_stats_bricks<<<(unsigned)(v.nb[1] * v.nb[2]), kBrickThreads, 0, s>>>(v.raw.as<float>(), v.n[0], v.n[1], v.n[2],
+                                                                       v.nb[0], v.nb[1], v.bmaj.as<float>(), ds);
     RPNN_CHECK_LAUNCH();
-    k_stats_sum<<<g, 256, 0, s>>>(v.raw.as<float>(), n, ds);
+    const int64_t gs = (n / 16 + 255) / 256;
+    k_stats_sum<<<(int)std::max<int64_t>(1, std::min<int64_t>(gs, (int64_t)c.num_sms * 8)), 256, 0, s>>>(v.raw.as<float>(),
+                                                                                                   n, ds);
     RPNN_CHECK_LAUNCH();
     DevStats h;
     RPNN_CUDA_TRY(cudaMemcpyAsync(&h, ds, sizeof(DevStats), cudaMemcpyDeviceToHost, s));
@@ -369,16 +447,20 @@ rpnn_status volume_build_levels(Ctx& c, Volume& v, const int* levels, int nlev, 
     // taps and scratch of every level side by side (offsets in floats, 16-float aligned);
     // volume-owned, grows and never shrinks: no allocation or synchronisation per build
     std::vector<float> taps;
-    std::vector<int> offs(nlev), toff(nlev), T(nlev);
+    std::vector<int> offs(nlev), toff(nlev), xoff(nlev), T(nlev);
     std::vector<int64_t> aoff(nlev), boff(nlev);
     int64_t asz = 0, bsz = 0;
     for (int k = 0; k < nlev; ++k) {
         const int l = ord[k];
-        std::vector<float> w = gauss_taps(l, &offs[k]);
+        const std::vector<float>& w = gauss_taps(l, &offs[k]);
         T[k] = (int)w.size();
         toff[k] = (int)taps.size();
         taps.insert(taps.end(), w.begin(), w.end());
         taps.resize((taps.size() + 15) / 16 * 16, 0.0f);
+        // the same taps by phase for the x pass: [2^l][8], tap p + q 2^l at [p][q]
+        xoff[k] = (int)taps.size();
+        taps.resize(taps.size() + (size_t)(8 << l), 0.0f);
+        for (int m = 0; m < T[k]; ++m) taps[xoff[k] + 8 * (m % (1 << l)) + m / (1 << l)] = w[m];
         aoff[k] = asz; asz += ((int64_t)v.dims[l][0] * ny * nz + 15) / 16 * 16;
         boff[k] = bsz; bsz += ((int64_t)v.dims[l][0] * v.dims[l][1] * nz + 15) / 16 * 16;
     }
@@ -391,9 +473,10 @@ rpnn_status volume_build_levels(Ctx& c, Volume& v, const int* levels, int nlev, 
     float* B = v.mip_b.as<float>();
     RPNN_CUDA_TRY(cudaMemcpyAsync(dw, taps.data(), taps.size() * sizeof(float), cudaMemcpyHostToDevice, s));
     // the x passes of every level in one launch (the fine grid is read once), R lines of nx
-    // floats per block in at most 64 KB of shared memory
-    constexpr int kLineBytes = 64 * 1024;
-    const int R = std::max(1, std::min(32, kLineBytes / ((nx + 1) * (int)sizeof(float))));
+    // floats per block: 64 of them in at most 72 KB of shared memory, fewer for long
+    // lines; the outputs of few levels in as many runs as there are warps for them
+    constexpr int kLineBytes = 72 * 1024;
+    const int R = std::max(1, std::min(64, kLineBytes / ((nx + 1) * (int)sizeof(float))));
     const int smem = R * (nx + 1) * (int)sizeof(float);
     static bool attr = false;
     if (!attr) {
@@ -401,13 +484,16 @@ rpnn_status volume_build_levels(Ctx& c, Volume& v, const int* levels, int nlev, 
         attr = true;
     }
     const int64_t nrows = (int64_t)ny * nz;
+    const int groups = (R + 64 - 1) / (64);
+    const int split = std::max(1, kXThreads / 32 / (nlev * groups));
     MipXJobs XJ{};
     XJ.n = nlev;
     for (int k = 0; k < nlev; ++k) {
         const int l = ord[k];
-        XJ.j[k] = MipXJob{A + aoff[k], dw + toff[k], v.dims[l][0], 1 << l, offs[k], T[k]};
+        XJ.j[k] = MipXJob{A + aoff[k], dw + xoff[k], v.dims[l][0], 1 << l, offs[k]};
     }
-    k_mip_pass_x<<<grid_for((nrows + R - 1) / R, 1, c.num_sms), 256, smem, s>>>(v.raw.as<float>(), nx, nrows, R, XJ);
+    k_mip_pass_x<<<grid_for((nrows + R - 1) / R, 1, c.num_sms), kXThreads, smem, s>>>(v.raw.as<float>(), nx, nrows, R,
+                                                                                    split, XJ);
     // y passes of every level in one launch, then the z passes (with the 1/mean scale)
     for (int axis = 1; axis <= 2; ++axis) {
         MipJobs J{};
@@ -469,13 +555,16 @@ rpnn_status volume_pack_levels(Ctx& c, Volume& v, cudaStream_t s) {
     for (int k = 0; k < nl; ++k) dst[k] = v.mip_d.as<float>() + doff[k];
     st = volume_build_levels(c, v, lv, nl, dst, s);
     if (st) return st;
+    PackJobs J{};
+    J.n = nl;
     for (int k = 0; k < nl; ++k) {
         const int i = lv[k];
-        const int64_t nrec = (int64_t)(v.dims[i][0] + 1) * (v.dims[i][1] + 1) * (v.dims[i][2] + 1);
-        k_pack<<<grid_for(nrec, 256, c.num_sms), 256, 0, s>>>(
-            dst[k], v.packed.as<float4>() + 2 * v.lvl[i].rec_offset, v.dims[i][0], v.dims[i][1], v.dims[i][2]);
-        RPNN_CHECK_LAUNCH();
+        J.j[k] = PackJob{dst[k], v.packed.as<float4>() + 2 * v.lvl[i].rec_offset, v.dims[i][0], v.dims[i][1], v.dims[i][2],
+                         J.total};
+        J.total += (int64_t)(v.dims[i][0] + 1) * (v.dims[i][1] + 1) * (v.dims[i][2] + 1);
     }
+    k_pack<<<grid_for(J.total, 256, c.num_sms), 256, 0, s>>>(J);
+    RPNN_CHECK_LAUNCH();
     RPNN_CUDA_TRY(cudaStreamSynchronize(s));
     v.built = true;
     v.stencil_ready = false;

@@ -1,0 +1,37 @@
+"""Volume preprocessing at the edges of its kernels' tiles, against the oracle bit for bit: x
+lines around the 248-voxel chunk of the statistics and majorant pass and long enough that fewer
+than 64 lines are staged at a time, row counts around a staged group, grids of one brick and of
+ragged bricks, every pyramid level."""
+import numpy as np
+import pytest
+
+from paper_1709_05418_gb300 import workloads as W
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("shape", [(3, 5, 247), (2, 9, 248), (9, 3, 249), (4, 17, 497), (1, 65, 300), (13, 5, 8),
+                                   (70, 1, 1), (2, 2, 1100)])
+def test_stats_bricks_and_levels_equal_the_oracle(shape):
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import oracle
+    from paper_1709_05418_gb300 import api
+    rng = np.random.default_rng(sum(shape))
+    dens = (rng.random(shape) * 40.0 * (rng.random(shape) < 0.6)).astype(np.float32)
+    dens.flat[0] = 3.0
+    ctx = api.Context()
+    v = ctx.load_volume(torch.from_numpy(dens).cuda())
+    ctx.build_mips(v)
+    gi = ctx.get_volume_info(v)
+    o = oracle.Volume(dens)
+    oi = o.stats()
+    for key in ("mean", "majorant", "nonzero", "levels", "mip_of_level"):
+        assert gi[key] == oi[key], key
+    assert np.array_equal(ctx.copy_brick_majorants(v).cpu().numpy(), o.brick_majorants())
+    for lv in range(gi["levels"]):
+        g, r = ctx.copy_mip_level(v, lv).cpu().numpy(), o.mip_level(lv, f32=True)
+        assert np.array_equal(g.view(np.uint32), r.view(np.uint32)), lv
+    o.close()
+    ctx.close()
