@@ -329,13 +329,14 @@ __global__ void k_build_image(const float* __restrict__ P, ParamLayout L, TcArgs
         const int c = chunk * 32 + (((pos / 8) ^ ((n >> 1) & 3)) * 8) + pos % 8;
         constexpr int KZ = FmtBF16::KZB / 2;
         // layers l >= 1 read the activation, whose column 200 is the constant 1: the
-        // image holds the layer's bias in that column
+        // image holds the layer's bias in that column.  Layer 0 has no W1 (L.W1[0] = -1): its
+        // last block's columns 240 .. 255, which no MMA reads, are zeros
         float v = 0.0f;
         if (n < RPNN_H) {
             if (l < 20 && !(l & 1)) {
                 const int k = l / 2;
                 if (c < RPNN_DIN) v = P[L.V[k] + (int64_t)n * RPNN_DIN + c];
-                else if (c >= KZ && c < KZ + RPNN_H) v = P[L.W1[k] + (int64_t)n * RPNN_H + (c - KZ)];
+                else if (l > 0 && c >= KZ && c < KZ + RPNN_H) v = P[L.W1[k] + (int64_t)n * RPNN_H + (c - KZ)];
                 else if (c == KZ + RPNN_H && l > 0) v = P[L.b1[k] + n];
             } else if (c < RPNN_H) {
                 const int64_t off = l < 20 ? L.W2[l / 2] : L.T[l - 20];
