@@ -456,14 +456,16 @@ def run_batch(args, ws, rank, local):
 
 
 def train_launches(tab, bf16, batch):
-    """Kernels of one training step.  FP32: 23 forward GEMMs, the loss (2), 78 backward launches
-    (GEMMs, bias-gradient sums, one mask), Adam and the BF16 render image.  BF16: the training
+    """Kernels of one training step.  FP32: 23 forward launches, the loss (2), the output layer's
+    backward (4: mask, weight gradient, bias sum, data gradient), 21 data gradients, the grouped
+    bias sums and weight gradients (1 each), Adam and the BF16 render image.  BF16: the training
     weight image and descriptor conversion, the forward (one launch of the persistent
     tensor-core network in its training form), the loss (2), 4 output-layer backward launches,
-    1 conversion, 74 backward GEMMs and sums, Adam and the render image.  Plus one reduction
-    per split-K weight-gradient GEMM: the 200 x 200 shape runs 21 times a step (T1, T2, W2 x 10,
-    W1 x 9), the 200 x 226 one 10 times, the 1 x 200 once."""
-    n = 86 if bf16 else 105
+    1 conversion, 74 backward GEMMs and sums, Adam and the render image.  Plus the reductions of
+    split-K weight gradients: one for FP32's grouped launch and for the 1 x 200 one; in BF16 one
+    per GEMM, of which the 200 x 200 shape runs 21 times a step (T1, T2, W2 x 10, W1 x 9) and
+    the 200 x 226 one 10 times."""
+    n = 86 if bf16 else 54
     for e in tab:
         if e["splits"] <= 1 or e["K0"] != batch:
             continue
@@ -471,7 +473,7 @@ def train_launches(tab, bf16, batch):
         if e["M"] == 1:
             n += 1
         elif tc == bf16:
-            n += 21 if e["N"] == 200 else 10
+            n += (21 if e["N"] == 200 else 10) if bf16 else 1
     return n
 
 

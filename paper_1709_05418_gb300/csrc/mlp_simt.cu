@@ -327,6 +327,55 @@ k_gemm(int M_host, const int* __restrict__ M_dev, int N, const __grid_constant__
     gemm_tile<BM, BN, BK, TM, TN>(sm, M, M_host, N, m0, n0, n1, (int)blockIdx.z, s0, s1, nseg, e, splits, ws);
 }
 
+// Weight gradients of many layers in one launch, C_j = A_j^T B_j with A_j [K][M] and B_j [K][N_j]
+// (rows pitch M and ldb): block z takes run z % splits of job z / splits.  One layer's gradient
+// (200 x 200 outputs) is 28 blocks or fewer; all 32 fill the chip without a split of K.
+constexpr int kMaxWJobs = 40;
+struct WJob {
+    const float *A, *B;
+    float* C;
+    int64_t ldb;
+    int N;
+};
+struct WJobs {
+    WJob j[kMaxWJobs];
+    int n, M, K, splits;
+    float* ws;                // splits > 1: partial sums, job j's at ws + j * ws_job
+    int64_t ws_job;
+};
+template <int BM, int BN, int BK, int TM, int TN>
+__global__ void __launch_bounds__(GemmCfg<BM, BN, BK, TM, TN>::NT, GemmCfg<BM, BN, BK, TM, TN>::BLOCKS)
+k_wgrad(const __grid_constant__ WJobs J) {
+    using C = GemmCfg<BM, BN, BK, TM, TN>;
+    __shared__ __align__(16) float sm[C::STAGES * C::STAGE];
+    const int job = (int)blockIdx.z / J.splits, z = (int)blockIdx.z % J.splits;
+    const WJob& w = J.j[job];
+    const int tiles = (w.N + BN - 1) / BN;
+    if ((int)blockIdx.x >= tiles) return;
+    int n0, n1;
+    column_range(w.N, tiles, C::STRIP, (int)blockIdx.x, n0, n1);
+    if (n0 >= n1) return;
+    Seg s;
+    s.A = w.A; s.sam = 1; s.sak = J.M;
+    s.B = w.B; s.sbk = w.ldb; s.sbn = 1;
+    s.K = J.K;
+    Epi e{};
+    e.C = w.C; e.ldc = w.N;
+    gemm_tile<BM, BN, BK, TM, TN>(sm, J.M, J.M, w.N, (int)blockIdx.y * BM, n0, n1, z, s, s, 1, e, J.splits,
+                                  J.ws + job * J.ws_job);
+}
+// the runs' partial sums of every job, added in run order
+__global__ void k_wgrad_sum(const __grid_constant__ WJobs J) {
+    const WJob& w = J.j[blockIdx.y];
+    const float* ws = J.ws + blockIdx.y * J.ws_job;
+    const int64_t total = (int64_t)J.M * w.N;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+        float v = 0.0f;
+        for (int z = 0; z < J.splits; ++z) v += ws[z * total + i];
+        w.C[i] = v;
+    }
+}
+
 // N = 1 (the output layer): one thread per row sums its K products in increasing k with one
 // FMA each, as a k_gemm output does; the block's 64 rows pass through shared memory in pieces
 // of 40 columns so the loads are coalesced.
@@ -403,8 +452,8 @@ __global__ void k_mask(const float* __restrict__ x, const float* __restrict__ m,
 // (x, y) sums rows y, y + 128, ... of column x in increasing order, then the 128 partial sums
 // are added in y order (a fixed order for given M).
 constexpr int kColsumCols = 8, kColsumRows = 128;
-__global__ void __launch_bounds__(kColsumCols * kColsumRows) k_colsum(const float* __restrict__ X, int M, int N,
-                                                                   int64_t ld, float* __restrict__ out) {
+__device__ __forceinline__ void colsum_block(const float* __restrict__ X, int M, int N, int64_t ld,
+                                             float* __restrict__ out) {
     __shared__ float part[kColsumRows][kColsumCols + 1];
     const int n = blockIdx.x * kColsumCols + threadIdx.x;
     float s = 0.0f;
@@ -417,6 +466,19 @@ __global__ void __launch_bounds__(kColsumCols * kColsumRows) k_colsum(const floa
         for (int y = 0; y < kColsumRows; ++y) t += part[y][threadIdx.x];
         out[n] = t;
     }
+}
+__global__ void __launch_bounds__(kColsumCols * kColsumRows) k_colsum(const float* __restrict__ X, int M, int N,
+                                                                   int64_t ld, float* __restrict__ out) {
+    colsum_block(X, M, N, ld, out);
+}
+// the bias gradients of many layers, each [M][N]
+struct ColsumJobs {
+    const float* X[kMaxWJobs];
+    float* out[kMaxWJobs];
+    int n, M, N;
+};
+__global__ void __launch_bounds__(kColsumCols * kColsumRows) k_colsums(const __grid_constant__ ColsumJobs J) {
+    colsum_block(J.X[blockIdx.y], J.M, J.N, J.N, J.out[blockIdx.y]);
 }
 
 void launch_colsum(const float* X, int M, int N, int64_t ld, float* out, cudaStream_t s) {
@@ -480,6 +542,32 @@ rpnn_status launch_gemm(int tile, int splits, int M, const int* M_dev, int N, co
         int64_t b = (total + 255) / 256;
         if (b > 152 * 8) b = 152 * 8;
         k_splitk_epi<<<(unsigned)b, 256, 0, s>>>(ws, splits, M, M_dev, N, e);
+        RPNN_CHECK_LAUNCH();
+    }
+    return RPNN_OK;
+}
+
+template <int BM, int BN, int BK, int TM, int TN>
+void launch_wtile(const WJobs& J, cudaStream_t s) {
+    int nmax = 1;
+    for (int j = 0; j < J.n; ++j) nmax = std::max(nmax, J.j[j].N);
+    const dim3 grid((nmax + BN - 1) / BN, (J.M + BM - 1) / BM, J.n * J.splits);
+    k_wgrad<BM, BN, BK, TM, TN><<<grid, GemmCfg<BM, BN, BK, TM, TN>::NT, 0, s>>>(J);
+}
+
+rpnn_status launch_wgrads(int tile, const WJobs& J, cudaStream_t s) {
+    switch (tile) {
+        case 0: launch_wtile<64, 64, 16, 4, 8>(J, s); break;
+        case 1: launch_wtile<128, 64, 16, 8, 8>(J, s); break;
+        case 2: launch_wtile<64, 128, 16, 8, 8>(J, s); break;
+        case 3: launch_wtile<128, 128, 8, 8, 8>(J, s); break;
+        case 4: launch_wtile<32, 64, 16, 4, 4>(J, s); break;
+        case 5: launch_wtile<128, 32, 16, 8, 4>(J, s); break;
+        default: launch_wtile<32, 128, 16, 4, 8>(J, s); break;
+    }
+    RPNN_CHECK_LAUNCH();
+    if (J.splits > 1) {
+        k_wgrad_sum<<<dim3(32, J.n), 256, 0, s>>>(J);
         RPNN_CHECK_LAUNCH();
     }
     return RPNN_OK;
@@ -595,7 +683,84 @@ rpnn_status gemm(Ctx* c, int M, const int* M_dev, int N, const Seg& s0, const Se
     return launch_gemm(ch.tile, ch.splits, M, M_dev, N, s0, s1r, nseg, e, ws, s);
 }
 
-// Deterministic log-MSE loss (Sec. 5.2): one block; FP64 tree reduction.
+// All of J's weight gradients; the tile and split of the shape (M, first job's N, K) are timed
+// on the whole launch at its first use like gemm()'s, and recorded under the key one such GEMM
+// has.
+rpnn_status wgrads(Ctx& c, WJobs& J, cudaStream_t s) {
+    if (J.n == 0) return RPNN_OK;
+    GemmTuner& tu = c.tuner;
+    int nmax = 1;
+    for (int j = 0; j < J.n; ++j) nmax = std::max(nmax, J.j[j].N);
+    J.ws_job = 0;
+    J.splits = 1;
+    int tile = 0;
+    if (tu.enabled) {
+        Seg sg = seg(J.j[0].A, 1, J.M, J.j[0].B, J.j[0].ldb, 1, J.K);
+        const GemmKey key = make_key(J.M, J.j[0].N, sg, nullptr, epi(J.j[0].C, J.j[0].N), false);
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        RPNN_CUDA_TRY(cudaStreamIsCapturing(s, &cs));
+        const GemmChoice* hit = tu.find(key);
+        if (hit) {
+            tile = hit->tile;
+            J.splits = hit->splits;
+        } else if (cs == cudaStreamCaptureStatusNone) {
+            struct Cand { int t, sp; };
+            std::vector<Cand> cands;
+            int maxsplit = 1;
+            for (int t = 0; t < kNumTiles; ++t) {
+                const TileShape& ts = kTiles[t];
+                const int64_t blocks = (int64_t)((nmax + ts.bn - 1) / ts.bn) * ((J.M + ts.bm - 1) / ts.bm) * J.n;
+                for (int sp : kSplits) {
+                    if (sp > 1 && (J.K < kMinSplitK || blocks >= 4 * c.num_sms || J.K / ts.bk / sp < 4)) continue;
+                    cands.push_back({t, sp});
+                    maxsplit = std::max(maxsplit, sp);
+                }
+            }
+            const int64_t out_job = (int64_t)J.M * nmax;
+            rpnn_status st = tu.scratch.reserve((size_t)out_job * J.n * sizeof(float));
+            if (!st && maxsplit > 1) st = tu.ws.reserve((size_t)maxsplit * out_job * J.n * sizeof(float));
+            if (st) return st;
+            if (!tu.ev0) {
+                RPNN_CUDA_TRY(cudaEventCreate(&tu.ev0));
+                RPNN_CUDA_TRY(cudaEventCreate(&tu.ev1));
+            }
+            WJobs T = J;
+            for (int j = 0; j < J.n; ++j) T.j[j].C = tu.scratch.as<float>() + j * out_job;
+            T.ws = tu.ws.as<float>();
+            GemmChoice best{0, 1, 1e30f, 0.0f};
+            for (const Cand& cd : cands) {
+                T.splits = cd.sp;
+                T.ws_job = cd.sp * out_job;
+                st = launch_wgrads(cd.t, T, s);            // warm
+                if (st) return st;
+                RPNN_CUDA_TRY(cudaEventRecord(tu.ev0, s));
+                for (int r = 0; r < 3; ++r) {
+                    st = launch_wgrads(cd.t, T, s);
+                    if (st) return st;
+                }
+                RPNN_CUDA_TRY(cudaEventRecord(tu.ev1, s));
+                RPNN_CUDA_TRY(cudaEventSynchronize(tu.ev1));
+                float ms = 0.0f;
+                RPNN_CUDA_TRY(cudaEventElapsedTime(&ms, tu.ev0, tu.ev1));
+                const float us = ms * 1000.0f / 3.0f / J.n;
+                if (cd.t == 0 && cd.sp == 1) best.default_us = us;
+                if (us < best.us) { best.us = us; best.tile = cd.t; best.splits = cd.sp; }
+            }
+            tu.table.emplace_back(key, best);
+            ++tu.version;
+            tile = best.tile;
+            J.splits = best.splits;
+        }
+    }
+    if (J.splits > 1) {
+        J.ws_job = (int64_t)J.splits * J.M * nmax;
+        rpnn_status st = tu.ws.reserve((size_t)J.ws_job * J.n * sizeof(float));
+        if (st) return st;
+        J.ws = tu.ws.as<float>();
+    }
+    return launch_wgrads(tile, J, s);
+}
+
 // log-MSE loss (Sec. 5.2): per element r = log1p(g) - log1p(t) and dl/dg = 2 r / ((1 + g) B)
 // in FP64, block sums of r^2 in a fixed tree, then the block sums in block order.  Spread
 // over blocks: an FP64 log1p per element on one SM took tens of microseconds per step.
@@ -757,14 +922,49 @@ rpnn_status rpnn_backward_f32(Ctx& c, const NetDims& nd, const float* P, const f
     const int64_t H = RPNN_H, ZS = (int64_t)RPNN_K * nd.stride;
     auto slot = [&](int i) { return saved + (size_t)i * q * H; };
     const float* g = saved + (size_t)22 * q * H;
-    rpnn_status st = c.act0.reserve((size_t)q * H * sizeof(float));
-    if (!st) st = c.act1.reserve((size_t)q * H * sizeof(float));
-    if (!st) st = c.act2.reserve((size_t)q * H * sizeof(float));
-    if (!st) st = c.t_dg.reserve((size_t)q * sizeof(float));
+    // Up to kGroupRows rows every layer's gradient is kept and the 32 weight gradients and 22
+    // bias sums follow the data-gradient chain as one launch each: one layer's cannot fill the
+    // chip (a step of 1,000 rows: 1.41 -> 0.64 ms).  Beyond that a layer's own launches do,
+    // and two buffers instead of 22 are enough.
+    constexpr int64_t kGroupRows = 1 << 17;
+    const bool group = q <= kGroupRows;
+    constexpr int NG = 22;
+    rpnn_status st = c.t_dg.reserve((size_t)q * sizeof(float));
+    if (group) {
+        if (!st) st = c.t_gb32.reserve((size_t)NG * q * H * sizeof(float));
+    } else {
+        if (!st) st = c.act0.reserve((size_t)q * H * sizeof(float));
+        if (!st) st = c.act1.reserve((size_t)q * H * sizeof(float));
+        if (!st) st = c.act2.reserve((size_t)q * H * sizeof(float));
+    }
     if (st) return st;
-    float* bufA = c.act0.as<float>();
-    float* bufB = c.act1.as<float>();
-    float* da = c.act2.as<float>();
+    float* const two[2] = {c.act0.as<float>(), c.act1.as<float>()};
+    int next = 0, flip = 0;
+    // buffers of the layers' pre-activation gradients: dpre of a block or standard layer, and da1
+    auto pre = [&]() { return group ? c.t_gb32.as<float>() + (size_t)(next++) * q * H : two[flip ^= 1]; };
+    auto inner = [&]() { return group ? c.t_gb32.as<float>() + (size_t)(next++) * q * H : c.act2.as<float>(); };
+    WJobs wj{};
+    wj.M = RPNN_H; wj.K = M;
+    ColsumJobs cj{};
+    cj.M = M; cj.N = RPNN_H;
+    // dW = da^T x over the q rows, x [q][N] with row pitch ldx
+    auto wgrad = [&](const float* da, const float* x, int64_t ldx, int N, float* dst) -> rpnn_status {
+        if (group) {
+            wj.j[wj.n++] = WJob{da, x, dst, ldx, N};
+            return RPNN_OK;
+        }
+        return gemm(&c, RPNN_H, nullptr, N, seg(da, 1, H, x, ldx, 1, M), nullptr, epi(dst, N), s);
+    };
+    auto bgrad = [&](const float* da, float* dst) -> rpnn_status {
+        if (group) {
+            cj.X[cj.n] = da;
+            cj.out[cj.n++] = dst;
+            return RPNN_OK;
+        }
+        launch_colsum(da, M, RPNN_H, H, dst, s);
+        RPNN_CHECK_LAUNCH();
+        return RPNN_OK;
+    };
     float* da3 = c.t_dg.as<float>();
     // last layer: g = relu(T3 o12 + bT3): da3 = dout * (g > 0)
     k_mask<<<(M + 255) / 256, 256, 0, s>>>(dout, g, M, da3);
@@ -775,53 +975,55 @@ rpnn_status rpnn_backward_f32(Ctx& c, const NetDims& nd, const float* P, const f
     launch_colsum(da3, M, 1, 1, dP + L.bT[2], s);
     RPNN_CHECK_LAUNCH();
     // da2 = (da3 T3) * (o12 > 0)
+    float* A = pre();
     st = gemm(&c, M, nullptr, RPNN_H, seg(da3, 1, 1, P + L.T[2], H, 1, 1), nullptr,
-              epi(bufA, H, nullptr, 0, nullptr, 0, slot(21), H), s);
+              epi(A, H, nullptr, 0, nullptr, 0, slot(21), H), s);
     if (st) return st;
     // standard layer 2: input o11 (slot 20); layer 1: input o10 (slot 9)
     const float* tin[2] = {slot(9), slot(20)};
     for (int t = 1; t >= 0; --t) {
         // dT = da^T x_in; db = colsum(da)
-        st = gemm(&c, RPNN_H, nullptr, RPNN_H, seg(bufA, 1, H, tin[t], H, 1, M), nullptr, epi(dP + L.T[t], H), s);
+        st = wgrad(A, tin[t], H, RPNN_H, dP + L.T[t]);
+        if (!st) st = bgrad(A, dP + L.bT[t]);
         if (st) return st;
-        launch_colsum(bufA, M, RPNN_H, H, dP + L.bT[t], s);
-        RPNN_CHECK_LAUNCH();
         // d x_in = da T, masked by (x_in > 0) (x_in is a ReLU output)
-        st = gemm(&c, M, nullptr, RPNN_H, seg(bufA, H, 1, P + L.T[t], H, 1, RPNN_H), nullptr,
-                  epi(bufB, H, nullptr, 0, nullptr, 0, tin[t], H), s);
+        float* B = pre();
+        st = gemm(&c, M, nullptr, RPNN_H, seg(A, H, 1, P + L.T[t], H, 1, RPNN_H), nullptr,
+                  epi(B, H, nullptr, 0, nullptr, 0, tin[t], H), s);
         if (st) return st;
-        float* tmp = bufA; bufA = bufB; bufB = tmp;
+        A = B;
     }
-    // bufA = dpre_10 = dl/d(pre-activation of o^10)
+    // A = dpre_10 = dl/d(pre-activation of o^10)
     for (int k = RPNN_K - 1; k >= 0; --k) {
         const float* f1 = slot(10 + k);
         // dW2 = dpre^T F1; db2 = colsum(dpre)
-        st = gemm(&c, RPNN_H, nullptr, RPNN_H, seg(bufA, 1, H, f1, H, 1, M), nullptr, epi(dP + L.W2[k], H), s);
+        st = wgrad(A, f1, H, RPNN_H, dP + L.W2[k]);
+        if (!st) st = bgrad(A, dP + L.b2[k]);
         if (st) return st;
-        launch_colsum(bufA, M, RPNN_H, H, dP + L.b2[k], s);
-        RPNN_CHECK_LAUNCH();
         // da1 = (dpre W2) * (F1 > 0)
-        st = gemm(&c, M, nullptr, RPNN_H, seg(bufA, H, 1, P + L.W2[k], H, 1, RPNN_H), nullptr,
+        float* da = inner();
+        st = gemm(&c, M, nullptr, RPNN_H, seg(A, H, 1, P + L.W2[k], H, 1, RPNN_H), nullptr,
                   epi(da, H, nullptr, 0, nullptr, 0, f1, H), s);
-        if (st) return st;
         // dV = da1^T z^k; db1 = colsum(da1)
-        st = gemm(&c, RPNN_H, nullptr, nd.din, seg(da, 1, H, desc + k * nd.stride, ZS, 1, M), nullptr,
-                  epi(dP + L.V[k], nd.din), s);
+        if (!st) st = wgrad(da, desc + k * nd.stride, ZS, nd.din, dP + L.V[k]);
+        if (!st) st = bgrad(da, dP + L.b1[k]);
         if (st) return st;
-        launch_colsum(da, M, RPNN_H, H, dP + L.b1[k], s);
-        RPNN_CHECK_LAUNCH();
         if (k > 0) {
             const float* oprev = slot(k - 1);
-            st = gemm(&c, RPNN_H, nullptr, RPNN_H, seg(da, 1, H, oprev, H, 1, M), nullptr, epi(dP + L.W1[k], H), s);
+            st = wgrad(da, oprev, H, RPNN_H, dP + L.W1[k]);
             if (st) return st;
             // dpre_{k-1} = (dpre_k + da1 W1) * (o^{k-1} > 0)
+            float* B = pre();
             st = gemm(&c, M, nullptr, RPNN_H, seg(da, H, 1, P + L.W1[k], H, 1, RPNN_H), nullptr,
-                      epi(bufB, H, nullptr, 0, bufA, H, oprev, H), s);
+                      epi(B, H, nullptr, 0, A, H, oprev, H), s);
             if (st) return st;
-            float* tmp = bufA; bufA = bufB; bufB = tmp;
+            A = B;
         }
     }
-    return RPNN_OK;
+    if (!group) return RPNN_OK;
+    k_colsums<<<dim3((RPNN_H + kColsumCols - 1) / kColsumCols, cj.n), dim3(kColsumCols, kColsumRows), 0, s>>>(cj);
+    RPNN_CHECK_LAUNCH();
+    return wgrads(c, wj, s);
 }
 
 rpnn_status mlp_backward_f32(Ctx& c, const float* desc, int64_t q, const float* saved,
