@@ -71,7 +71,8 @@ rpnn_status train_desc(Ctx& c, const void* desc, int dtype, int64_t q, const flo
 
 // Forward with saved activations in the context's training precision (FP32 CUDA cores,
 // or BF16 tensor-core GEMMs with FP32 master weights); the prediction goes to t_out.
-rpnn_status train_forward(Ctx& c, const void* desc, int dtype, const float* d32, int64_t q, cudaStream_t s) {
+rpnn_status train_forward(Ctx& c, const void* desc, int dtype, const float* d32, int64_t q, cudaStream_t s,
+                          const cudaStream_t* side = nullptr) {
     const size_t saved = c.train_precision == RPNN_BF16 ? train_bf16_saved32_floats(q)
                                                         : mlp_saved_floats_per_row() * (size_t)q;
     rpnn_status st = c.t_saved.reserve(saved * sizeof(float));
@@ -81,7 +82,7 @@ rpnn_status train_forward(Ctx& c, const void* desc, int dtype, const float* d32,
         st = c.t_saved16.reserve(train_bf16_saved_elems(q) * 2);
         if (st) return st;
         return mlp_forward_bf16_train(c, desc, dtype, q, c.t_out.as<float>(), c.t_saved.as<float>(),
-                                      c.t_saved16.as<uint16_t>(), s);
+                                      c.t_saved16.as<uint16_t>(), s, side);
     }
     return mlp_forward_f32(c, d32, q, nullptr, c.t_out.as<float>(), c.t_saved.as<float>(), s);
 }
@@ -926,21 +927,22 @@ namespace {
 rpnn_status train_step_body(Ctx& c, const void* desc, int32_t dtype, const float* target, int64_t q,
                             const rpnn_adam_cfg& adam, int64_t step, const float* cc, float* params, float* m,
                             float* v, double* loss, cudaStream_t s) {
-    const float* d32 = nullptr;
-    rpnn_status st = train_desc(c, desc, dtype, q, &d32, s);
-    if (!st) st = train_forward(c, desc, dtype, d32, q, s);
-    if (st) return st;
-    float* dg = c.sample_val.as<float>();
-    st = launch_loss(c, c.t_out.as<float>(), target, (int)q, loss, dg, s);
-    if (st) return st;
     // a captured BF16 step runs the weight gradients on two more streams, beside the
-    // data-gradient chain (a direct step keeps one stream: it may time new GEMM shapes)
+    // data-gradient chain, and what only the backward reads beside the forward (a direct step
+    // keeps one stream: it may time new GEMM shapes)
     const cudaStream_t* side = nullptr;
     cudaStreamCaptureStatus cst = cudaStreamCaptureStatusNone;
     RPNN_CUDA_TRY(cudaStreamIsCapturing(s, &cst));
     if (cst == cudaStreamCaptureStatusActive && c.train_precision == RPNN_BF16 && c.side_stream[1] &&
         (int)c.t_events.size() >= kTrainEvents)
         side = c.side_stream;
+    const float* d32 = nullptr;
+    rpnn_status st = train_desc(c, desc, dtype, q, &d32, s);
+    if (!st) st = train_forward(c, desc, dtype, d32, q, s, side);
+    if (st) return st;
+    float* dg = c.sample_val.as<float>();
+    st = launch_loss(c, c.t_out.as<float>(), target, (int)q, loss, dg, s);
+    if (st) return st;
     st = train_backward(c, d32, q, dg, c.t_grad.as<float>(), s, side);
     // a direct step sizes the second weight-gradient stream's split-K workspace like the
     // tuner's, so that a later capture allocates nothing

@@ -115,6 +115,36 @@ k_tc_gemm(const __grid_constant__ CUtensorMap a0, const __grid_constant__ CUtens
     tc::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
+    // The epilogue's residual and mask do not depend on the MMAs: tiles of up to 64 columns load
+    // them first, all at once, so that they arrive while the operands do (loaded after the MMAs,
+    // one chunk of 16 columns after the other, they cost a step of 4,096 rows 26 us on its chain of
+    // 21 data gradients: 635 -> 609 us)
+    const int row0 = m0 + warp * 32, row = row0 + lane;
+    constexpr bool EARLY = BN <= 64;
+    constexpr int NC = EARLY ? BN / 16 : 1;
+    float er[NC][16], em[NC][16];
+    if (EARLY && g.splits == 1) {
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+            if (g.e.res) {
+#pragma unroll
+                for (int it = 0; it < 16; ++it) {
+                    const int m = row0 + 2 * it + (lane >> 4), n = n0 + 16 * c + (lane & 15);
+                    er[c][it] = m < g.M && n < g.N ? g.e.res[(int64_t)m * g.e.ldr + n] : 0.0f;
+                }
+            }
+            if (g.e.mask) {
+#pragma unroll
+                for (int it = 0; it < 16; ++it) {
+                    // transposed masks: column 16 c + it of this lane's row
+                    const int m = g.e.mask_t ? row : row0 + 2 * it + (lane >> 4);
+                    const int n = n0 + 16 * c + (g.e.mask_t ? it : lane & 15);
+                    em[c][it] = m < g.M && n < g.N ? g.e.mask[g.e.mask_t ? (int64_t)n * g.e.ldm + m : (int64_t)m * g.e.ldm + n] : 1.0f;
+                }
+            }
+        }
+    }
+
     if (nst > 0) {
         if (threadIdx.x == 0) {                              // producer
             for (int it = 0; it < nst; ++it) {
@@ -165,9 +195,11 @@ k_tc_gemm(const __grid_constant__ CUtensorMap a0, const __grid_constant__ CUtens
     // transposed mask into a second tile the same way.
     float* stile = reinterpret_cast<float*>(sbase) + warp * (32 * 17);
     float* mtile = reinterpret_cast<float*>(sbase) + (4 + warp) * (32 * 17);
-    const int row0 = m0 + warp * 32, row = row0 + lane;
     const uint32_t trow = tmem + ((uint32_t)(warp * 32) << 16);
-    for (int c0 = 0; c0 < BN && n0 + c0 < g.N; c0 += 16) {
+#pragma unroll(EARLY ? NC : 1)
+    for (int c0 = 0; c0 < BN; c0 += 16) {
+        if (n0 + c0 >= g.N) break;
+        const int ec = EARLY ? c0 / 16 : 0;
         float v[16];
         if (nst > 0) {
             tc::tmem_ld16(trow + (uint32_t)c0, v);
@@ -181,7 +213,8 @@ k_tc_gemm(const __grid_constant__ CUtensorMap a0, const __grid_constant__ CUtens
 #pragma unroll
             for (int jj = 0; jj < 16; ++jj) {
                 const int n = n0 + c0 + jj;
-                mtile[lane * 17 + jj] = (row < g.M && n < g.N) ? g.e.mask[(int64_t)n * g.e.ldm + row] : 1.0f;
+                mtile[lane * 17 + jj] = EARLY ? em[ec][jj]
+                                              : ((row < g.M && n < g.N) ? g.e.mask[(int64_t)n * g.e.ldm + row] : 1.0f);
             }
         }
         __syncwarp();
@@ -201,9 +234,9 @@ k_tc_gemm(const __grid_constant__ CUtensorMap a0, const __grid_constant__ CUtens
             for (int it = 0; it < 16; ++it) {
                 const int m = row0 + 2 * it + (lane >> 4);
                 const bool in = m < g.M && ncol;
-                rv[it] = (g.e.res && in) ? g.e.res[(int64_t)m * g.e.ldr + n] : 0.0f;
+                rv[it] = (g.e.res && in) ? (EARLY ? er[ec][it] : g.e.res[(int64_t)m * g.e.ldr + n]) : 0.0f;
                 mv[it] = (g.e.mask && in) ? (g.e.mask_t ? mtile[(2 * it + (lane >> 4)) * 17 + j]
-                                                        : g.e.mask[(int64_t)m * g.e.ldm + n])
+                                                        : (EARLY ? em[ec][it] : g.e.mask[(int64_t)m * g.e.ldm + n]))
                                           : 1.0f;
             }
 #pragma unroll

@@ -204,7 +204,7 @@ struct TrainGraph {
     DevBuf desc, target, adam;        // staged minibatch, {c1, c2} of Adam's bias correction
 };
 
-constexpr int kTrainEvents = 25;   // 22 per-layer gradients, fork, two joins
+constexpr int kTrainEvents = 29;   // 22 per-layer gradients, fork, two joins, preparation fork and its two ends, da3
 
 struct Ctx {
     int device = 0;
@@ -379,10 +379,12 @@ rpnn_status tc_gemm(Ctx& c, int M, int N, const TgSeg& s0, const TgSeg* s1, cons
 
 // FP32 output layer g = relu(T3 t1 + bT3) and its backward (da3 = dout * (g > 0); dT3, dbT3
 // into dP; da2 = (da3 T3) * (t1 > 0)); bias-gradient column sums.  The backward's t1 is
-// [q][200] row-major, or (ldt1 > 0) transposed [200][ldt1].
+// [q][200] row-major, or (ldt1 > 0) transposed [200][ldt1].  ev: the weight and bias gradients
+// run on stream sw once ev, recorded after da3, has completed (null: everything on s).
 rpnn_status mlp_output_layer_f32(Ctx& c, const float* t1, int64_t q, float* out, cudaStream_t s);
 rpnn_status mlp_output_layer_backward_f32(Ctx& c, const float* t1, const float* g, const float* dout, int64_t q,
-                                          float* dP, float* da2, cudaStream_t s, int64_t ldt1 = 0);
+                                          float* dP, float* da2, cudaStream_t s, int64_t ldt1 = 0,
+                                          cudaStream_t sw = nullptr, cudaEvent_t ev = nullptr);
 rpnn_status colsum_f32(Ctx& c, const float* X, int M, int N, float* out, cudaStream_t s);
 
 // Plain ("all-at-once") MLP of the architecture comparison (Sec. 7): n hidden layers of
@@ -401,8 +403,10 @@ size_t train_bf16_saved_elems(int64_t q);
 // slots, then g [q])
 size_t train_bf16_saved32_floats(int64_t q);
 // desc: q rows [10][240] of dtype desc_dtype (RPNN_F32 or RPNN_BF16)
+// side: two more streams (captured steps), the first for what only the backward reads; the
+// backward given the same streams orders itself after it
 rpnn_status mlp_forward_bf16_train(Ctx& c, const void* desc, int desc_dtype, int64_t q, float* out, float* saved,
-                                   uint16_t* s16, cudaStream_t s);
+                                   uint16_t* s16, cudaStream_t s, const cudaStream_t* side = nullptr);
 // exact FP32 widening of n BF16 values
 rpnn_status launch_bf16_to_f32(const void* in, float* out, int64_t n, int sms, cudaStream_t s);
 rpnn_status mlp_backward_bf16_train(Ctx& c, int64_t q, const float* saved, const uint16_t* s16, const float* dout,

@@ -1041,7 +1041,8 @@ rpnn_status mlp_output_layer_f32(Ctx& c, const float* t1, int64_t q, float* out,
 }
 
 rpnn_status mlp_output_layer_backward_f32(Ctx& c, const float* t1, const float* g, const float* dout, int64_t q,
-                                          float* dP, float* da2, cudaStream_t s, int64_t ldt1) {
+                                          float* dP, float* da2, cudaStream_t s, int64_t ldt1, cudaStream_t sw,
+                                          cudaEvent_t ev) {
     // t1 = o^12: [q][200] row-major, or (ldt1 > 0) transposed [200][ldt1]
     const int64_t rs = ldt1 > 0 ? 1 : RPNN_H, cs = ldt1 > 0 ? ldt1 : 1;
     const ParamLayout& L = param_layout();
@@ -1053,9 +1054,15 @@ rpnn_status mlp_output_layer_backward_f32(Ctx& c, const float* t1, const float* 
     float* da3 = c.t_dg.as<float>();
     k_mask<<<(M + 255) / 256, 256, 0, s>>>(dout, g, M, da3);
     RPNN_CHECK_LAUNCH();
-    st = gemm(&c, 1, nullptr, RPNN_H, seg(da3, 0, 1, t1, rs, cs, M), nullptr, epi(dP + L.T[2], H), s);
+    if (ev) {
+        RPNN_CUDA_TRY(cudaEventRecord(ev, s));
+        RPNN_CUDA_TRY(cudaStreamWaitEvent(sw, ev, 0));
+    } else {
+        sw = s;
+    }
+    st = gemm(&c, 1, nullptr, RPNN_H, seg(da3, 0, 1, t1, rs, cs, M), nullptr, epi(dP + L.T[2], H), sw);
     if (st) return st;
-    launch_colsum(da3, M, 1, 1, dP + L.bT[2], s);
+    launch_colsum(da3, M, 1, 1, dP + L.bT[2], sw);
     RPNN_CHECK_LAUNCH();
     return gemm(&c, M, nullptr, RPNN_H, seg(da3, 1, 1, P + L.T[2], H, 1, 1), nullptr,
                 epi(da2, H, nullptr, 0, nullptr, 0, t1, rs, cs), s);

@@ -203,19 +203,27 @@ rpnn_status train_build_image(Ctx& c, cudaStream_t s) {
 // contiguous bytes per column, then g [q] (train_bf16_saved32_floats(q) floats in `saved`);
 // BF16 copies in `s16` (train_bf16_saved_elems(q)).
 rpnn_status mlp_forward_bf16_train(Ctx& c, const void* desc, int desc_dtype, int64_t q, float* out, float* saved,
-                                   uint16_t* s16, cudaStream_t s) {
+                                   uint16_t* s16, cudaStream_t s, const cudaStream_t* side) {
     const int64_t ldq = train_ldq(q);
-    // the transposed weight image the backward reads
-    rpnn_status st = train_build_image(c, s);
+    // The transposed weight image and descriptors are read by the backward only: beside the
+    // forward, whose q / 128 blocks leave most of the chip idle, where there are streams for it
+    // (a captured step; FP32 records are converted for the forward in the same launch).
+    const cudaStream_t sp = side ? side[0] : s;
+    if (side) {
+        RPNN_CUDA_TRY(cudaEventRecord(c.t_events[25], s));
+        RPNN_CUDA_TRY(cudaStreamWaitEvent(sp, c.t_events[25], 0));
+    }
+    rpnn_status st = train_build_image(c, sp);
     if (st) return st;
+    if (side) RPNN_CUDA_TRY(cudaEventRecord(c.t_events[26], sp));
     uint16_t* zb = s16 + (size_t)22 * q * H + (size_t)22 * H * ldq;
     uint16_t* zt = zb + (size_t)q * RPNN_K * RPNN_DESC_STRIDE;
     const dim3 tgrid((unsigned)((q + 31) / 32), (RPNN_K * RPNN_DIN + 31) / 32);
     // BF16 records are the forward's operand as they are; FP32 ones are rounded into zb
     const void* zfwd = desc;
     if (desc_dtype == RPNN_BF16) {
-        k_train_desc<<<tgrid, dim3(32, 8), 0, s>>>(static_cast<const __nv_bfloat16*>(desc), q, ldq, nullptr,
-                                                  reinterpret_cast<__nv_bfloat16*>(zt));
+        k_train_desc<<<tgrid, dim3(32, 8), 0, sp>>>(static_cast<const __nv_bfloat16*>(desc), q, ldq, nullptr,
+                                                   reinterpret_cast<__nv_bfloat16*>(zt));
     } else {
         k_train_desc<<<tgrid, dim3(32, 8), 0, s>>>(static_cast<const float*>(desc), q, ldq,
                                                   reinterpret_cast<__nv_bfloat16*>(zb),
@@ -223,6 +231,7 @@ rpnn_status mlp_forward_bf16_train(Ctx& c, const void* desc, int desc_dtype, int
         zfwd = zb;
     }
     RPNN_CHECK_LAUNCH();
+    if (side) RPNN_CUDA_TRY(cudaEventRecord(c.t_events[27], sp));
     // the 22 layers in the persistent tensor-core network kernel (one 128-row tile per CTA,
     // layer after layer in shared and tensor memory), in its training form: FP32 biases in
     // the epilogue, every ReLU output stored FP32 and BF16 transposed for the backward
@@ -252,7 +261,7 @@ rpnn_status mlp_backward_bf16_train(Ctx& c, int64_t q, const float* saved, const
     rpnn_status st = c.t_gb32.reserve((size_t)NG * q * H * sizeof(float));
     if (!st) st = c.t_gb16.reserve((size_t)NG * per16 * 2);
     if (st) return st;
-    static_assert(NG + 3 <= kTrainEvents, "gradient-ready events");
+    static_assert(NG + 7 <= kTrainEvents, "gradient-ready, fork, join and preparation events");
     if (side && (int)c.t_events.size() < kTrainEvents) { set_error("weight-gradient stream events missing"); return RPNN_ERR_STATE; }
     struct Buf { float* f; uint16_t* b; uint16_t* t; int id; };
     auto buf = [&](int i) {
@@ -288,11 +297,16 @@ rpnn_status mlp_backward_bf16_train(Ctx& c, int64_t q, const float* saved, const
         RPNN_CUDA_TRY(cudaEventRecord(c.t_events[NG], s));
         RPNN_CUDA_TRY(cudaStreamWaitEvent(ws[0], c.t_events[NG], 0));
         RPNN_CUDA_TRY(cudaStreamWaitEvent(ws[1], c.t_events[NG], 0));
+        // the forward's preparation on side[0]: the weight image for the data gradients, the
+        // transposed descriptors for the V gradients
+        RPNN_CUDA_TRY(cudaStreamWaitEvent(s, c.t_events[26], 0));
+        RPNN_CUDA_TRY(cudaStreamWaitEvent(ws[1], c.t_events[27], 0));
     }
     int next = 0;
     Buf A = buf(next++);
     // output layer (CUDA cores): A.f = dl/d(pre-activation of o^12 ... ) masked, dT3, dbT3
-    st = mlp_output_layer_backward_f32(c, slot(21), saved + (size_t)22 * H * ldq, dout, q, dP, A.f, s, ldq);
+    st = mlp_output_layer_backward_f32(c, slot(21), saved + (size_t)22 * H * ldq, dout, q, dP, A.f, s, ldq, ws[0],
+                                       side ? c.t_events[28] : nullptr);
     if (st) return st;
     k_train_act<<<dim3((unsigned)((q + 31) / 32), (H + 31) / 32), dim3(32, 8), 0, s>>>(
         A.f, q, ldq, reinterpret_cast<__nv_bfloat16*>(A.b), reinterpret_cast<__nv_bfloat16*>(A.t));
