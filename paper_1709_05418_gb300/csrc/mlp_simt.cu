@@ -329,7 +329,7 @@ k_gemm(int M_host, const int* __restrict__ M_dev, int N, const __grid_constant__
 
 // Weight gradients of many layers in one launch, C_j = A_j^T B_j with A_j [K][M] and B_j [K][N_j]
 // (rows pitch M and ldb): block z takes run z % splits of job z / splits.  One layer's gradient
-// (200 x 200 outputs) is 28 blocks or fewer; all 32 fill the chip without a split of K.
+// (200 x 200 outputs) is 28 blocks or fewer; all 31 fill the chip.
 constexpr int kMaxWJobs = 40;
 struct WJob {
     const float *A, *B;
@@ -600,13 +600,16 @@ rpnn_status tune(Ctx& c, const GemmKey& key, int M, const int* M_dev, int N, con
         const TileShape& ts = kTiles[t];
         if (t > 0 && ts.bm > 2 * M) continue;
         const int64_t blocks = (int64_t)((N + ts.bn - 1) / ts.bn) * ((M + ts.bm - 1) / ts.bm);
-        for (int sp : kSplits) {
-            if (sp > 1 && (ksteps16 * 16 < kMinSplitK || blocks >= c.num_sms || blocks * sp > (int64_t)c.num_sms * 8 ||
-                           (ksteps16 * 16 / ts.bk) / sp < 4))
-                continue;
-            cands.push_back({t, sp});
-            if (sp > maxsplit) maxsplit = sp;
-        }
+        // of the admissible splits the largest: the shortest runs have the smallest rounding error,
+        // and the bits do not depend on which of several equally fast splits a timing favours
+        int best_sp = 1;
+        for (int sp : kSplits)
+            if (ksteps16 * 16 >= kMinSplitK && blocks < c.num_sms && blocks * sp <= (int64_t)c.num_sms * 8 &&
+                (ksteps16 * 16 / ts.bk) / sp >= 4)
+                best_sp = std::max(best_sp, sp);
+        cands.push_back({t, best_sp});
+        if (t == 0 && best_sp > 1) cands.push_back({0, 1});      // the default's time, for the table
+        maxsplit = std::max(maxsplit, best_sp);
     }
     rpnn_status st = tu.scratch.reserve((size_t)M * N * sizeof(float));
     if (!st && maxsplit > 1) st = tu.ws.reserve((size_t)maxsplit * M * N * sizeof(float));
@@ -709,12 +712,13 @@ rpnn_status wgrads(Ctx& c, WJobs& J, cudaStream_t s) {
             int maxsplit = 1;
             for (int t = 0; t < kNumTiles; ++t) {
                 const TileShape& ts = kTiles[t];
-                const int64_t blocks = (int64_t)((nmax + ts.bn - 1) / ts.bn) * ((J.M + ts.bm - 1) / ts.bm) * J.n;
-                for (int sp : kSplits) {
-                    if (sp > 1 && (J.K < kMinSplitK || blocks >= 4 * c.num_sms || J.K / ts.bk / sp < 4)) continue;
-                    cands.push_back({t, sp});
-                    maxsplit = std::max(maxsplit, sp);
-                }
+                // a sum over K rows in as many runs as one such GEMM takes: the launch is full without,
+                // but the runs' lengths set the sums' rounding
+                int sp = 1;
+                for (int x : kSplits)
+                    if (J.K >= kMinSplitK && (J.K + 15) / 16 * 16 / ts.bk / x >= 4) sp = x;
+                cands.push_back({t, sp});
+                maxsplit = std::max(maxsplit, sp);
             }
             const int64_t out_job = (int64_t)J.M * nmax;
             rpnn_status st = tu.scratch.reserve((size_t)out_job * J.n * sizeof(float));
@@ -743,7 +747,7 @@ rpnn_status wgrads(Ctx& c, WJobs& J, cudaStream_t s) {
                 float ms = 0.0f;
                 RPNN_CUDA_TRY(cudaEventElapsedTime(&ms, tu.ev0, tu.ev1));
                 const float us = ms * 1000.0f / 3.0f / J.n;
-                if (cd.t == 0 && cd.sp == 1) best.default_us = us;
+                if (cd.t == 0) best.default_us = us;                // the default tile, with its runs
                 if (us < best.us) { best.us = us; best.tile = cd.t; best.splits = cd.sp; }
             }
             tu.table.emplace_back(key, best);
