@@ -650,7 +650,8 @@ rpnn_status tune(Ctx& c, const GemmKey& key, int M, const int* M_dev, int N, con
 rpnn_status gemm(Ctx* c, int M, const int* M_dev, int N, const Seg& s0, const Seg* s1, const Epi& e,
                  cudaStream_t s) {
     if (M <= 0 || N <= 0) return RPNN_OK;
-    if (N == 1 && !s1) {
+    // (a sum over many rows keeps the tiled kernel, which may split it)
+    if (N == 1 && !s1 && s0.sak == 1) {
         k_rowdot<<<(M + kDotRows - 1) / kDotRows, 256, 0, s>>>(M, M_dev, s0, e);
         RPNN_CHECK_LAUNCH();
         return RPNN_OK;

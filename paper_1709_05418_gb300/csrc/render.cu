@@ -121,8 +121,9 @@ k_primary(const VolumeView v_, const RenderArgs a_, int64_t P_, float* __restric
         base = __shfl_sync(0xffffffffu, base, 0);
         if (want) {
             const int slot = base + __popc(mask & ((1u << lane) - 1u));
-            qx[3 * slot] = x.x; qx[3 * slot + 1] = x.y; qx[3 * slot + 2] = x.z;
-            qd[3 * slot] = d.x; qd[3 * slot + 1] = d.y; qd[3 * slot + 2] = d.z;
+            const int64_t o = 3 * (int64_t)slot;
+            qx[o] = x.x; qx[o + 1] = x.y; qx[o + 2] = x.z;
+            qd[o] = d.x; qd[o + 1] = d.y; qd[o + 2] = d.z;
             qps[slot] = (uint32_t)ps;
         }
     }
@@ -261,14 +262,16 @@ struct RenderPaths {
         const int lane = threadIdx.x & 31;
         const bool take = want && lane < lanes;
         const unsigned m = __ballot_sync(0xffffffffu, take);
-        int base = 0;
-        if (m && lane == __ffs(m) - 1) base = atomicAdd(next, __popc(m));
+        // (unsigned: the lanes that find no path left count on beyond total)
+        unsigned base = 0;
+        if (m && lane == __ffs(m) - 1) base = (unsigned)atomicAdd(next, __popc(m));
         base = __shfl_sync(0xffffffffu, base, m ? __ffs(m) - 1 : 0);
-        const int i = base + __popc(m & ((1u << lane) - 1u));
-        if (!take || i >= total) return -1;
+        const unsigned i = base + __popc(m & ((1u << lane) - 1u));
+        if (!take || i >= (unsigned)total) return -1;
         ps = qps[i];
-        x = f3(qx[3 * i], qx[3 * i + 1], qx[3 * i + 2]);
-        d = f3(qd[3 * i], qd[3 * i + 1], qd[3 * i + 2]);
+        const int64_t o = 3 * (int64_t)i;
+        x = f3(qx[o], qx[o + 1], qx[o + 2]);
+        d = f3(qd[o], qd[o + 1], qd[o + 2]);
         rng = make_rng(a.seed, ps / (uint32_t)a.spp, ps % (uint32_t)a.spp, kDomPath);
         return 1;
     }
@@ -413,11 +416,14 @@ struct LabelPaths {
         int first = 0;
         if (m && lane == __ffs(m) - 1) first = atomicAdd(&r.next, __popc(m));
         first = __shfl_sync(0xffffffffu, first, m ? __ffs(m) - 1 : 0);
-        if (claim) j = first + __popc(m & ((1u << lane) - 1u));
+        if (claim) {
+            j = first + __popc(m & ((1u << lane) - 1u));
+            if (j < 0) j = 0x7fffffff;             // beyond the last path index
+        }
         if (!want || j >= n_max) return -1;
         const int base = vr.base;
         __threadfence_block();
-        if (j >= base + kRing) return 0;
+        if (j - base >= kRing) return 0;
         x = x0; d = d0;
         rng = make_rng(seed, rec, (uint32_t)j, kDomLabel);
         return 1;
