@@ -546,9 +546,11 @@ rpnn_status launch_primary(Ctx& c, const VolumeView& vv, const rpnn_render_desc&
                            float* sample_val, float* qx, float* qd, uint32_t* qps, int* qcount,
                            int* hit, float* xo, float* dout, float* Ld, cudaStream_t s) {
     const int64_t P = (int64_t)rd.width * rd.height * rd.spp;
-    // as many samples per warp as give every resident warp (24 per SM) some, two at least
+    // as many samples per warp as give 20 warps per SM some (24 fit), two at least; above 48,640
+    // samples the issue rate counts, not the latency (BF16 renders of a 224^3 cloud: 128 x 128
+    // samples 260 us with 32 per warp, 236 with 8; 208 x 208: 390, with 16 375; 240 x 240: 409, with 16 418)
     int lanes = 2;
-    while (lanes < 32 && (int64_t)lanes * c.num_sms * 24 < P) lanes *= 2;
+    while (lanes < 32 && (int64_t)lanes * c.num_sms * 20 < P) lanes *= 2;
     const int64_t blocks = (P + 4 * lanes - 1) / (4 * lanes);
     k_primary<false><<<(unsigned)blocks, 128, 0, s>>>(vv, make_args(rd), P, sample_val, qx, qd, qps, qcount,
                                                       hit, xo, dout, Ld, c.status.as<uint32_t>(), nullptr, 0, lanes);
