@@ -51,6 +51,7 @@ struct TgEpiDev {
 struct TgArgs {
     int M, N, K0, K1;                     // K1 = 0: one segment
     int splits;
+    int vec;                              // the epilogue's rows are 16-byte aligned, N is a multiple of 8
     float* ws;                            // [splits][M][N] partial sums when splits > 1
     TgEpiDev e;
     uint32_t* status;
@@ -61,20 +62,20 @@ struct TgCfg {
     static constexpr uint32_t BBOX = BN * 64;
     static constexpr uint32_t STAGE = 2 * ABOX + 2 * BBOX;
     static constexpr int STAGES = BN == 256 ? 3 : 4;
-    static_assert(2 * 4 * 32 * 17 * 4 <= STAGES * STAGE, "epilogue tiles reuse the stage ring");
+    static_assert(4 * 32 * 17 * 4 <= STAGES * STAGE, "epilogue tiles reuse the stage ring");
     static constexpr uint32_t OFF_BAR = STAGES * STAGE;
     static constexpr uint32_t SMEM = OFF_BAR + 256 + 1024;   // barriers, TMEM slot, alignment slack
 };
 
-__device__ __forceinline__ void tg_store(const TgEpiDev& e, int m, int n, float v) {
+// everything but the transposed copy; returns the stored value
+__device__ __forceinline__ float tg_store(const TgEpiDev& e, int m, int n, float v) {
     if (e.bias) v += e.bias[n];
     if (e.res) v += e.res[(int64_t)m * e.ldr + n];
     if (e.relu) v = fmaxf(v, 0.0f);
     if (e.mask && !(e.mask[e.mask_t ? (int64_t)n * e.ldm + m : (int64_t)m * e.ldm + n] > 0.0f)) v = 0.0f;
     if (e.C) e.C[(int64_t)m * e.ldc + n] = v;
-    const __nv_bfloat16 b = __float2bfloat16_rn(v);
-    if (e.Cb) e.Cb[(int64_t)m * e.ldb + n] = b;
-    if (e.Ct) e.Ct[(int64_t)n * e.ldt + m] = b;
+    if (e.Cb) e.Cb[(int64_t)m * e.ldb + n] = __float2bfloat16_rn(v);
+    return v;
 }
 
 template <int BN>
@@ -97,6 +98,22 @@ k_tc_gemm(const __grid_constant__ CUtensorMap a0, const __grid_constant__ CUtens
     const int tb = (int)blockIdx.z * per;
     const int nst = max(0, min(T, tb + per) - tb);
 
+    // operand tiles of stage `it` of this block's K run (thread 0)
+    auto load_stage = [&](int it) {
+        const int t = tb + it;
+        const bool first = t < T0;
+        const void* am = first ? static_cast<const void*>(&a0) : static_cast<const void*>(&a1);
+        const void* bm = first ? static_cast<const void*>(&b0) : static_cast<const void*>(&b1);
+        const int k0 = (first ? t : t - T0) * KST;
+        const uint32_t st = base + (uint32_t)(it % C::STAGES) * C::STAGE;
+        const uint32_t fb = bar + 8u * (it % C::STAGES);
+        tc::mbar_expect_tx(fb, C::STAGE);
+        tc::tma_load_2d(st, am, k0, m0, fb);
+        tc::tma_load_2d(st + ABOX, am, k0 + 32, m0, fb);
+        tc::tma_load_2d(st + 2 * ABOX, bm, k0, n0, fb);
+        tc::tma_load_2d(st + 2 * ABOX + C::BBOX, bm, k0 + 32, n0, fb);
+    };
+    // the first stages are on their way before anything else is set up
     if (threadIdx.x == 0) {
         for (int s = 0; s < C::STAGES; ++s) {
             tc::mbar_init(bar + 8u * s, 1);
@@ -105,65 +122,53 @@ k_tc_gemm(const __grid_constant__ CUtensorMap a0, const __grid_constant__ CUtens
         tc::mbar_init(done, 1);
         *abort_flag = 0;
         tc::fence_mbar_init();
+        for (int it = 0; it < min(nst, C::STAGES); ++it) load_stage(it);
     }
-    if (warp == 0) {
+    if (warp == 2) {
         tc::tmem_alloc(tc::smem_u32(tmem_slot), BN);
         tc::tmem_relinquish();
+    }
+    // The epilogue's residual and mask do not depend on the MMAs: tiles of up to 64 columns load
+    // them first, all at once, so that they arrive while the operands do (loaded after the MMAs,
+    // one chunk of 16 columns after the other, they cost a step of 4,096 rows 26 us on its chain of
+    // 21 data gradients)
+    const int row0 = m0 + warp * 32, row = row0 + lane;
+    constexpr bool EARLY = BN <= 64;
+    constexpr int NC = EARLY ? BN / 16 : 1;
+    float er[NC][16], em[NC][16];
+    // this lane's row of the 16 columns from n on (vec: 8 or 16 of them exist)
+    auto row16 = [&](const float* p, float (&r)[16], int n) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            if (n + 4 * q >= g.N || row >= g.M) continue;
+            const float4 t = *reinterpret_cast<const float4*>(p + 4 * q);
+            r[4 * q] = t.x; r[4 * q + 1] = t.y; r[4 * q + 2] = t.z; r[4 * q + 3] = t.w;
+        }
+    };
+    auto operands = [&](int n, float (&r)[16], float (&k)[16]) {
+        if (g.e.res) row16(g.e.res + (int64_t)row * g.e.ldr + n, r, n);
+        if (g.e.mask && !g.e.mask_t) row16(g.e.mask + (int64_t)row * g.e.ldm + n, k, n);
+        if (g.e.mask && g.e.mask_t) {
+            const float* p = g.e.mask + (int64_t)n * g.e.ldm + row;
+#pragma unroll
+            for (int jj = 0; jj < 16; ++jj)
+                if (n + jj < g.N && row < g.M) k[jj] = p[jj * g.e.ldm];
+        }
+    };
+    if (EARLY && g.vec) {
+#pragma unroll
+        for (int c = 0; c < NC; ++c) operands(n0 + 16 * c, er[c], em[c]);
     }
     tc::tc_fence_before();
     __syncthreads();
     tc::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
-    // The epilogue's residual and mask do not depend on the MMAs: tiles of up to 64 columns load
-    // them first, all at once, so that they arrive while the operands do (loaded after the MMAs,
-    // one chunk of 16 columns after the other, they cost a step of 4,096 rows 26 us on its chain of
-    // 21 data gradients: 635 -> 609 us)
-    const int row0 = m0 + warp * 32, row = row0 + lane;
-    constexpr bool EARLY = BN <= 64;
-    constexpr int NC = EARLY ? BN / 16 : 1;
-    float er[NC][16], em[NC][16];
-    if (EARLY && g.splits == 1) {
-#pragma unroll
-        for (int c = 0; c < NC; ++c) {
-            if (g.e.res) {
-#pragma unroll
-                for (int it = 0; it < 16; ++it) {
-                    const int m = row0 + 2 * it + (lane >> 4), n = n0 + 16 * c + (lane & 15);
-                    er[c][it] = m < g.M && n < g.N ? g.e.res[(int64_t)m * g.e.ldr + n] : 0.0f;
-                }
-            }
-            if (g.e.mask) {
-#pragma unroll
-                for (int it = 0; it < 16; ++it) {
-                    // transposed masks: column 16 c + it of this lane's row
-                    const int m = g.e.mask_t ? row : row0 + 2 * it + (lane >> 4);
-                    const int n = n0 + 16 * c + (g.e.mask_t ? it : lane & 15);
-                    em[c][it] = m < g.M && n < g.N ? g.e.mask[g.e.mask_t ? (int64_t)n * g.e.ldm + m : (int64_t)m * g.e.ldm + n] : 1.0f;
-                }
-            }
-        }
-    }
-
     if (nst > 0) {
         if (threadIdx.x == 0) {                              // producer
-            for (int it = 0; it < nst; ++it) {
-                const int s = it % C::STAGES;
-                if (it >= C::STAGES &&
-                    !tc::mbar_wait(bar + 8u * (C::STAGES + s), ((it / C::STAGES) - 1) & 1, abort_flag))
-                    break;
-                const int t = tb + it;
-                const bool first = t < T0;
-                const void* am = first ? static_cast<const void*>(&a0) : static_cast<const void*>(&a1);
-                const void* bm = first ? static_cast<const void*>(&b0) : static_cast<const void*>(&b1);
-                const int k0 = (first ? t : t - T0) * KST;
-                const uint32_t st = base + (uint32_t)s * C::STAGE;
-                const uint32_t fb = bar + 8u * s;
-                tc::mbar_expect_tx(fb, C::STAGE);
-                tc::tma_load_2d(st, am, k0, m0, fb);
-                tc::tma_load_2d(st + ABOX, am, k0 + 32, m0, fb);
-                tc::tma_load_2d(st + 2 * ABOX, bm, k0, n0, fb);
-                tc::tma_load_2d(st + 2 * ABOX + C::BBOX, bm, k0 + 32, n0, fb);
+            for (int it = C::STAGES; it < nst; ++it) {
+                if (!tc::mbar_wait(bar + 8u * (C::STAGES + it % C::STAGES), ((it / C::STAGES) - 1) & 1, abort_flag)) break;
+                load_stage(it);
             }
         } else if (threadIdx.x == 32) {                      // MMA issuer
             const uint32_t idesc = tc::idesc_bf16(TGM, BN);
@@ -187,85 +192,106 @@ k_tc_gemm(const __grid_constant__ CUtensorMap a0, const __grid_constant__ CUtens
         tc::tc_fence_after();
     }
 
-    // epilogue: warp w owns accumulator lanes (tile rows) 32 w .. 32 w + 31.  Each 32 x 16
-    // chunk goes through a per-warp shared tile (the stage ring is idle once the MMAs are
-    // done): a row-major pass (half a warp per row, 16 consecutive columns) applies bias,
-    // residual, ReLU and mask and makes the FP32 / BF16 / split-K stores coalesced; a
-    // column pass (one lane per row) makes the transposed BF16 store coalesced, and reads a
-    // transposed mask into a second tile the same way.
-    float* stile = reinterpret_cast<float*>(sbase) + warp * (32 * 17);
-    float* mtile = reinterpret_cast<float*>(sbase) + (4 + warp) * (32 * 17);
+    // epilogue: warp w owns accumulator lanes (tile rows) 32 w .. 32 w + 31, a lane one row, 16
+    // columns at a time.  Aligned rows go straight from registers: 16-byte loads and stores per
+    // lane, and transposed stores (masks) of 32 consecutive rows per warp.  Bound: latency; the
+    // code runs once per block.  Passing every 16 columns through shared memory with each load
+    // and store under its own condition took 6,000-10,000 clocks of a
+    // block's 13,000-19,000; now 2,500-3,800 of 9,000-13,000 (step of 4,096 rows 613 -> 554 us, with the
+    // first stages and the operands requested before the barrier).
     const uint32_t trow = tmem + ((uint32_t)(warp * 32) << 16);
-#pragma unroll(EARLY ? NC : 1)
-    for (int c0 = 0; c0 < BN; c0 += 16) {
-        if (n0 + c0 >= g.N) break;
-        const int ec = EARLY ? c0 / 16 : 0;
-        float v[16];
+    auto chunk = [&](int c0, float (&v)[16]) {
         if (nst > 0) {
             tc::tmem_ld16(trow + (uint32_t)c0, v);
         } else {
 #pragma unroll
             for (int j = 0; j < 16; ++j) v[j] = 0.0f;
         }
+    };
+    if (g.vec) {
+#pragma unroll(EARLY ? NC : 1)
+        for (int c0 = 0; c0 < BN; c0 += 16) {
+            if (n0 + c0 >= g.N) break;
+            const int ec = EARLY ? c0 / 16 : 0;
+            float v[16];
+            chunk(c0, v);
+            if (!EARLY) operands(n0 + c0, er[0], em[0]);
+            if (row < g.M) {
 #pragma unroll
-        for (int j = 0; j < 16; ++j) stile[lane * 17 + j] = v[j];
-        if (g.splits == 1 && g.e.mask && g.e.mask_t) {
+                for (int h = 0; h < 16; h += 8) {
+                    const int n = n0 + c0 + h;
+                    if (n >= g.N) break;
+                    float* x = v + h;
+                    if (g.e.bias) {
 #pragma unroll
-            for (int jj = 0; jj < 16; ++jj) {
-                const int n = n0 + c0 + jj;
-                mtile[lane * 17 + jj] = EARLY ? em[ec][jj]
-                                              : ((row < g.M && n < g.N) ? g.e.mask[(int64_t)n * g.e.ldm + row] : 1.0f);
-            }
-        }
-        __syncwarp();
-        const int j = lane & 15, n = n0 + c0 + j;
-        const bool ncol = n < g.N;
-        if (g.splits > 1) {
+                        for (int j = 0; j < 8; ++j) x[j] += g.e.bias[n + j];
+                    }
+                    if (g.e.res) {
 #pragma unroll
-            for (int it = 0; it < 16; ++it) {
-                const int rr = 2 * it + (lane >> 4), m = row0 + rr;
-                if (m < g.M && ncol) g.ws[((int64_t)blockIdx.z * g.M + m) * g.N + n] = stile[rr * 17 + j];
-            }
-        } else {
-            // all of the chunk's residual and mask loads first (independent, in flight together)
-            float rv[16], mv[16];
-            const float bias = (g.e.bias && ncol) ? g.e.bias[n] : 0.0f;
+                        for (int j = 0; j < 8; ++j) x[j] += er[ec][h + j];
+                    }
+                    if (g.e.relu) {
 #pragma unroll
-            for (int it = 0; it < 16; ++it) {
-                const int m = row0 + 2 * it + (lane >> 4);
-                const bool in = m < g.M && ncol;
-                rv[it] = (g.e.res && in) ? (EARLY ? er[ec][it] : g.e.res[(int64_t)m * g.e.ldr + n]) : 0.0f;
-                mv[it] = (g.e.mask && in) ? (g.e.mask_t ? mtile[(2 * it + (lane >> 4)) * 17 + j]
-                                                        : (EARLY ? em[ec][it] : g.e.mask[(int64_t)m * g.e.ldm + n]))
-                                          : 1.0f;
-            }
+                        for (int j = 0; j < 8; ++j) x[j] = fmaxf(x[j], 0.0f);
+                    }
+                    if (g.e.mask) {
 #pragma unroll
-            for (int it = 0; it < 16; ++it) {
-                const int rr = 2 * it + (lane >> 4), m = row0 + rr;
-                if (m < g.M && ncol) {
-                    float x = stile[rr * 17 + j];
-                    if (g.e.bias) x += bias;
-                    if (g.e.res) x += rv[it];
-                    if (g.e.relu) x = fmaxf(x, 0.0f);
-                    if (g.e.mask && !(mv[it] > 0.0f)) x = 0.0f;
-                    if (g.e.C) g.e.C[(int64_t)m * g.e.ldc + n] = x;
-                    if (g.e.Cb) g.e.Cb[(int64_t)m * g.e.ldb + n] = __float2bfloat16_rn(x);
-                    stile[rr * 17 + j] = x;
+                        for (int j = 0; j < 8; ++j) x[j] = em[ec][h + j] > 0.0f ? x[j] : 0.0f;
+                    }
+                    if (g.e.C) {
+                        float4* c = reinterpret_cast<float4*>(g.e.C + (int64_t)row * g.e.ldc + n);
+                        c[0] = make_float4(x[0], x[1], x[2], x[3]);
+                        c[1] = make_float4(x[4], x[5], x[6], x[7]);
+                    }
+                    __align__(16) __nv_bfloat16 b[8];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) b[j] = __float2bfloat16_rn(x[j]);
+                    if (g.e.Cb) *reinterpret_cast<uint4*>(g.e.Cb + (int64_t)row * g.e.ldb + n) = *reinterpret_cast<const uint4*>(b);
+                    if (g.e.Ct) {
+                        __nv_bfloat16* t = g.e.Ct + (int64_t)n * g.e.ldt + row;
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) t[j * g.e.ldt] = b[j];
+                    }
                 }
             }
-        }
-        if (g.splits == 1 && g.e.Ct) {
             __syncwarp();
-            if (row < g.M) {
-                for (int jj = 0; jj < 16 && n0 + c0 + jj < g.N; ++jj)
-                    g.e.Ct[(int64_t)(n0 + c0 + jj) * g.e.ldt + row] = __float2bfloat16_rn(stile[lane * 17 + jj]);
-            }
         }
-        __syncwarp();
+    } else {
+        // partial sums and unaligned rows: each 32 x 16 chunk through a per-warp shared tile (the
+        // stage ring is idle once the MMAs are done), half a warp per row, then a lane per row for the
+        // transposed store
+        float* stile = reinterpret_cast<float*>(sbase) + warp * (32 * 17);
+        for (int c0 = 0; c0 < BN; c0 += 16) {
+            if (n0 + c0 >= g.N) break;
+            float v[16];
+            chunk(c0, v);
+#pragma unroll
+            for (int j = 0; j < 16; ++j) stile[lane * 17 + j] = v[j];
+            __syncwarp();
+            const int j = lane & 15, n = n0 + c0 + j;
+            if (g.splits > 1) {
+#pragma unroll 8
+                for (int it = 0; it < 16; ++it) {
+                    const int rr = 2 * it + (lane >> 4), m = row0 + rr;
+                    if (m < g.M && n < g.N) g.ws[((int64_t)blockIdx.z * g.M + m) * g.N + n] = stile[rr * 17 + j];
+                }
+            } else {
+#pragma unroll 4
+                for (int it = 0; it < 16; ++it) {
+                    const int rr = 2 * it + (lane >> 4), m = row0 + rr;
+                    if (m < g.M && n < g.N) stile[rr * 17 + j] = tg_store(g.e, m, n, stile[rr * 17 + j]);
+                }
+                __syncwarp();
+                if (g.e.Ct && row < g.M)
+                    for (int jj = 0; jj < 16 && n0 + c0 + jj < g.N; ++jj)
+                        g.e.Ct[(int64_t)(n0 + c0 + jj) * g.e.ldt + row] = __float2bfloat16_rn(stile[lane * 17 + jj]);
+            }
+            __syncwarp();
+        }
     }
     tc::tc_fence_before();
     __syncthreads();
-    if (warp == 0) tc::tmem_dealloc(tmem, BN);
+    if (warp == 2) tc::tmem_dealloc(tmem, BN);
     if (threadIdx.x == 0 && *abort_flag) atomicOr(g.status, kStatTimeout);
 }
 
@@ -276,7 +302,8 @@ __global__ void k_tg_splitk(const float* __restrict__ ws, int splits, int M, int
         const int m = (int)(i / N), n = (int)(i % N);
         float v = 0.0f;
         for (int z = 0; z < splits; ++z) v += ws[((int64_t)z * M + m) * N + n];
-        tg_store(e, m, n, v);
+        v = tg_store(e, m, n, v);
+        if (e.Ct) e.Ct[(int64_t)n * e.ldt + m] = __float2bfloat16_rn(v);
     }
 }
 
@@ -338,9 +365,10 @@ rpnn_status launch_bn(const CUtensorMap* maps, const TgArgs& a, cudaStream_t s) 
     return RPNN_OK;
 }
 
-// One launch (plus the split-K reduction) with tile width bn and `splits` K runs.
+// One launch (plus the split-K reduction) with tile width bn and `splits` K runs; `reps` of them for
+// the tuner.
 rpnn_status launch_tg(Ctx& c, int bn, int splits, int M, int N, const TgSeg& s0, const TgSeg* s1,
-                      const TgEpiDev& e, float* ws, cudaStream_t s) {
+                      const TgEpiDev& e, float* ws, cudaStream_t s, int reps = 1) {
     if ((M + TGM - 1) / TGM > 65535) { set_error("BF16 GEMM with %d rows exceeds the grid limit", M); return RPNN_ERR_ARG; }
     CUtensorMap maps[4];
     rpnn_status st = make_map(c, &maps[0], s0.A, s0.lda, s0.K, M, TGM);
@@ -352,19 +380,28 @@ rpnn_status launch_tg(Ctx& c, int bn, int splits, int M, int N, const TgSeg& s0,
     TgArgs a;
     a.M = M; a.N = N; a.K0 = s0.K; a.K1 = s1 ? s1->K : 0;
     a.splits = splits; a.ws = ws; a.e = e; a.status = c.status.as<uint32_t>();
-    switch (bn) {
-        case 32: st = launch_bn<32>(maps, a, s); break;
-        case 64: st = launch_bn<64>(maps, a, s); break;
-        case 128: st = launch_bn<128>(maps, a, s); break;
-        default: st = launch_bn<256>(maps, a, s); break;
-    }
-    if (st) return st;
-    if (splits > 1) {
-        const int64_t total = (int64_t)M * N;
-        int64_t b = (total + 255) / 256;
-        if (b > (int64_t)c.num_sms * 8) b = (int64_t)c.num_sms * 8;
-        k_tg_splitk<<<(unsigned)b, 256, 0, s>>>(ws, splits, M, N, e);
-        RPNN_CHECK_LAUNCH();
+    // the direct epilogue: 16-byte accesses along the rows of what is there (the transposed ones take
+    // any pitch), and whole groups of eight columns
+    auto rows16 = [](const void* p, int64_t ld, size_t el) {
+        return !p || (reinterpret_cast<uintptr_t>(p) % 16 == 0 && (size_t)ld * el % 16 == 0);
+    };
+    a.vec = splits == 1 && N % 8 == 0 && rows16(e.res, e.ldr, 4) && (e.mask_t || rows16(e.mask, e.ldm, 4)) &&
+            rows16(e.C, e.ldc, 4) && rows16(e.Cb, e.ldb, 2);
+    for (int r = 0; r < reps; ++r) {
+        switch (bn) {
+            case 32: st = launch_bn<32>(maps, a, s); break;
+            case 64: st = launch_bn<64>(maps, a, s); break;
+            case 128: st = launch_bn<128>(maps, a, s); break;
+            default: st = launch_bn<256>(maps, a, s); break;
+        }
+        if (st) return st;
+        if (splits > 1) {
+            const int64_t total = (int64_t)M * N;
+            int64_t b = (total + 255) / 256;
+            if (b > (int64_t)c.num_sms * 8) b = (int64_t)c.num_sms * 8;
+            k_tg_splitk<<<(unsigned)b, 256, 0, s>>>(ws, splits, M, N, e);
+            RPNN_CHECK_LAUNCH();
+        }
     }
     return RPNN_OK;
 }
@@ -389,8 +426,8 @@ rpnn_status tc_gemm(Ctx& c, int M, int N, const TgSeg& s0, const TgSeg* s1, cons
             bn = hit->tile;
             splits = hit->splits;
         } else if (cs == cudaStreamCaptureStatusNone) {   // never time under stream capture
-            // time every admissible (tile width, split) on the call's operands, writing the
-            // FP32 result into scratch only
+            // time every admissible (tile width, split) on the call's operands, writing into
+            // scratch only
             struct Cand { int bn, sp; };
             std::vector<Cand> cands;
             int maxsplit = 1;
@@ -406,7 +443,11 @@ rpnn_status tc_gemm(Ctx& c, int M, int N, const TgSeg& s0, const TgSeg* s1, cons
                     maxsplit = std::max(maxsplit, sp);
                 }
             }
-            rpnn_status st = tu.scratch.reserve((size_t)M * N * sizeof(float));
+            // the copies are timed too: they are most of a gradient's epilogue (timed without them, a
+            // 128-wide tile with a third of the blocks came out ahead and cost a step of 4,096 rows up to 45 us)
+            const size_t nc = (size_t)M * N * sizeof(float), nb = e.Cb ? (size_t)M * e.ldb * 2 : 0, nt = e.Ct ? (size_t)N * e.ldt * 2 : 0;
+            auto up16 = [](size_t n) { return (n + 15) / 16 * 16; };
+            rpnn_status st = tu.scratch.reserve(up16(nc) + up16(nb) + nt);
             if (!st && maxsplit > 1) st = tu.ws.reserve((size_t)maxsplit * M * N * sizeof(float));
             if (st) return st;
             if (!tu.ev0) {
@@ -416,22 +457,24 @@ rpnn_status tc_gemm(Ctx& c, int M, int N, const TgSeg& s0, const TgSeg* s1, cons
             TgEpiDev es = e;
             es.C = tu.scratch.as<float>();
             es.ldc = N;
-            es.Cb = nullptr;
-            es.Ct = nullptr;
+            unsigned char* copies = tu.scratch.as<unsigned char>() + up16(nc);
+            if (e.Cb) es.Cb = reinterpret_cast<__nv_bfloat16*>(copies);
+            if (e.Ct) es.Ct = reinterpret_cast<__nv_bfloat16*>(copies + up16(nb));
             GemmChoice best{bn, 1, 1e30f, 0.0f};
             for (const Cand& cd : cands) {
                 st = launch_tg(c, cd.bn, cd.sp, M, N, s0, s1, es, tu.ws.as<float>(), s);
                 if (st) return st;
                 RPNN_CUDA_TRY(cudaEventRecord(tu.ev0, s));
-                for (int r = 0; r < 3; ++r) {
-                    st = launch_tg(c, cd.bn, cd.sp, M, N, s0, s1, es, tu.ws.as<float>(), s);
-                    if (st) return st;
-                }
+                // together: with the host's preparation between them the launches of short kernels took
+                // turns with it, and a 64-wide tile in 16 runs timed like a 32-wide one in 8 (step 580, 550 us)
+                constexpr int kReps = 8;
+                st = launch_tg(c, cd.bn, cd.sp, M, N, s0, s1, es, tu.ws.as<float>(), s, kReps);
+                if (st) return st;
                 RPNN_CUDA_TRY(cudaEventRecord(tu.ev1, s));
                 RPNN_CUDA_TRY(cudaEventSynchronize(tu.ev1));
                 float ms = 0.0f;
                 RPNN_CUDA_TRY(cudaEventElapsedTime(&ms, tu.ev0, tu.ev1));
-                const float us = ms * 1000.0f / 3.0f;
+                const float us = ms * 1000.0f / kReps;
                 if (cd.bn == bn && cd.sp == 1) best.default_us = us;
                 if (us < best.us) { best.us = us; best.tile = cd.bn; best.splits = cd.sp; }
             }
