@@ -927,17 +927,21 @@ rpnn_status rpnn_backward_f32(Ctx& c, const NetDims& nd, const float* P, const f
     const int64_t H = RPNN_H, ZS = (int64_t)RPNN_K * nd.stride;
     auto slot = [&](int i) { return saved + (size_t)i * q * H; };
     const float* g = saved + (size_t)22 * q * H;
-    // Up to kGroupRows rows every layer's gradient is kept and the 32 weight gradients and 22
+    // Up to kGroupRows rows every layer's gradient is kept and the 31 weight gradients and 22
     // bias sums follow the data-gradient chain as one launch each: one layer's cannot fill the
-    // chip (a step of 1,000 rows: 1.41 -> 0.64 ms).  Beyond that a layer's own launches do,
-    // and two buffers instead of 22 are enough.
+    // chip (a step of 1,000 rows: 1.41 -> 0.64 ms).  Beyond that, or where the 22 buffers do not
+    // fit beside what is allocated, a layer's own launches do with three.
     constexpr int64_t kGroupRows = 1 << 17;
-    const bool group = q <= kGroupRows;
+    bool group = q <= std::min(kGroupRows, c.group_rows);
     constexpr int NG = 22;
     rpnn_status st = c.t_dg.reserve((size_t)q * sizeof(float));
-    if (group) {
-        if (!st) st = c.t_gb32.reserve((size_t)NG * q * H * sizeof(float));
-    } else {
+    if (st) return st;
+    if (group && c.t_gb32.reserve((size_t)NG * q * H * sizeof(float)) != RPNN_OK) {
+        cudaGetLastError();
+        c.group_rows = q - 1;             // not tried again (a captured step must not allocate)
+        group = false;
+    }
+    if (!group) {
         if (!st) st = c.act0.reserve((size_t)q * H * sizeof(float));
         if (!st) st = c.act1.reserve((size_t)q * H * sizeof(float));
         if (!st) st = c.act2.reserve((size_t)q * H * sizeof(float));
