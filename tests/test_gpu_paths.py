@@ -1,0 +1,73 @@
+"""The path tracer's scheduling must not show in its results: which lane traces a path, how many
+warps share a record and in which order paths end.  Labels are compared bit for bit between
+calls that give a record's block 1, 2 or 4 warps, at path limits around the rounds of 32 and the
+512 slots kept in flight, and path-traced images with the oracle, from fewer samples than one
+warp has lanes to more than all lanes of the GPU."""
+import numpy as np
+import pytest
+
+from paper_1709_05418_gb300 import workloads as W
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def env():
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import oracle
+    from paper_1709_05418_gb300 import api
+    ctx = api.Context()
+    dens = W.blob_cloud(32, nblobs=6, seed=1)
+    vol = ctx.load_volume(torch.from_numpy(dens).cuda())
+    ctx.build_mips(vol)
+    orc = oracle.Volume(dens)
+    yield api, ctx, vol, dens.shape, orc
+    orc.close()
+    ctx.close()
+
+
+@pytest.mark.parametrize("n_min,n_max,rel_ci", [(1, 1, 1e-7), (5, 31, 1e-7), (1, 33, 1e-7), (32, 511, 0.3),
+                                                 (64, 513, 1e-7), (100, 1100, 0.1)])
+def test_labels_do_not_depend_on_the_warps_of_a_record(env, n_min, n_max, rel_ci):
+    _, ctx, vol, _, orc = env
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    one = [t.cpu() for t in ctx.gen_records(vol, 11, 64 * sms + 5, 77, rel_ci=rel_ci, n_min=n_min, n_max=n_max)]
+    for off, n in ((3, 32 * sms + 1), (64 * sms - 4, 9), (0, 1)):              # two warps, four, four
+        part = [t.cpu() for t in ctx.gen_records(vol, 11 + off, n, 77, rel_ci=rel_ci, n_min=n_min, n_max=n_max)]
+        for a, b in zip(one, part):
+            assert torch.equal(a[off:off + n], b)
+    ctx.sync_status()
+    npaths = one[4][one[3] > 0].numpy()
+    assert npaths.min() >= n_min and npaths.max() <= n_max
+    if rel_ci < 1e-6:
+        if n_max >= 64:                 # fewer paths may agree to the last bit
+            assert np.all(npaths == n_max)
+        # The mean of the oracle's n_max paths: a decision flips on an FP32 rounding about once in
+        # 5,000 paths; two such paths of 10 times the mean move a mean of 513 by 2 x 10 / 513 = 4 %,
+        # and one of the six records may have lost a brighter path.
+        if n_max == 513:
+            ref = [orc.gen_record(77, 11 + i, rel_ci=rel_ci, n_min=n_min, n_max=n_max)["label"] for i in range(6)]
+            assert sum(abs(float(a) - r) <= 0.04 * r + 1e-7 for a, r in zip(one[3], ref)) >= 5
+
+
+@pytest.mark.parametrize("w,h,spp", [(17, 1, 1), (37, 23, 3), (640, 480, 1)])
+def test_path_images_follow_the_oracle(env, w, h, spp):
+    api, ctx, vol, shape, orc = env
+    cam = W.camera(shape, w, h, spp=spp, seed=5, light_seed=6)
+    got = ctx.render(vol, cam, precision=api.F32, mode=api.MODE_PATH).cpu().numpy().ravel().astype(np.float64)
+    again = ctx.render(vol, cam, precision=api.F32, mode=api.MODE_PATH).cpu().numpy().ravel()
+    ctx.sync_status()
+    assert np.array_equal(got, again)
+    pix = np.arange(w * h)
+    if w * h > 2000:
+        pix = np.random.default_rng(1).choice(pix, 2000, replace=False)
+    ref = orc.render_pixels(cam, pix, mode=1)
+    # as the path render at 64 x 64: a path whose decision flips on an FP32 rounding differs
+    tol = 1e-3 * np.maximum(np.abs(ref), 1e-3 * np.abs(ref).max()) + 1e-7
+    assert (np.abs(got[pix] - ref) <= tol).mean() >= 0.9
+    away = dict(cam, cam_fwd=tuple(-np.asarray(cam["cam_fwd"])), cam_right=tuple(-np.asarray(cam["cam_right"])))
+    img = ctx.render(vol, away, precision=api.F32, mode=api.MODE_PATH)
+    ctx.sync_status()
+    assert float(img.abs().max()) == 0.0
