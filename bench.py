@@ -596,7 +596,7 @@ def run_train(args, ws, rank, local):
                     "capped_at_max_paths": int((npa >= args.train_max_paths).sum()),
                     "met_rule_fraction": float((npa < args.train_max_paths).double().mean()),
                     "desc_dtype": "bf16" if desc_dtype == torch.bfloat16 else "f32",
-                    "kernel": "k_records: one warp per record, 32 paths per round, the rule tested at every "
+                    "kernel": "k_records: a block of 1, 2 or 4 warps per record, the rule tested at every "
                               "path count (FP32 prefix sums, Kahan-compensated totals)"},
         "gpu_launches": None,
         "e2e": {"value": total / e2e_s, "unit": "samples/s", "h2d_bytes_per_step": int(dz.numel() * dz.element_size() + dt_.numel() * 4),
@@ -691,7 +691,7 @@ def run_records(args, ws, rank, local):
         "met_rule_fraction": met,
         "capped_at_max_paths": int((npa >= n_max).sum()),
         "seconds_for_2M_records": 2e6 / rate,
-        "gpu_launches": 32,
+        "gpu_launches": 64,               # k_record_start and k_records per cloud
     }
     if rank == 0:
         print(json.dumps(line), flush=True)
