@@ -39,14 +39,14 @@ L2_FLUSH_BYTES = 256 << 20
 # summaries under profiles/ give the commands), with the SHA-256 prefixes of the sources the
 # captured build was compiled from.  A kernel whose sources changed since reports null.
 NCU_TRAFFIC = {
-    "descriptor": {"bytes_per_query": (795.414272e6 + 5.620736e6) / 178675,
-                   "sources": {"descriptor.cu": "05b2f345e006b04d", "desc_lookup.cuh": "96d43ff4040f8e82",
-                               "volume.cu:k_pack": "f1b80b6358e59e22"}},
-    "network": {"bytes_per_query": (886.175488e6 + 3.624960e6) / 178675,
-                "sources": {"mlp_tc.cu": "57c21e9d2ae6b860", "tc_ptx.cuh": "294268ada12e7cd2",
+    "descriptor": {"bytes_per_query": (795.742208e6 + 5.595392e6) / 178675,
+                   "sources": {"descriptor.cu": "3eeba11fdbbab198", "desc_lookup.cuh": "96d43ff4040f8e82",
+                               "volume.cu:k_pack": "375ff27268e0095e"}},
+    "network": {"bytes_per_query": (884.246528e6 + 0.669696e6) / 178675,
+                "sources": {"mlp_tc.cu": "fb9da248a167cbcd", "tc_ptx.cuh": "294268ada12e7cd2",
                             "tc_net.cuh": "84cfe3d7ca7bea66"}},
-    "network_fp8": {"bytes_per_query": (460.973824e6 + 1.656832e6) / 178675,
-                    "sources": {"mlp_tc.cu": "57c21e9d2ae6b860", "tc_ptx.cuh": "294268ada12e7cd2",
+    "network_fp8": {"bytes_per_query": (460.915200e6 + 1.886720e6) / 178675,
+                    "sources": {"mlp_tc.cu": "fb9da248a167cbcd", "tc_ptx.cuh": "294268ada12e7cd2",
                                 "tc_net.cuh": "84cfe3d7ca7bea66"}},
 }
 
