@@ -290,7 +290,11 @@ k_paths(const VolumeView v, const RenderArgs a, const float* __restrict__ qx, co
         const uint32_t* __restrict__ qps, const int* __restrict__ qcount, int* next, float* sample_val,
         uint32_t* status) {
     const int total = *qcount, warps = (int)(gridDim.x * (blockDim.x >> 5));
-    const int lanes = min(32, max(1, (total + warps - 1) / warps));
+    // up to 8 paths per warp: all at once; beyond, 5 lanes for 8 paths (lanes that end early take
+    // the others: 300 x 300 samples of a 224^3 cloud 2.70 ms with 20 lanes, 2.39 with 12; 512 x 512 x 2
+    // of it 4.69 ms with 32 lanes, a path per lane in nested loops 5.61)
+    const int n = max(1, (total + warps - 1) / warps);
+    const int lanes = n <= 8 ? n : min(32, max(8, (int)((5 * (int64_t)n + 7) / 8)));
     RenderPaths src{v, a, qx, qd, qps, qcount, next, sample_val, status, total, lanes, 0};
     trace_paths(v, f3(a.wl[0], a.wl[1], a.wl[2]), a.E, src);
 }
