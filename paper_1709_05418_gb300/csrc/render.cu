@@ -11,6 +11,7 @@
 
 #include "common.cuh"
 #include "paths.cuh"
+#include "rules.h"
 
 namespace rpnn {
 
@@ -121,7 +122,7 @@ k_primary(const VolumeView v_, const RenderArgs a_, int64_t P_, float* __restric
         base = __shfl_sync(0xffffffffu, base, 0);
         if (want) {
             const int slot = base + __popc(mask & ((1u << lane) - 1u));
-            const int64_t o = 3 * (int64_t)slot;
+            const int64_t o = query_at(slot);
             qx[o] = x.x; qx[o + 1] = x.y; qx[o + 2] = x.z;
             qd[o] = d.x; qd[o + 1] = d.y; qd[o + 2] = d.z;
             qps[slot] = (uint32_t)ps;
@@ -135,10 +136,10 @@ __global__ void k_scatter(const float* __restrict__ g, const uint32_t* __restric
                           const int* __restrict__ g_total, float scale, float* __restrict__ sample_val) {
     // predictions of this render's queries start at g[*g_off] (batched renders) and no
     // index reaches *g_total
-    const int o = g_off ? *g_off : 0;
-    int n = *qcount;
+    const int64_t o = g_off ? *g_off : 0;
+    int64_t n = *qcount;
     if (g_total && *g_total - o < n) n = *g_total - o;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
         sample_val[qps[i]] += scale * g[o + i];
 }
 
@@ -151,12 +152,12 @@ __global__ void __launch_bounds__(128)
 k_nee_env(const VolumeView v, const RenderArgs a, const float* __restrict__ qx, const float* __restrict__ qd,
           const uint32_t* __restrict__ qps, const int* __restrict__ qcount, const float* __restrict__ dirs,
           const float* __restrict__ E, int j0, int n, float* __restrict__ sample_val, uint32_t* status) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, o = query_at(i);
     if (i >= *qcount) return;
     const uint32_t ps = qps[i];
     const uint32_t pixel = ps / (uint32_t)a.spp, s = ps % (uint32_t)a.spp;
-    const float3 x = f3(qx[3 * i], qx[3 * i + 1], qx[3 * i + 2]);
-    const float3 d = f3(qd[3 * i], qd[3 * i + 1], qd[3 * i + 2]);
+    const float3 x = f3(qx[o], qx[o + 1], qx[o + 2]);
+    const float3 d = f3(qd[o], qd[o + 1], qd[o + 2]);
     const Rng rng = make_rng(a.seed, pixel, s, kDomShadow);
     bool capped = false;
     float Ld = 0.0f;
@@ -269,7 +270,7 @@ struct RenderPaths {
         const unsigned i = base + __popc(m & ((1u << lane) - 1u));
         if (!take || i >= (unsigned)total) return -1;
         ps = qps[i];
-        const int64_t o = 3 * (int64_t)i;
+        const int64_t o = query_at(i);
         x = f3(qx[o], qx[o + 1], qx[o + 2]);
         d = f3(qd[o], qd[o + 1], qd[o + 2]);
         rng = make_rng(a.seed, ps / (uint32_t)a.spp, ps % (uint32_t)a.spp, kDomPath);
