@@ -20,19 +20,20 @@
 // (v.lmc, v.dscale, v.albedo_c).
 #pragma once
 #include "common.cuh"
+#include "rules.h"
 
 namespace rpnn {
 
 constexpr int kEventLanes = 11;               // 5 to 18 lanes, 3 to 6 bricks: within 5 % of one another
 constexpr int kWalkSteps = 4;
-constexpr uint32_t kPathPolls = 1u << 24;     // bound on a warp's polls for other warps' results
 
 // Source of paths and sink of estimates for trace_paths:
 //   int fetch(bool want, x, d, rng)  warp-collective; 1: the lane got a path, 0: none yet, -1: none
 //   void finish(L, capped)           the lane's path ended (capped: a device loop reached its cap)
 //   bool stopped()                   warp-uniform: drop everything in flight
 //   bool keep()                      warp-uniform: stay although no lane has work left
-//   void gave_up()                   the bound on polls was reached
+//   void beat()                      a bounce of this warp's lanes: what other warps' waits see as progress
+//   bool idle(bound)                 warp-uniform: one more poll for other warps; false: the bound is reached
 template <class Src>
 __device__ __forceinline__ void trace_paths(const VolumeView& v, const float3 wl, const float E, Src& src) {
     enum { kHit, kFetch, kEnd, kExit, kTurn, kFly, kShadow, kWait, kDone };
@@ -40,7 +41,7 @@ __device__ __forceinline__ void trace_paths(const VolumeView& v, const float3 wl
     float3 x = f3(0.f, 0.f, 0.f), d = f3(0.f, 0.f, 1.f);
     float t = 0.0f, t1 = 0.0f, L = 0.0f, T = 1.0f, te = 0.0f, mu_b = 0.0f;
     float tau = -1.0f;                  // shadow ray: optical depth left to spend, < 0: draw first
-    uint32_t ctr = 0, n = 0, polls = 0;
+    uint32_t ctr = 0, n = 0;
     Rng rng = make_rng(0, 0, 0, 0);
     BrickWalk w{};
     bool capped = false;
@@ -65,6 +66,7 @@ __device__ __forceinline__ void trace_paths(const VolumeView& v, const float3 wl
         if (src.stopped()) break;
         const bool do_hits = hits >= min(kEventLanes, run), do_turns = turns >= min(kEventLanes, run);
         if (do_hits && hits) {
+            src.beat();
             if (state == kHit) {
                 const float4 xi = rng.draw(ctr++);
                 float t0;
@@ -89,6 +91,7 @@ __device__ __forceinline__ void trace_paths(const VolumeView& v, const float3 wl
             continue;
         }
         if (do_turns && (turns || run == 0)) {
+            if (turns) src.beat();
             if (state == kExit) {
                 // next-event estimate of the vertex x from the shadow ray's transmittance; next bounce
                 const float ct = __fmaf_rn(d.z, wl.z, __fmaf_rn(d.x, wl.x, __fmul_rn(d.y, wl.y)));
@@ -120,7 +123,7 @@ __device__ __forceinline__ void trace_paths(const VolumeView& v, const float3 wl
             }
             if (run == 0 && turns == 0 && !__any_sync(0xffffffffu, state < kWait)) {
                 // only waiting for other warps of the block
-                if (++polls >= kPathPolls) { src.gave_up(); break; }
+                if (!src.idle(path_poll_bound(v.track_cap))) break;
                 __nanosleep(200);
             }
             continue;

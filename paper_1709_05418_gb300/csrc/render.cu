@@ -282,7 +282,8 @@ struct RenderPaths {
     }
     __device__ __forceinline__ bool stopped() const { return false; }
     __device__ __forceinline__ bool keep() const { return false; }
-    __device__ __forceinline__ void gave_up() { raise_status(status, kStatTimeout); }
+    __device__ __forceinline__ void beat() {}
+    __device__ __forceinline__ bool idle(uint32_t) { raise_status(status, kStatTimeout); return false; }   // no lane waits
 };
 
 constexpr int kPathBlocks = 5;       // blocks of 128 threads per SM
@@ -361,6 +362,8 @@ struct RecordRing {
     uint32_t slot[kRing];
     unsigned char cap[kRing];
     int next, base, done;
+    uint32_t beats;              // bounces of the block's paths
+    PollBound wait[4];           // of each warp
 };
 struct LabelPaths {
     RecordRing& r;
@@ -445,7 +448,18 @@ struct LabelPaths {
         return __any_sync(0xffffffffu, vr.done != 0);
     }
     __device__ __forceinline__ bool keep() const { return threadIdx.x < 32; }
-    __device__ __forceinline__ void gave_up() { raise_status(status, kStatTimeout); }
+    __device__ __forceinline__ void beat() {
+        if ((threadIdx.x & 31) == 0) atomicAdd(&r.beats, 1u);
+    }
+    __device__ __forceinline__ bool idle(uint32_t bound) {
+        volatile RecordRing& vr = r;
+        int go = 1;
+        if ((threadIdx.x & 31) == 0) {
+            go = r.wait[threadIdx.x >> 5].poll(vr.beats + (uint32_t)vr.base, bound);
+            if (!go) raise_status(status, kStatTimeout);
+        }
+        return __shfl_sync(0xffffffffu, go, 0);
+    }
 };
 
 // 72 registers, 28 warps per SM: 4,096 records of 256 paths in 12.9 ms, with 94 and 20 in 14.7
@@ -462,7 +476,8 @@ k_records(const VolumeView v, int64_t first, int64_t n, uint64_t seed, float rel
             continue;
         }
         for (int k = threadIdx.x; k < kRing; k += blockDim.x) { ring.slot[k] = kEmpty; ring.cap[k] = 0; }
-        if (threadIdx.x == 0) { ring.next = 0; ring.base = 0; ring.done = 0; }
+        if (threadIdx.x == 0) { ring.next = 0; ring.base = 0; ring.done = 0; ring.beats = 0; }
+        if (threadIdx.x < 4) ring.wait[threadIdx.x] = PollBound{0, 0};
         __syncthreads();
         LabelPaths src{ring, f3(xo[3 * i], xo[3 * i + 1], xo[3 * i + 2]), f3(dout[3 * i], dout[3 * i + 1], dout[3 * i + 2]),
                        seed, (uint32_t)(first + i), rel_ci, n_min, n_max, status, -1, KahanF(), KahanF(), 0.0f, 0};

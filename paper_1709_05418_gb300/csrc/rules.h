@@ -15,4 +15,22 @@ namespace rpnn {
 // A render has up to 2^31 - 1 samples, so from i = 715,827,883 on the offset needs 64 bits.
 RPNN_RULE int64_t query_at(int64_t i) { return 3 * i; }
 
+// Waits of a warp whose lanes have no work while other warps of its block trace the paths they wait
+// for.  `progress` counts what those warps get done (bounces of their paths, rounds taken into the
+// label), so the bound is on polls during which nothing happened anywhere in the block, however
+// long the record: the longest such stretch of a healthy block is one tracking call, at most
+// `track_cap` collisions of about 4 us each, and a poll takes at least 0.2 us.
+RPNN_RULE uint32_t path_poll_bound(uint32_t track_cap) {
+    const uint64_t b = (1ull << 24) + 32ull * track_cap;
+    return b > 0xffffffffull ? 0xffffffffu : (uint32_t)b;
+}
+struct PollBound {
+    uint32_t polls, seen;
+    // one more poll; false once `bound` polls in a row saw no progress
+    RPNN_RULE bool poll(uint32_t progress, uint32_t bound) {
+        if (progress != seen) { seen = progress; polls = 0; }
+        return ++polls < bound;
+    }
+};
+
 }  // namespace rpnn

@@ -14,6 +14,17 @@ SHIM = r"""
 using namespace rpnn;
 extern "C" {
 int64_t t_query_at(int64_t i) { return query_at(i); }
+uint32_t t_poll_bound(uint32_t cap) { return path_poll_bound(cap); }
+// polls a wait makes until it gives up, or `total` if it does not; progress every `every` polls
+int64_t t_polls(uint32_t bound, int64_t total, int64_t every) {
+    PollBound w{0, 0};
+    uint32_t progress = 0;
+    for (int64_t i = 0; i < total; ++i) {
+        if (every && i % every == 0) ++progress;
+        if (!w.poll(progress, bound)) return i + 1;
+    }
+    return total;
+}
 }
 """
 
@@ -27,6 +38,8 @@ def rules(tmp_path_factory):
                     str(d / "shim.cpp"), "-o", so], check=True)
     L = ctypes.CDLL(so)
     L.t_query_at.argtypes, L.t_query_at.restype = [ctypes.c_int64], ctypes.c_int64
+    L.t_poll_bound.argtypes, L.t_poll_bound.restype = [ctypes.c_uint32], ctypes.c_uint32
+    L.t_polls.argtypes, L.t_polls.restype = [ctypes.c_uint32, ctypes.c_int64, ctypes.c_int64], ctypes.c_int64
     return L
 
 
@@ -42,3 +55,16 @@ def test_shading_point_offsets_need_64_bits(rules):
         body = src[src.index(kernel + "("):]
         body = body[:body.index("\n}\n")]
         assert not re.search(r"\bint i = blockIdx", body), kernel
+
+
+def test_waits_for_other_warps_are_bounded_from_the_last_progress(rules):
+    """A record of millions of paths adds up more polls than the bound while its block gets on; only
+    polls without any progress may end it, and those do."""
+    assert rules.t_polls(1000, 1000000, 999) == 1000000
+    assert rules.t_polls(1000, 1000000, 0) == 1000
+    assert rules.t_polls(1000, 1000000, 5000) == 1000
+    # no progress for as long as one tracking call may take; the sum does not wrap
+    for cap in (0, 1000000, 2 ** 32 - 1):
+        assert rules.t_poll_bound(cap) >= min(2 ** 24 + 32 * cap, 2 ** 32 - 1)
+    src = open(os.path.join(CSRC, "paths.cuh")).read()
+    assert "++polls" not in src and "src.idle(path_poll_bound(v.track_cap))" in src
