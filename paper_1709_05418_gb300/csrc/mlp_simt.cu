@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "rules.h"
 
 namespace rpnn {
 
@@ -526,7 +527,7 @@ void launch_tile(int M, const int* M_dev, int N, const Seg& s0, const Seg& s1, i
 rpnn_status launch_gemm(int tile, int splits, int M, const int* M_dev, int N, const Seg& s0, const Seg& s1,
                         int nseg, const Epi& e, float* ws, cudaStream_t s) {
     const TileShape& t = kTiles[tile];
-    if ((M + t.bm - 1) / t.bm > 65535) { set_error("GEMM with %d rows exceeds the grid limit", M); return RPNN_ERR_ARG; }
+    if (!gemm_rows_fit(M, t.bm)) { set_error("GEMM with %d rows exceeds the grid limit", M); return RPNN_ERR_ARG; }
     switch (tile) {
         case 0: launch_tile<64, 64, 16, 4, 8>(M, M_dev, N, s0, s1, nseg, e, splits, ws, s); break;
         case 1: launch_tile<128, 64, 16, 8, 8>(M, M_dev, N, s0, s1, nseg, e, splits, ws, s); break;
@@ -587,7 +588,8 @@ GemmKey make_key(int M, int N, const Seg& s0, const Seg* s1, const Epi& e, bool 
 rpnn_status tune(Ctx& c, const GemmKey& key, int M, const int* M_dev, int N, const Seg& s0, const Seg& s1,
                  int nseg, const Epi& e, cudaStream_t s, GemmChoice* out) {
     GemmTuner& tu = c.tuner;
-    // admissible (tile, split) pairs: tiles no taller than twice the rows; a split only
+    // admissible (tile, split) pairs: tiles no taller than twice the rows (the default always) and
+    // not too low for the grid; a split only
     // for inner sizes of at least kMinSplitK (the weight gradients, which sum over the
     // batch; forward GEMMs therefore never split and give the default tile's bits), where
     // the tiles alone fill fewer than one wave, keeping >= 4 K tiles per run and at most
@@ -598,7 +600,7 @@ rpnn_status tune(Ctx& c, const GemmKey& key, int M, const int* M_dev, int N, con
     const int ksteps16 = (s0.K + 15) / 16 + (nseg > 1 ? (s1.K + 15) / 16 : 0);
     for (int t = 0; t < kNumTiles; ++t) {
         const TileShape& ts = kTiles[t];
-        if (t > 0 && ts.bm > 2 * M) continue;
+        if (t > 0 && (ts.bm > 2 * (int64_t)M || !gemm_rows_fit(M, ts.bm))) continue;
         const int64_t blocks = (int64_t)((N + ts.bn - 1) / ts.bn) * ((M + ts.bm - 1) / ts.bm);
         // of the admissible splits the largest: the shortest runs have the smallest rounding error,
         // and the bits do not depend on which of several equally fast splits a timing favours
@@ -672,7 +674,7 @@ rpnn_status gemm(Ctx* c, int M, const int* M_dev, int N, const Seg& s0, const Se
         const GemmKey key = make_key(M, N, s0, s1, e, M_dev != nullptr);
         const GemmChoice* hit = c->tuner.find(key);
         if (hit) {
-            ch = *hit;
+            if (gemm_rows_fit(M, kTiles[hit->tile].bm)) ch = *hit;      // (a table set by the caller may not)
         } else if (cs == cudaStreamCaptureStatusNone) {
             rpnn_status st = tune(*c, key, M, M_dev, N, s0, s1r, nseg, e, s, &ch);
             if (st) return st;

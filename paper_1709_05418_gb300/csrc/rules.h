@@ -33,4 +33,8 @@ struct PollBound {
     }
 };
 
+// FP32 GEMM: row tiles are blocks of grid.y, at most 65,535 of them.  The default tile (64 rows)
+// takes every row count the entry points accept, a 32-row tile half of them.
+RPNN_RULE bool gemm_rows_fit(int64_t M, int bm) { return (M + bm - 1) / bm <= 65535; }
+
 }  // namespace rpnn

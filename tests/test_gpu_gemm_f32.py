@@ -46,3 +46,22 @@ def test_dense_at_tile_edges(widths, din, q, tuned):
     got = ctx.dense_backward(widths, params, x, dout).double()
     assert float(((got - grad).abs() / grad).max()) <= bwd
     ctx.close()
+
+
+def test_tuned_rows_beyond_the_low_tiles():
+    """2,097,121 rows, one more than 65,535 tiles of 32 hold: tuned calls and calls with a 32-row tile
+    from a table run (they are accepted up to 65,535 x 64) and give the default tile's bits."""
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_1709_05418_gb300 import api
+    q, widths, din = 32 * 65535 + 1, (8,), 4
+    params = torch.from_numpy(W.dense_he_init(widths, din, seed=3, bias=0.1)).cuda()
+    x = torch.rand((q, din), generator=torch.Generator().manual_seed(1)).cuda()
+    tuned, plain, given = api.Context(), api.Context(), api.Context()
+    plain.set_autotune(False)
+    ref = plain.dense_forward(widths, params, x)
+    assert torch.equal(tuned.dense_forward(widths, params, x), ref)
+    given.set_autotune_table([dict(e, tile_m=32, tile_n=64, tile_k=16) for e in tuned.autotune_table()])
+    assert torch.equal(given.dense_forward(widths, params, x), ref)
+    for c in (tuned, plain, given):
+        c.close()

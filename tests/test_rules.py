@@ -15,6 +15,7 @@ using namespace rpnn;
 extern "C" {
 int64_t t_query_at(int64_t i) { return query_at(i); }
 uint32_t t_poll_bound(uint32_t cap) { return path_poll_bound(cap); }
+int t_rows_fit(int64_t M, int bm) { return gemm_rows_fit(M, bm); }
 // polls a wait makes until it gives up, or `total` if it does not; progress every `every` polls
 int64_t t_polls(uint32_t bound, int64_t total, int64_t every) {
     PollBound w{0, 0};
@@ -39,6 +40,7 @@ def rules(tmp_path_factory):
     L = ctypes.CDLL(so)
     L.t_query_at.argtypes, L.t_query_at.restype = [ctypes.c_int64], ctypes.c_int64
     L.t_poll_bound.argtypes, L.t_poll_bound.restype = [ctypes.c_uint32], ctypes.c_uint32
+    L.t_rows_fit.argtypes, L.t_rows_fit.restype = [ctypes.c_int64, ctypes.c_int], ctypes.c_int
     L.t_polls.argtypes, L.t_polls.restype = [ctypes.c_uint32, ctypes.c_int64, ctypes.c_int64], ctypes.c_int64
     return L
 
@@ -68,3 +70,16 @@ def test_waits_for_other_warps_are_bounded_from_the_last_progress(rules):
         assert rules.t_poll_bound(cap) >= min(2 ** 24 + 32 * cap, 2 ** 32 - 1)
     src = open(os.path.join(CSRC, "paths.cuh")).read()
     assert "++polls" not in src and "src.idle(path_poll_bound(v.track_cap))" in src
+
+
+def test_row_tiles_fit_the_grid(rules):
+    """Every accepted row count (65,535 x 64) has its default tile; tiles of 32 rows end at half of it,
+    and the tuner asks before it times one."""
+    for bm in (32, 64, 128):
+        for M in (1, bm * 65535):
+            assert rules.t_rows_fit(M, bm)
+        for M in (bm * 65535 + 1, 2 ** 31 - 1):
+            assert not rules.t_rows_fit(M, bm)
+    src = open(os.path.join(CSRC, "mlp_simt.cu")).read()
+    body = src[src.index("rpnn_status tune("):]
+    assert "gemm_rows_fit" in body[:body.index("cands.push_back")]
