@@ -515,7 +515,6 @@ constexpr TileShape kTiles[] = {
 };
 constexpr int kNumTiles = sizeof(kTiles) / sizeof(kTiles[0]);
 constexpr int kSplits[] = {1, 2, 4, 8, 16, 32};
-constexpr int kMinSplitK = 1024;
 
 template <int BM, int BN, int BK, int TM, int TN>
 void launch_tile(int M, const int* M_dev, int N, const Seg& s0, const Seg& s1, int nseg, const Epi& e,
@@ -606,7 +605,7 @@ rpnn_status tune(Ctx& c, const GemmKey& key, int M, const int* M_dev, int N, con
         // and the bits do not depend on which of several equally fast splits a timing favours
         int best_sp = 1;
         for (int sp : kSplits)
-            if (ksteps16 * 16 >= kMinSplitK && blocks < c.num_sms && blocks * sp <= (int64_t)c.num_sms * 8 &&
+            if (gemm_may_split(ksteps16 * 16) && blocks < c.num_sms && blocks * sp <= (int64_t)c.num_sms * 8 &&
                 (ksteps16 * 16 / ts.bk) / sp >= 4)
                 best_sp = std::max(best_sp, sp);
         cands.push_back({t, best_sp});
@@ -652,8 +651,7 @@ rpnn_status tune(Ctx& c, const GemmKey& key, int M, const int* M_dev, int N, con
 rpnn_status gemm(Ctx* c, int M, const int* M_dev, int N, const Seg& s0, const Seg* s1, const Epi& e,
                  cudaStream_t s) {
     if (M <= 0 || N <= 0) return RPNN_OK;
-    // (a sum over many rows keeps the tiled kernel, which may split it)
-    if (N == 1 && !s1 && s0.sak == 1) {
+    if (gemm_row_dot(N, s0.K) && !s1 && s0.sak == 1) {
         k_rowdot<<<(M + kDotRows - 1) / kDotRows, 256, 0, s>>>(M, M_dev, s0, e);
         RPNN_CHECK_LAUNCH();
         return RPNN_OK;
@@ -719,7 +717,7 @@ rpnn_status wgrads(Ctx& c, WJobs& J, cudaStream_t s) {
                 // but the runs' lengths set the sums' rounding
                 int sp = 1;
                 for (int x : kSplits)
-                    if (J.K >= kMinSplitK && (J.K + 15) / 16 * 16 / ts.bk / x >= 4) sp = x;
+                    if (gemm_may_split(J.K) && (J.K + 15) / 16 * 16 / ts.bk / x >= 4) sp = x;
                 cands.push_back({t, sp});
                 maxsplit = std::max(maxsplit, sp);
             }

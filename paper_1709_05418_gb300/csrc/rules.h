@@ -37,4 +37,13 @@ struct PollBound {
 // takes every row count the entry points accept, a 32-row tile half of them.
 RPNN_RULE bool gemm_rows_fit(int64_t M, int bm) { return (M + bm - 1) / bm <= 65535; }
 
+// FP32 GEMM: inner sizes whose sum the tuner may split into runs (counted in K tiles of 16).
+constexpr int kMinSplitK = 1024;
+RPNN_RULE bool gemm_may_split(int64_t K) { return (K + 15) / 16 * 16 >= kMinSplitK; }
+// One output column: a thread per row sums all K products in a row below that, as the tiled kernel
+// would, which adds up to K roundings; longer sums keep the tiled kernel and its runs (at most
+// K / 32 + 32 roundings, and more than one warp per 32 rows: 4,096 rows of 2,400 take 71 us tuned,
+// 131 with a thread each; 100 rows of 16,384 take 85 and 791).
+RPNN_RULE bool gemm_row_dot(int N, int64_t K) { return N == 1 && !gemm_may_split(K); }
+
 }  // namespace rpnn

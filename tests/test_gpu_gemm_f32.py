@@ -65,3 +65,46 @@ def test_tuned_rows_beyond_the_low_tiles():
     assert torch.equal(given.dense_forward(widths, params, x), ref)
     for c in (tuned, plain, given):
         c.close()
+
+
+def small_terms(n):
+    """1, then n - 1 terms of 2^-25: added to 1 one by one, each is rounded away."""
+    t = torch.full((n,), 2.0 ** -25)
+    t[0] = 1.0
+    return t
+
+
+@pytest.mark.parametrize("K,q", [(2400, 1), (2400, 130), (4096, 65), (16384, 3)])
+def test_long_one_column_sums_keep_their_terms(K, q):
+    """No hidden layer: output = a sum of K products.  In runs of at most K / 16 terms (the tuner's
+    fewest above 1,024) the first run loses K / 16 of the small terms at the most, 2^-25 each; a
+    chain of all of them loses K - 1.  Also the last layer of a K-wide network, from relu(x w) = w."""
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_1709_05418_gb300 import api
+    ctx = api.Context()
+    terms = small_terms(K).cuda()
+    exact = float(terms.double().sum())
+    bound = (K / 16) * 2.0 ** -25 + 64 * 2.0 ** -24        # and one rounding per run, two runs' worth
+    params = torch.cat([terms, torch.zeros(1, device="cuda")])
+    got = ctx.dense_forward((), params, torch.ones((q, K), device="cuda"))
+    assert float((got.double() - exact).abs().max()) <= bound
+    wide = torch.cat([torch.ones(K, device="cuda"), torch.zeros(K, device="cuda"), params])
+    got = ctx.dense_forward((K,), wide, torch.ones((q, 1), device="cuda"))
+    assert float((got.double() - exact).abs().max()) <= bound
+    ctx.close()
+
+
+def test_long_sums_over_rows_of_one_wide_layers_keep_their_terms():
+    """The weight gradient of a 1-wide layer on 1 input is one sum over the rows."""
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_1709_05418_gb300 import api
+    ctx = api.Context()
+    q = 16384
+    dout = small_terms(q).cuda()
+    params = torch.tensor([1.0, 0.0, 1.0, 0.0], device="cuda")          # w, b, w_out, b_out
+    grad = ctx.dense_backward((1,), params, torch.ones((q, 1), device="cuda"), dout).double()
+    exact = float(dout.double().sum())
+    assert abs(float(grad[0]) - exact) <= (q / 16) * 2.0 ** -25 + 64 * 2.0 ** -24
+    ctx.close()

@@ -16,6 +16,7 @@ extern "C" {
 int64_t t_query_at(int64_t i) { return query_at(i); }
 uint32_t t_poll_bound(uint32_t cap) { return path_poll_bound(cap); }
 int t_rows_fit(int64_t M, int bm) { return gemm_rows_fit(M, bm); }
+int t_row_dot(int N, int64_t K) { return gemm_row_dot(N, K); }
 // polls a wait makes until it gives up, or `total` if it does not; progress every `every` polls
 int64_t t_polls(uint32_t bound, int64_t total, int64_t every) {
     PollBound w{0, 0};
@@ -41,6 +42,7 @@ def rules(tmp_path_factory):
     L.t_query_at.argtypes, L.t_query_at.restype = [ctypes.c_int64], ctypes.c_int64
     L.t_poll_bound.argtypes, L.t_poll_bound.restype = [ctypes.c_uint32], ctypes.c_uint32
     L.t_rows_fit.argtypes, L.t_rows_fit.restype = [ctypes.c_int64, ctypes.c_int], ctypes.c_int
+    L.t_row_dot.argtypes, L.t_row_dot.restype = [ctypes.c_int, ctypes.c_int64], ctypes.c_int
     L.t_polls.argtypes, L.t_polls.restype = [ctypes.c_uint32, ctypes.c_int64, ctypes.c_int64], ctypes.c_int64
     return L
 
@@ -83,3 +85,11 @@ def test_row_tiles_fit_the_grid(rules):
     src = open(os.path.join(CSRC, "mlp_simt.cu")).read()
     body = src[src.index("rpnn_status tune("):]
     assert "gemm_rows_fit" in body[:body.index("cands.push_back")]
+
+
+def test_long_one_column_sums_are_not_one_chain(rules):
+    """A column whose sum may be split is not summed by one thread per row."""
+    for K in (1, 200, 1008):
+        assert rules.t_row_dot(1, K) and not rules.t_row_dot(2, K)
+    for K in (1009, 2400, 16384, 2 ** 22):
+        assert not rules.t_row_dot(1, K)
