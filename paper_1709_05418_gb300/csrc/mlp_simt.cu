@@ -588,11 +588,11 @@ rpnn_status tune(Ctx& c, const GemmKey& key, int M, const int* M_dev, int N, con
                  int nseg, const Epi& e, cudaStream_t s, GemmChoice* out) {
     GemmTuner& tu = c.tuner;
     // admissible (tile, split) pairs: tiles no taller than twice the rows (the default always) and
-    // not too low for the grid; a split only
-    // for inner sizes of at least kMinSplitK (the weight gradients, which sum over the
-    // batch; forward GEMMs therefore never split and give the default tile's bits), where
-    // the tiles alone fill fewer than one wave, keeping >= 4 K tiles per run and at most
-    // 8 blocks per SM
+    // not too low for the grid; a split only for inner sizes of at least kMinSplitK, where the
+    // tiles alone fill fewer than one wave, keeping >= 4 K tiles per run and at most 8 blocks per
+    // SM.  Those are the weight gradients, which sum over the batch, and layers of 1,009 inputs or
+    // more (plain MLPs, the larger stencils); the network's own forward layers sum 226 + 200
+    // products and give the default tile's bits.
     struct Cand { int t, sp; };
     std::vector<Cand> cands;
     int maxsplit = 1;
@@ -601,15 +601,18 @@ rpnn_status tune(Ctx& c, const GemmKey& key, int M, const int* M_dev, int N, con
         const TileShape& ts = kTiles[t];
         if (t > 0 && (ts.bm > 2 * (int64_t)M || !gemm_rows_fit(M, ts.bm))) continue;
         const int64_t blocks = (int64_t)((N + ts.bn - 1) / ts.bn) * ((M + ts.bm - 1) / ts.bm);
-        // of the admissible splits the largest: the shortest runs have the smallest rounding error,
-        // and the bits do not depend on which of several equally fast splits a timing favours
+        // of a tile's admissible splits the largest: the shortest runs have the smallest rounding
+        // error.  The tile itself, and with it the runs, is the timing's choice, as is one run where
+        // the default tile is fastest so: a sum that may be split has its bits from the table, and
+        // repeats them where the table is restored.  (Runs from the shape alone were 10 to 20 %
+        // slower, in the gradients of 400 x 2,400 layers or in their forward.)
         int best_sp = 1;
         for (int sp : kSplits)
             if (gemm_may_split(ksteps16 * 16) && blocks < c.num_sms && blocks * sp <= (int64_t)c.num_sms * 8 &&
                 (ksteps16 * 16 / ts.bk) / sp >= 4)
                 best_sp = std::max(best_sp, sp);
         cands.push_back({t, best_sp});
-        if (t == 0 && best_sp > 1) cands.push_back({0, 1});      // the default's time, for the table
+        if (t == 0 && best_sp > 1) cands.push_back({0, 1});      // the default itself
         maxsplit = std::max(maxsplit, best_sp);
     }
     rpnn_status st = tu.scratch.reserve((size_t)M * N * sizeof(float));
