@@ -438,7 +438,8 @@ rpnn_status rpnn_set_train_precision(rpnn_ctx* ctx, int32_t precision);
  * 64 x 64 tile without a split and the table is kept. */
 rpnn_status rpnn_set_autotune(rpnn_ctx* ctx, int32_t on);
 typedef struct {
-    int32_t M, N, K0, K1;          /* rows, columns, inner sizes of the two operand segments */
+    int32_t M, N, K0, K1;          /* rows, columns, inner sizes of the two operand segments
+                                      (grouped weight gradients: of one, and their number) */
     int32_t flags;                 /* operand layouts and epilogue kind (library-defined bits) */
     int32_t tile_m, tile_n, tile_k, splits;   /* the choice */
     float us, default_us;          /* its measured time and that of the default tile (us) */

@@ -573,6 +573,7 @@ rpnn_status launch_wgrads(int tile, const WJobs& J, cudaStream_t s) {
     return RPNN_OK;
 }
 
+constexpr int kGroupedFlag = 1 << 9;       // (bit 8: the tensor-core GEMM)
 GemmKey make_key(int M, int N, const Seg& s0, const Seg* s1, const Epi& e, bool dyn) {
     GemmKey k{};
     k.M = M; k.N = N; k.K0 = s0.K; k.K1 = s1 ? s1->K : 0;
@@ -690,9 +691,17 @@ rpnn_status gemm(Ctx* c, int M, const int* M_dev, int N, const Seg& s0, const Se
     return launch_gemm(ch.tile, ch.splits, M, M_dev, N, s0, s1r, nseg, e, ws, s);
 }
 
-// All of J's weight gradients; the tile and split of the shape (M, first job's N, K) are timed
-// on the whole launch at its first use like gemm()'s, and recorded under the key one such GEMM
-// has.
+// The grouped weight gradients' entry in the tuner's table: one launch of n problems, up to `nmax`
+// columns wide, is neither fastest with what one such GEMM is, nor is another group.
+GemmKey wgrads_key(const WJobs& J, int nmax) {
+    GemmKey k{};
+    k.M = J.M; k.N = nmax; k.K0 = J.K; k.K1 = J.n;
+    k.flags = kGroupedFlag;
+    return k;
+}
+
+// All of J's weight gradients; the tile and split are timed on the whole launch at its first use
+// like gemm()'s.
 rpnn_status wgrads(Ctx& c, WJobs& J, cudaStream_t s) {
     if (J.n == 0) return RPNN_OK;
     GemmTuner& tu = c.tuner;
@@ -702,8 +711,7 @@ rpnn_status wgrads(Ctx& c, WJobs& J, cudaStream_t s) {
     J.splits = 1;
     int tile = 0;
     if (tu.enabled) {
-        Seg sg = seg(J.j[0].A, 1, J.M, J.j[0].B, J.j[0].ldb, 1, J.K);
-        const GemmKey key = make_key(J.M, J.j[0].N, sg, nullptr, epi(J.j[0].C, J.j[0].N), false);
+        const GemmKey key = wgrads_key(J, nmax);
         cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
         RPNN_CUDA_TRY(cudaStreamIsCapturing(s, &cs));
         const GemmChoice* hit = tu.find(key);

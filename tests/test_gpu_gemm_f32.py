@@ -108,3 +108,31 @@ def test_long_sums_over_rows_of_one_wide_layers_keep_their_terms():
     exact = float(dout.double().sum())
     assert abs(float(grad[0]) - exact) <= (q / 16) * 2.0 ** -25 + 64 * 2.0 ** -24
     ctx.close()
+
+
+def test_grouped_gradients_do_not_share_a_plain_gradients_tile():
+    """The network's 31 weight gradients are one launch and a 200 x 200 plain layer's is one GEMM:
+    each is timed by itself, so neither's split nor speed depends on which ran first.  Networks of
+    another input width group other problems."""
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_1709_05418_gb300 import api
+    q = 64
+    g = torch.Generator().manual_seed(8)
+    ctx = api.Context()
+
+    def entries():
+        return {(e["M"], e["N"], e["K0"], e["K1"], e["flags"]) for e in ctx.autotune_table() if e["K0"] == q}
+
+    params = torch.from_numpy(W.dense_he_init((200, 200), 200, seed=3, bias=0.1)).cuda()
+    ctx.dense_backward((200, 200), params, torch.rand((q, 200), generator=g).cuda(), torch.rand(q, generator=g).cuda())
+    plain = entries()
+    assert plain
+    for n_xy, din in ((5, 226), (2, 13)):
+        before = entries()
+        n = ctx.stencil_param_count(n_xy)
+        ctx.stencil_backward(n_xy, torch.randn(n, generator=g).cuda() * 0.05, torch.rand((q, 10, din), generator=g).cuda(),
+                             torch.rand(q, generator=g).cuda())
+        new = [k for k in entries() - before if k[0] == 200]
+        assert len(new) == 1 and new[0][:4] == (200, max(din, 200), q, 31), new
+    ctx.close()
