@@ -223,7 +223,6 @@ struct Ctx {
     DevBuf t_lpart;                     // block sums of the loss
     DevBuf t_w16, t_saved16;            // BF16 training: weight image, activation copies
     DevBuf t_gb32, t_gb16;              // BF16 training: per-layer gradients (FP32; BF16 and transposed BF16)
-    int64_t group_rows = INT64_MAX;     // rows up to which the FP32 backward keeps every layer's gradient
     std::vector<cudaEvent_t> t_events;  // BF16 training: kTrainEvents gradient-ready / fork / join events
     cudaStream_t side_stream[2] = {nullptr, nullptr};   // BF16 training: weight gradients beside the
     DevBuf t_ws2;                       // data-gradient chain; the second stream's split-K workspace

@@ -700,6 +700,17 @@ GemmKey wgrads_key(const WJobs& J, int nmax) {
     return k;
 }
 
+// Buffers of the grouped gradients of q rows beside the kept gradients: partial sums (*ws) and the
+// tuner's outputs (*scratch).
+void wgrads_need(const Ctx& c, const WJobs& J, int nmax, bool capturing, size_t* ws, size_t* scratch) {
+    const GemmChoice* hit = c.tuner.enabled ? c.tuner.find(wgrads_key(J, nmax)) : nullptr;
+    const bool timed = c.tuner.enabled && !hit && !capturing;
+    const int runs = hit ? hit->splits : (timed ? grouped_runs(J.K, 8) : 1);     // (8: the smallest K step)
+    const size_t out = (size_t)J.M * nmax * J.n * sizeof(float);
+    *ws = runs > 1 ? runs * out : 0;
+    *scratch = timed ? out : 0;
+}
+
 // All of J's weight gradients; the tile and split are timed on the whole launch at its first use
 // like gemm()'s.
 rpnn_status wgrads(Ctx& c, WJobs& J, cudaStream_t s) {
@@ -726,9 +737,7 @@ rpnn_status wgrads(Ctx& c, WJobs& J, cudaStream_t s) {
                 const TileShape& ts = kTiles[t];
                 // a sum over K rows in as many runs as one such GEMM takes: the launch is full without,
                 // but the runs' lengths set the sums' rounding
-                int sp = 1;
-                for (int x : kSplits)
-                    if (gemm_may_split(J.K) && (J.K + 15) / 16 * 16 / ts.bk / x >= 4) sp = x;
+                const int sp = grouped_runs(J.K, ts.bk);
                 cands.push_back({t, sp});
                 maxsplit = std::max(maxsplit, sp);
             }
@@ -940,18 +949,30 @@ rpnn_status rpnn_backward_f32(Ctx& c, const NetDims& nd, const float* P, const f
     const float* g = saved + (size_t)22 * q * H;
     // Up to kGroupRows rows every layer's gradient is kept and the 31 weight gradients and 22
     // bias sums follow the data-gradient chain as one launch each: one layer's cannot fill the
-    // chip (a step of 1,000 rows: 1.41 -> 0.64 ms).  Beyond that, or where the 22 buffers do not
-    // fit beside what is allocated, a layer's own launches do with three.
-    constexpr int64_t kGroupRows = 1 << 17;
-    bool group = q <= std::min(kGroupRows, c.group_rows);
-    constexpr int NG = 22;
+    // chip (a step of 1,000 rows: 1.41 -> 0.64 ms).  Beyond that, or where the 22 buffers and the
+    // launch's workspace do not fit beside what is allocated, a layer's own launches do with three.
+    constexpr int NG = 22, NW = 31;
     rpnn_status st = c.t_dg.reserve((size_t)q * sizeof(float));
     if (st) return st;
-    if (group && c.t_gb32.reserve((size_t)NG * q * H * sizeof(float)) != RPNN_OK) {
-        cudaGetLastError();
-        c.group_rows = q - 1;             // not tried again (a captured step must not allocate)
+    WJobs wj{};
+    wj.M = RPNN_H; wj.K = M; wj.n = NW;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    RPNN_CUDA_TRY(cudaStreamIsCapturing(s, &cs));
+    const bool capturing = cs != cudaStreamCaptureStatusNone;
+    size_t need[3] = {(size_t)NG * q * H * sizeof(float), 0, 0}, mem_free = 0, mem_total = 0;
+    wgrads_need(c, wj, std::max<int>(nd.din, RPNN_H), capturing, &need[1], &need[2]);
+    DevBuf* const buf[3] = {&c.t_gb32, &c.tuner.ws, &c.tuner.scratch};
+    int64_t missing = 0;
+    for (int i = 0; i < 3; ++i) missing += need[i] > buf[i]->bytes ? (int64_t)need[i] : 0;
+    if (missing && !capturing) RPNN_CUDA_TRY(cudaMemGetInfo(&mem_free, &mem_total));
+    bool group = group_gradients(q, missing, capturing, (int64_t)mem_free);
+    for (int i = 0; i < 3 && group; ++i) {
+        if (need[i] <= buf[i]->bytes || buf[i]->reserve(need[i]) == RPNN_OK) continue;
+        cudaGetLastError();               // taken by another process or thread meanwhile
+        c.t_gb32.release();
         group = false;
     }
+    wj.n = 0;
     if (!group) {
         if (!st) st = c.act0.reserve((size_t)q * H * sizeof(float));
         if (!st) st = c.act1.reserve((size_t)q * H * sizeof(float));
@@ -963,8 +984,6 @@ rpnn_status rpnn_backward_f32(Ctx& c, const NetDims& nd, const float* P, const f
     // buffers of the layers' pre-activation gradients: dpre of a block or standard layer, and da1
     auto pre = [&]() { return group ? c.t_gb32.as<float>() + (size_t)(next++) * q * H : two[flip ^= 1]; };
     auto inner = [&]() { return group ? c.t_gb32.as<float>() + (size_t)(next++) * q * H : c.act2.as<float>(); };
-    WJobs wj{};
-    wj.M = RPNN_H; wj.K = M;
     ColsumJobs cj{};
     cj.M = M; cj.N = RPNN_H;
     // dW = da^T x over the q rows, x [q][N] with row pitch ldx

@@ -46,4 +46,21 @@ RPNN_RULE bool gemm_may_split(int64_t K) { return (K + 15) / 16 * 16 >= kMinSpli
 // 131 with a thread each; 100 rows of 16,384 take 85 and 791).
 RPNN_RULE bool gemm_row_dot(int N, int64_t K) { return N == 1 && !gemm_may_split(K); }
 
+// FP32 backward with all weight gradients in one launch: every layer's gradient is kept until then,
+// 17,600 bytes a row.  A layer's own launches do beyond kGroupRows rows (where they fill the chip),
+// and where the buffers that are missing would not fit beside what is allocated; asked again at each
+// call, so that a step that could not have them once may later.  While a stream is being
+// captured nothing is allocated: the buffers of the direct run before it are there or not.
+constexpr int64_t kGroupRows = 1 << 17;
+constexpr int64_t kGroupSlack = 64 << 20;         // for rounding of the allocations and the rest of the step
+RPNN_RULE bool group_gradients(int64_t rows, int64_t missing, bool capturing, int64_t free_bytes) {
+    return rows <= kGroupRows && (missing == 0 || (!capturing && missing + kGroupSlack <= free_bytes));
+}
+// Runs of its sums over K rows for a tile of K step bk (as many as one such GEMM takes at most).
+RPNN_RULE int grouped_runs(int64_t K, int bk) {
+    int runs = 1;
+    while (gemm_may_split(K) && runs < 32 && (K + 15) / 16 * 16 / bk / (2 * runs) >= 4) runs *= 2;
+    return runs;
+}
+
 }  // namespace rpnn

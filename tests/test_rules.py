@@ -17,6 +17,8 @@ int64_t t_query_at(int64_t i) { return query_at(i); }
 uint32_t t_poll_bound(uint32_t cap) { return path_poll_bound(cap); }
 int t_rows_fit(int64_t M, int bm) { return gemm_rows_fit(M, bm); }
 int t_row_dot(int N, int64_t K) { return gemm_row_dot(N, K); }
+int t_group(int64_t rows, int64_t missing, int capturing, int64_t mem) { return group_gradients(rows, missing, capturing != 0, mem); }
+int t_grouped_runs(int64_t K, int bk) { return grouped_runs(K, bk); }
 // polls a wait makes until it gives up, or `total` if it does not; progress every `every` polls
 int64_t t_polls(uint32_t bound, int64_t total, int64_t every) {
     PollBound w{0, 0};
@@ -43,6 +45,8 @@ def rules(tmp_path_factory):
     L.t_poll_bound.argtypes, L.t_poll_bound.restype = [ctypes.c_uint32], ctypes.c_uint32
     L.t_rows_fit.argtypes, L.t_rows_fit.restype = [ctypes.c_int64, ctypes.c_int], ctypes.c_int
     L.t_row_dot.argtypes, L.t_row_dot.restype = [ctypes.c_int, ctypes.c_int64], ctypes.c_int
+    L.t_group.argtypes, L.t_group.restype = [ctypes.c_int64, ctypes.c_int64, ctypes.c_int, ctypes.c_int64], ctypes.c_int
+    L.t_grouped_runs.argtypes, L.t_grouped_runs.restype = [ctypes.c_int64, ctypes.c_int], ctypes.c_int
     L.t_polls.argtypes, L.t_polls.restype = [ctypes.c_uint32, ctypes.c_int64, ctypes.c_int64], ctypes.c_int64
     return L
 
@@ -93,3 +97,20 @@ def test_long_one_column_sums_are_not_one_chain(rules):
         assert rules.t_row_dot(1, K) and not rules.t_row_dot(2, K)
     for K in (1009, 2400, 16384, 2 ** 22):
         assert not rules.t_row_dot(1, K)
+
+
+def test_grouped_gradients_only_where_everything_they_need_fits(rules):
+    """The kept gradients and the grouped launch's workspace together decide, nothing is allocated
+    under capture, and memory that is free again is used again."""
+    rows, need, slack = 100000, 2 * 10 ** 9, 64 << 20
+    assert rules.t_group(rows, need, 0, need + slack)
+    assert not rules.t_group(rows, need, 0, need + slack - 1)          # the buffers alone would fit
+    assert not rules.t_group(rows, need, 1, 2 ** 40)
+    assert rules.t_group(rows, 0, 1, 0) and rules.t_group(2 ** 17, 0, 0, 0)
+    assert not rules.t_group(2 ** 17 + 1, 0, 0, 2 ** 40)
+    for K, bk, runs in ((1008, 16, 1), (1009, 16, 16), (1009, 8, 32), (2047, 16, 32), (2000, 16, 16), (4096, 16, 32), (10 ** 6, 8, 32)):
+        assert rules.t_grouped_runs(K, bk) == runs, (K, bk)
+    src = open(os.path.join(CSRC, "mlp_simt.cu")).read() + open(os.path.join(CSRC, "internal.h")).read()
+    assert "group_rows" not in src               # no limit outlives the call that met it
+    body = src[src.index("rpnn_status rpnn_backward_f32("):]
+    assert "wgrads_need" in body[:body.index("group_gradients(")]
