@@ -6,6 +6,7 @@
 #include <new>
 
 #include "common.cuh"
+#include "rules.h"
 
 namespace rpnn {
 
@@ -463,10 +464,16 @@ static rpnn_status render_impl(Ctx* c, int32_t vol, const rpnn_render_desc* desc
     st = c->sample_val.reserve(P * sizeof(float));
     if (!st) st = c->q_count.reserve((2 + nchunks) * sizeof(int));
     if (!st) st = c->light.reserve(lights.size() * sizeof(float));
-    if (queries) {
-        if (!st) st = c->q_x.reserve(P * 3 * sizeof(float));
-        if (!st) st = c->q_d.reserve(P * 3 * sizeof(float));
-        if (!st) st = c->q_ps.reserve(P * sizeof(uint32_t));
+    int64_t slice = path ? path_slice(P) : P;       // samples whose shading points are listed at a time
+    while (queries && !st) {
+        st = c->q_x.reserve(slice * 3 * sizeof(float));
+        if (!st) st = c->q_d.reserve(slice * 3 * sizeof(float));
+        if (!st) st = c->q_ps.reserve(slice * sizeof(uint32_t));
+        if (!st || !path || slice <= kMinPathSlice) break;
+        c->q_x.release(); c->q_d.release(); c->q_ps.release();
+        cudaGetLastError();
+        slice = path_slice_smaller(slice);
+        st = RPNN_OK;
     }
     if (net) {
         if (!st) st = c->g_out.reserve(P * sizeof(float));
@@ -493,12 +500,13 @@ static rpnn_status render_impl(Ctx* c, int32_t vol, const rpnn_render_desc* desc
     // and environment next-event kernels
     RPNN_CUDA_TRY(cudaMemcpyAsync(c->light.p, lights.data(), lights.size() * sizeof(float), cudaMemcpyHostToDevice, s));
     const float* ldir = c->light.as<float>();
-    RPNN_CUDA_TRY(cudaMemsetAsync(qc, 0, 2 * sizeof(int), s));
-    {
+    for (int64_t first = 0; first < P; first += slice) {
         NvtxRange stage("primary");
+        RPNN_CUDA_TRY(cudaMemsetAsync(qc, 0, 2 * sizeof(int), s));
         st = launch_primary(*c, vv, rd0, c->sample_val.as<float>(), queries ? c->q_x.as<float>() : nullptr,
                             queries ? c->q_d.as<float>() : nullptr, queries ? c->q_ps.as<uint32_t>() : nullptr,
-                            queries ? qc : nullptr, nullptr, nullptr, nullptr, nullptr, s);
+                            queries ? qc : nullptr, nullptr, nullptr, nullptr, nullptr, s, first,
+                            std::min(slice, P - first));
         if (st) return st;
         if (path) {
             st = launch_paths(*c, vv, rd0, c->q_x.as<float>(), c->q_d.as<float>(), c->q_ps.as<uint32_t>(), qc, qc + 1,

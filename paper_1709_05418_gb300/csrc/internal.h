@@ -284,7 +284,8 @@ rpnn_status launch_descriptor_batch(Ctx& c, const BatchItemDev* items, int n, co
 // dout, Ld; per pixel sample) are each optional.
 rpnn_status launch_primary(Ctx& c, const VolumeView& vv, const rpnn_render_desc& rd,
                            float* sample_val, float* qx, float* qd, uint32_t* qps, int* qcount,
-                           int* hit, float* xo, float* dout, float* Ld, cudaStream_t s);
+                           int* hit, float* xo, float* dout, float* Ld, cudaStream_t s,
+                           int64_t first = 0, int64_t count = -1);
 // g_off / g_total (device, optional): this render's predictions start at g[*g_off] and
 // stop before g[*g_total] (batched renders)
 rpnn_status launch_scatter_composite(Ctx& c, const rpnn_render_desc& rd, float alpha,

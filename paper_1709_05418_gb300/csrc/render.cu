@@ -41,7 +41,7 @@ struct PrimaryItem {
 // RPNN_MAX_BATCH renders (items[i] from block first_block on); each block copies its item
 // into shared memory and works on that render's samples, writing into its region of the
 // per-sample buffers and appending its shading points to that region with its own count.
-// `lanes` (not BATCH): samples per warp.  A warp's rays diverge, so where the image has fewer
+// Not BATCH: samples first .. P - 1.  `lanes` (not BATCH): samples per warp.  A warp's rays diverge, so where the image has fewer
 // samples than the chip holds threads, fewer of them share a warp (64 x 64 samples, this pass alone: 118 us
 // with 32 per warp, 94 with 4, about 80 with 2).
 template <bool BATCH>
@@ -50,7 +50,7 @@ k_primary(const VolumeView v_, const RenderArgs a_, int64_t P_, float* __restric
           float* __restrict__ qx, float* __restrict__ qd, uint32_t* __restrict__ qps,
           int* __restrict__ qcount, int* __restrict__ hit_out, float* __restrict__ x_out,
           float* __restrict__ d_out, float* __restrict__ Ld_out, uint32_t* status,
-          const PrimaryItem* __restrict__ items, int n_items, int lanes) {
+          const PrimaryItem* __restrict__ items, int n_items, int lanes, int64_t first) {
     __shared__ __align__(16) PrimaryItem it;
     __shared__ int s_item;
     if (BATCH) {
@@ -76,7 +76,7 @@ k_primary(const VolumeView v_, const RenderArgs a_, int64_t P_, float* __restric
     const int64_t P = BATCH ? it.P : P_;
     const int wl = (int)threadIdx.x & 31;
     const int64_t ps = BATCH ? (blockIdx.x - it.first_block) * (int64_t)blockDim.x + threadIdx.x
-                             : ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * lanes + wl;
+                             : first + ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * lanes + wl;
     const bool active = ps < P && (BATCH || wl < lanes);
     int hit = 0;
     float3 x = f3(0.f, 0.f, 0.f), d = f3(0.f, 0.f, 1.f);
@@ -544,7 +544,7 @@ rpnn_status launch_primary_batch(Ctx& c, const void* tables, int n, int64_t bloc
     const PrimaryItem* pi = static_cast<const PrimaryItem*>(tables);
     k_primary<true><<<(unsigned)blocks, 128, 0, s>>>(VolumeView{}, RenderArgs{}, 0, sample_val, qx, qd, qps, qcount,
                                                      nullptr, nullptr, nullptr, nullptr, c.status.as<uint32_t>(), pi,
-                                                     n, 32);
+                                                     n, 32, 0);
     RPNN_CHECK_LAUNCH();
     return RPNN_OK;
 }
@@ -564,16 +564,16 @@ rpnn_status launch_scatter_composite_batch(Ctx& c, const void* tables, int n, in
 
 rpnn_status launch_primary(Ctx& c, const VolumeView& vv, const rpnn_render_desc& rd,
                            float* sample_val, float* qx, float* qd, uint32_t* qps, int* qcount,
-                           int* hit, float* xo, float* dout, float* Ld, cudaStream_t s) {
-    const int64_t P = (int64_t)rd.width * rd.height * rd.spp;
+                           int* hit, float* xo, float* dout, float* Ld, cudaStream_t s, int64_t first, int64_t count) {
+    const int64_t P = count < 0 ? (int64_t)rd.width * rd.height * rd.spp : count;
     // as many samples per warp as give 20 warps per SM some (24 fit), two at least; above 48,640
     // samples the issue rate counts, not the latency (BF16 renders of a 224^3 cloud: 128 x 128
     // samples 260 us with 32 per warp, 236 with 8; 208 x 208: 390, with 16 375; 240 x 240: 409, with 16 418)
     int lanes = 2;
     while (lanes < 32 && (int64_t)lanes * c.num_sms * 20 < P) lanes *= 2;
     const int64_t blocks = (P + 4 * lanes - 1) / (4 * lanes);
-    k_primary<false><<<(unsigned)blocks, 128, 0, s>>>(vv, make_args(rd), P, sample_val, qx, qd, qps, qcount,
-                                                      hit, xo, dout, Ld, c.status.as<uint32_t>(), nullptr, 0, lanes);
+    k_primary<false><<<(unsigned)blocks, 128, 0, s>>>(vv, make_args(rd), first + P, sample_val, qx, qd, qps, qcount, hit,
+                                                      xo, dout, Ld, c.status.as<uint32_t>(), nullptr, 0, lanes, first);
     RPNN_CHECK_LAUNCH();
     return RPNN_OK;
 }

@@ -19,6 +19,8 @@ int t_rows_fit(int64_t M, int bm) { return gemm_rows_fit(M, bm); }
 int t_row_dot(int N, int64_t K) { return gemm_row_dot(N, K); }
 int t_group(int64_t rows, int64_t missing, int capturing, int64_t mem) { return group_gradients(rows, missing, capturing != 0, mem); }
 int t_grouped_runs(int64_t K, int bk) { return grouped_runs(K, bk); }
+int64_t t_slice(int64_t P) { return path_slice(P); }
+int64_t t_slice_smaller(int64_t n) { return path_slice_smaller(n); }
 // polls a wait makes until it gives up, or `total` if it does not; progress every `every` polls
 int64_t t_polls(uint32_t bound, int64_t total, int64_t every) {
     PollBound w{0, 0};
@@ -47,6 +49,8 @@ def rules(tmp_path_factory):
     L.t_row_dot.argtypes, L.t_row_dot.restype = [ctypes.c_int, ctypes.c_int64], ctypes.c_int
     L.t_group.argtypes, L.t_group.restype = [ctypes.c_int64, ctypes.c_int64, ctypes.c_int, ctypes.c_int64], ctypes.c_int
     L.t_grouped_runs.argtypes, L.t_grouped_runs.restype = [ctypes.c_int64, ctypes.c_int], ctypes.c_int
+    for f in (L.t_slice, L.t_slice_smaller):
+        f.argtypes, f.restype = [ctypes.c_int64], ctypes.c_int64
     L.t_polls.argtypes, L.t_polls.restype = [ctypes.c_uint32, ctypes.c_int64, ctypes.c_int64], ctypes.c_int64
     return L
 
@@ -114,3 +118,18 @@ def test_grouped_gradients_only_where_everything_they_need_fits(rules):
     assert "group_rows" not in src               # no limit outlives the call that met it
     body = src[src.index("rpnn_status rpnn_backward_f32("):]
     assert "wgrads_need" in body[:body.index("group_gradients(")]
+
+
+def test_path_renders_list_a_bounded_slice(rules):
+    """The shading-point lists of a path-traced image do not grow with it (28 bytes a sample would be
+    60 GB at 2^31 - 1), and shrink to 2 MB before a render gives up."""
+    for P in (1, 2 ** 16, 2 ** 24, 2 ** 31 - 1):
+        n = rules.t_slice(P)
+        assert n == min(P, 2 ** 24) and 28 * n <= 470e6
+        while n > 2 ** 16:
+            assert rules.t_slice_smaller(n) < n
+            n = rules.t_slice_smaller(n)
+        assert 28 * n <= 2e6
+    src = open(os.path.join(CSRC, "capi.cu")).read()
+    body = src[src.index("static rpnn_status render_impl("):]
+    assert "slice = path ? path_slice(P) : P;" in body and "q_x.reserve(slice * 3" in body
