@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "rules.h"
 
 namespace rpnn {
 
@@ -197,8 +198,8 @@ __global__ void k_mip_pass_multi(const __grid_constant__ MipJobs J) {
 // i0 = off + m, output j covers blocks j .. j + Q - 1 of the line shifted by off.
 struct MipXJob {
     float* out;
-    const float* w;       // [st][8]: the Q weights m = p + q st of phase p
-    int ax, st, off;
+    const float* w;       // streamed: [st][8], the Q weights m = p + q st of phase p; else the T taps
+    int ax, st, off, T;
 };
 struct MipXJobs {
     MipXJob j[kMaxLevels];
@@ -236,6 +237,29 @@ __device__ __forceinline__ void mip_x_stream(const MipXJob& b, const float* line
         acc0[Q - 1] = acc1[Q - 1] = 0.0f;
     }
 }
+// nr consecutive x lines (src) into shared memory, line pitch nx + 1 floats
+__device__ __forceinline__ void stage_lines(const float* __restrict__ src, int nx, int nr, float* lines) {
+    const int pitch = nx + 1;
+    __syncthreads();                       // the previous lines' readers are done
+    // the nr lines are nr * nx consecutive floats: eight loads per thread in flight at once
+    const int total = nr * nx, nb = (int)blockDim.x;
+    int e = threadIdx.x;
+    for (; e + 7 * nb < total; e += 8 * nb) {
+        float v[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[k] = __ldg(src + e + k * nb);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const int ee = e + k * nb, r = ee / nx;
+            lines[r * pitch + ee - r * nx] = v[k];
+        }
+    }
+    for (; e < total; e += nb) {
+        const int r = e / nx;
+        lines[r * pitch + e - r * nx] = __ldg(src + e);
+    }
+    __syncthreads();
+}
 __global__ void __launch_bounds__(kXThreads)
 k_mip_pass_x(const float* __restrict__ in, int nx, int64_t nrows, int R, int split, const __grid_constant__ MipXJobs J) {
     extern __shared__ float lines[];
@@ -243,41 +267,48 @@ k_mip_pass_x(const float* __restrict__ in, int nx, int64_t nrows, int R, int spl
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int64_t r0 = (int64_t)blockIdx.x * R; r0 < nrows; r0 += (int64_t)gridDim.x * R) {
         const int nr = (int)min((int64_t)R, nrows - r0);
-        __syncthreads();                       // the previous lines' readers are done
-        // the nr lines are nr * nx consecutive floats: eight loads per thread in flight at once
-        const float* src = in + r0 * nx;
-        const int total = nr * nx, nb = (int)blockDim.x;
-        int e = threadIdx.x;
-        for (; e + 7 * nb < total; e += 8 * nb) {
-            float v[8];
-#pragma unroll
-            for (int k = 0; k < 8; ++k) v[k] = __ldg(src + e + k * nb);
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                const int ee = e + k * nb, r = ee / nx;
-                lines[r * pitch + ee - r * nx] = v[k];
-            }
-        }
-        for (; e < total; e += nb) {
-            const int r = e / nx;
-            lines[r * pitch + e - r * nx] = __ldg(src + e);
-        }
-        __syncthreads();
-        // a task: a level, 64 lines (two per lane; fewer where R is smaller), one of `split` runs of
-        // its outputs
-        const int groups = (R + 63) / 64;
-        for (int task = warp; task < J.n * groups * split; task += kXThreads / 32) {
-            const MipXJob& b = J.j[task / (groups * split)];
-            const int g = task / split % groups, part = task % split;
+        stage_lines(in + r0 * nx, nx, nr, lines);
+        // a task: a level, the R <= 64 lines (two per lane), one of `split` runs of its outputs
+        for (int task = warp; task < J.n * split; task += kXThreads / 32) {
+            const MipXJob& b = J.j[task / split];
+            const int part = task % split;
             const int per = (b.ax + split - 1) / split;
             const int j0 = part * per, j1 = min(b.ax, j0 + per);
             if (j0 >= j1) continue;
-            const int ra = g * 64 + lane, rb = ra + 32;
+            const int ra = lane, rb = ra + 32;
             const float* la = lines + min(ra, nr - 1) * pitch;
             const float* lb = lines + min(rb, nr - 1) * pitch;
             const int64_t wa = ra < nr ? r0 + ra : -1, wb = rb < nr ? r0 + rb : -1;
             if (b.st == 1) mip_x_stream<7>(b, la, lb, nx, wa, wb, j0, j1);
             else mip_x_stream<6>(b, la, lb, nx, wa, wb, j0, j1);
+        }
+    }
+}
+
+// The same passes where the streaming form's warps would be idle or few (mip_x_streams): every (line
+// r, output j) of every level is a task of its own, dealt with r fastest, so that a warp's lanes read
+// different lines at one position (different banks).  Bound: a weight and a voxel read per tap;
+// the same taps in the same order, the same bits.
+__global__ void __launch_bounds__(kXThreads)
+k_mip_pass_x_taps(const float* __restrict__ in, int nx, int64_t nrows, int R, const __grid_constant__ MipXJobs J) {
+    extern __shared__ float lines[];
+    const int pitch = nx + 1;
+    for (int64_t r0 = (int64_t)blockIdx.x * R; r0 < nrows; r0 += (int64_t)gridDim.x * R) {
+        const int nr = (int)min((int64_t)R, nrows - r0);
+        stage_lines(in + r0 * nx, nx, nr, lines);
+        for (int k = 0; k < J.n; ++k) {
+            const MipXJob& b = J.j[k];
+            for (int task = threadIdx.x; task < R * b.ax; task += blockDim.x) {
+                const int r = task % R, j = task / R;
+                if (r >= nr) continue;
+                const float* line = lines + r * pitch;
+                const int t0 = j * b.st + b.off;
+                const int mlo = max(0, -t0), mhi = min(b.T, nx - t0);
+                float acc = 0.0f;
+#pragma unroll 4
+                for (int m = mlo; m < mhi; ++m) acc = __fadd_rn(acc, __fmul_rn(__ldg(b.w + m), line[t0 + m]));
+                b.out[(r0 + r) * b.ax + j] = acc;
+            }
         }
     }
 }
@@ -472,28 +503,29 @@ rpnn_status volume_build_levels(Ctx& c, Volume& v, const int* levels, int nlev, 
     float* A = v.mip_a.as<float>();
     float* B = v.mip_b.as<float>();
     RPNN_CUDA_TRY(cudaMemcpyAsync(dw, taps.data(), taps.size() * sizeof(float), cudaMemcpyHostToDevice, s));
+    const int64_t nrows = (int64_t)ny * nz;
     // the x passes of every level in one launch (the fine grid is read once), R lines of nx
-    // floats per block: 64 of them in at most 72 KB of shared memory, fewer for long
-    // lines; the outputs of few levels in as many runs as there are warps for them
+    // floats per block; streamed, the outputs of few levels in as many runs as there are warps for them
     constexpr int kLineBytes = 72 * 1024;
-    const int R = std::max(1, std::min(64, kLineBytes / ((nx + 1) * (int)sizeof(float))));
+    const bool stream = mip_x_streams(nx, nrows, nlev, c.num_sms);
+    const int R = mip_x_lines(nx, stream);
     const int smem = R * (nx + 1) * (int)sizeof(float);
     static bool attr = false;
     if (!attr) {
         RPNN_CUDA_TRY(cudaFuncSetAttribute(k_mip_pass_x, cudaFuncAttributeMaxDynamicSharedMemorySize, kLineBytes));
+        RPNN_CUDA_TRY(cudaFuncSetAttribute(k_mip_pass_x_taps, cudaFuncAttributeMaxDynamicSharedMemorySize, kLineBytes));
         attr = true;
     }
-    const int64_t nrows = (int64_t)ny * nz;
-    const int groups = (R + 64 - 1) / (64);
-    const int split = std::max(1, kXThreads / 32 / (nlev * groups));
+    const int split = std::max(1, kXThreads / 32 / nlev);
     MipXJobs XJ{};
     XJ.n = nlev;
     for (int k = 0; k < nlev; ++k) {
         const int l = ord[k];
-        XJ.j[k] = MipXJob{A + aoff[k], dw + xoff[k], v.dims[l][0], 1 << l, offs[k]};
+        XJ.j[k] = MipXJob{A + aoff[k], dw + (stream ? xoff[k] : toff[k]), v.dims[l][0], 1 << l, offs[k], T[k]};
     }
-    k_mip_pass_x<<<grid_for((nrows + R - 1) / R, 1, c.num_sms), kXThreads, smem, s>>>(v.raw.as<float>(), nx, nrows, R,
-                                                                                    split, XJ);
+    const int xblocks = grid_for((nrows + R - 1) / R, 1, c.num_sms);
+    if (stream) k_mip_pass_x<<<xblocks, kXThreads, smem, s>>>(v.raw.as<float>(), nx, nrows, R, split, XJ);
+    else k_mip_pass_x_taps<<<xblocks, kXThreads, smem, s>>>(v.raw.as<float>(), nx, nrows, R, XJ);
     // y passes of every level in one launch, then the z passes (with the 1/mean scale)
     for (int axis = 1; axis <= 2; ++axis) {
         MipJobs J{};

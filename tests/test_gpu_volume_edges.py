@@ -35,3 +35,26 @@ def test_stats_bricks_and_levels_equal_the_oracle(shape):
         assert np.array_equal(g.view(np.uint32), r.view(np.uint32)), lv
     o.close()
     ctx.close()
+
+
+@pytest.mark.parametrize("shape", [(80, 124, 97), (76, 129, 287), (97, 101, 288), (76, 128, 640), (76, 128, 681), (70, 139, 95)])
+def test_levels_built_together_equal_the_oracle(shape):
+    """Enough lines for the streaming x pass (9,728 up to 680 voxels) and just outside its range: the
+    levels a descriptor reads are built together, so its values are the oracle's bit for bit."""
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import oracle
+    from paper_1709_05418_gb300 import api
+    rng = np.random.default_rng(sum(shape))
+    dens = (rng.random(shape) * 40.0 * (rng.random(shape) < 0.6)).astype(np.float32)
+    ctx = api.Context()
+    v = ctx.load_volume(torch.from_numpy(dens).cuda())
+    ctx.build_mips(v)
+    x, d = W.random_queries(shape, 700, seed=3)
+    x, d, wl = x.astype(np.float32), d.astype(np.float32), np.array([0.48, -0.6, 0.64], np.float32)
+    got = ctx.extract_descriptors(v, *(torch.from_numpy(a).cuda() for a in (x, d, wl))).cpu().numpy()
+    ctx.close()
+    o = oracle.Volume(dens)
+    ref = o.descriptor(x, d, wl, f32=True)
+    o.close()
+    assert np.array_equal(got[:, :, :225].view(np.uint32), ref[:, :, :225].view(np.uint32))

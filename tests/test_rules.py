@@ -21,6 +21,8 @@ int t_group(int64_t rows, int64_t missing, int capturing, int64_t mem) { return 
 int t_grouped_runs(int64_t K, int bk) { return grouped_runs(K, bk); }
 int64_t t_slice(int64_t P) { return path_slice(P); }
 int64_t t_slice_smaller(int64_t n) { return path_slice_smaller(n); }
+int t_x_streams(int nx, int64_t rows, int levels) { return mip_x_streams(nx, rows, levels, 152); }
+int t_x_lines(int nx, int stream) { return mip_x_lines(nx, stream != 0); }
 // polls a wait makes until it gives up, or `total` if it does not; progress every `every` polls
 int64_t t_polls(uint32_t bound, int64_t total, int64_t every) {
     PollBound w{0, 0};
@@ -51,6 +53,8 @@ def rules(tmp_path_factory):
     L.t_grouped_runs.argtypes, L.t_grouped_runs.restype = [ctypes.c_int64, ctypes.c_int], ctypes.c_int
     for f in (L.t_slice, L.t_slice_smaller):
         f.argtypes, f.restype = [ctypes.c_int64], ctypes.c_int64
+    L.t_x_streams.argtypes, L.t_x_streams.restype = [ctypes.c_int, ctypes.c_int64, ctypes.c_int], ctypes.c_int
+    L.t_x_lines.argtypes, L.t_x_lines.restype = [ctypes.c_int, ctypes.c_int], ctypes.c_int
     L.t_polls.argtypes, L.t_polls.restype = [ctypes.c_uint32, ctypes.c_int64, ctypes.c_int64], ctypes.c_int64
     return L
 
@@ -133,3 +137,18 @@ def test_path_renders_list_a_bounded_slice(rules):
     src = open(os.path.join(CSRC, "capi.cu")).read()
     body = src[src.index("static rpnn_status render_impl("):]
     assert "slice = path ? path_slice(P) : P;" in body and "q_x.reserve(slice * 3" in body
+
+
+def test_x_pass_streams_only_with_its_slots_filled(rules):
+    """Long lines, single levels and small grids keep the form whose tasks fill every lane; staged
+    lines fit the shared memory the launches ask for, whatever the length."""
+    assert rules.t_x_streams(256, 256 * 256, 6) and rules.t_x_streams(96, 9728, 2)
+    for nx, rows, levels in ((768, 65536, 6), (1024, 2 ** 20, 8), (8192, 10 ** 6, 9), (256, 65536, 1), (64, 4096, 5),
+                             (256, 9727, 6)):
+        assert not rules.t_x_streams(nx, rows, levels), (nx, rows, levels)
+    for nx in range(1, 8193):
+        for stream, most in ((0, 32), (1, 64)):
+            n = rules.t_x_lines(nx, stream)
+            assert 1 <= n <= most and n * (nx + 1) * 4 <= 72 * 1024
+        if rules.t_x_streams(nx, 10 ** 6, 6):
+            assert rules.t_x_lines(nx, 1) >= 27
