@@ -37,27 +37,32 @@ __device__ __forceinline__ void stats_max_one(float x, unsigned int& mx, unsigne
 // Statistics (majorant, voxels > 0, negative / NaN / Inf) and the tracking majorants in one
 // pass.  Brick b (kBrick^3 voxels) bounds the trilinear density over its region by the largest
 // of the voxels it interpolates, 8b - 1 .. 8b + 8 per axis (zero outside the grid); max and
-// count are exact in any order.  A block takes one row of bricks: thread x reads voxel x of the
-// row's 10 x 10 lines (coalesced, a plane's ten loads in flight together), keeps the
+// count are exact in any order.  W threads take one row of bricks (brick_row_threads): thread x reads
+// voxel x of the row's 10 x 10 lines (coalesced, a plane's ten loads in flight together), keeps the
 // largest and, for the 8 x 8 lines of its own bricks, the statistics; then each brick takes
 // the largest of its ten columns.  256^3: 30 us (a thread per brick reading scattered
 // lines 55 us, and 34 us for a statistics pass of its own).
 constexpr int kBrickThreads = 256;
+template <int W>
 __global__ void __launch_bounds__(kBrickThreads)
-k_stats_bricks(const float* __restrict__ raw, int nx, int ny, int nz, int bx, int by, float* __restrict__ out,
+k_stats_bricks(const float* __restrict__ raw, int nx, int ny, int nz, int bx, int by, int rows, float* __restrict__ out,
                DevStats* st) {
-    __shared__ float col[kBrickThreads + 2 * kBrick];
-    const int yb = blockIdx.x % by, zb = blockIdx.x / by;
+    __shared__ float col[kBrickThreads];
+    const int tx = (int)threadIdx.x & (W - 1);
+    float* const c = col + ((int)threadIdx.x - tx);
+    const int row = (int)(blockIdx.x * (kBrickThreads / W) + threadIdx.x / W);
+    const bool live = W == kBrickThreads || row < rows;
+    const int yb = row % by, zb = row / by;
     const int y0 = yb * kBrick - 1, z0 = zb * kBrick - 1;
     unsigned int mx = 0, bad = 0, cnt = 0;
-    // columns in chunks of kBrickThreads - 2 voxels, whole bricks each, with a voxel of overlap
-    constexpr int kChunk = (kBrickThreads - 2) / kBrick * kBrick;
-    for (int c0 = 0; c0 < nx; c0 += kChunk) {
-        const int x = c0 - 1 + (int)threadIdx.x;
-        const bool inx = x >= 0 && x < nx;
-        const bool own = inx && x >= c0 && x < c0 + kChunk;       // counted by this chunk
+    // columns in chunks of W - 2 voxels, whole bricks each, with a voxel of overlap
+    constexpr int chunk = brick_chunk(W);
+    for (int c0 = 0; c0 < nx; c0 += chunk) {
+        const int x = c0 - 1 + tx;
+        const bool inx = live && x >= 0 && x < nx;
+        const bool own = inx && x >= c0 && x < c0 + chunk;        // counted by this chunk
         float m = 0.0f;
-        if (inx && (int)threadIdx.x < kChunk + 2) {
+        if (inx && tx < chunk + 2) {
             for (int dz = 0; dz < kBrick + 2; ++dz) {
                 const int z = z0 + dz;
                 if (z < 0 || z >= nz) continue;
@@ -75,14 +80,14 @@ k_stats_bricks(const float* __restrict__ raw, int nx, int ny, int nz, int bx, in
             }
         }
         __syncthreads();                                          // the previous chunk's readers are done
-        col[threadIdx.x] = m;
+        c[tx] = m;
         __syncthreads();
-        const int b = c0 / kBrick + (int)threadIdx.x;
-        if ((int)threadIdx.x < kChunk / kBrick && b < bx) {
+        const int b = c0 / kBrick + tx;
+        if (live && tx < chunk / kBrick && b < bx) {
             float q = 0.0f;
 #pragma unroll
-            for (int k = 0; k < kBrick + 2; ++k) q = fmaxf(q, col[kBrick * threadIdx.x + k]);
-            out[(int64_t)blockIdx.x * bx + b] = q;
+            for (int k = 0; k < kBrick + 2; ++k) q = fmaxf(q, c[kBrick * tx + k]);
+            out[(int64_t)row * bx + b] = q;
         }
     }
     unsigned long long c64 = cnt;
@@ -416,8 +421,11 @@ rpnn_status volume_stats(Ctx& c, Volume& v, cudaStream_t s) {
     for (int a = 0; a < 3; ++a) v.info.bricks[a] = v.nb[a] = (v.n[a] + kBrick - 1) / kBrick;
     st = v.bmaj.reserve((size_t)v.nb[0] * v.nb[1] * v.nb[2] * sizeof(float));
     if (st) return st;
-    k_stats_bricks<<<(unsigned)(v.nb[1] * v.nb[2]), kBrickThreads, 0, s>>>(v.raw.as<float>(), v.n[0], v.n[1], v.n[2],
-                                                                       v.nb[0], v.nb[1], v.bmaj.as<float>(), ds);
+    const int rows = v.nb[1] * v.nb[2], W = brick_row_threads(v.n[0], rows, c.num_sms), per = kBrickThreads / W;
+    auto* const kernel = W == 16 ? k_stats_bricks<16> : W == 32 ? k_stats_bricks<32> : W == 64 ? k_stats_bricks<64>
+                         : W == 128 ? k_stats_bricks<128> : k_stats_bricks<256>;
+    kernel<<<(unsigned)((rows + per - 1) / per), kBrickThreads, 0, s>>>(v.raw.as<float>(), v.n[0], v.n[1], v.n[2],
+                                                                      v.nb[0], v.nb[1], rows, v.bmaj.as<float>(), ds);
     RPNN_CHECK_LAUNCH();
     const int64_t gs = (n / 16 + 255) / 256;
     k_stats_sum<<<(int)std::max<int64_t>(1, std::min<int64_t>(gs, (int64_t)c.num_sms * 8)), 256, 0, s>>>(v.raw.as<float>(),

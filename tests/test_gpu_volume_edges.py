@@ -58,3 +58,28 @@ def test_levels_built_together_equal_the_oracle(shape):
     ref = o.descriptor(x, d, wl, f32=True)
     o.close()
     assert np.array_equal(got[:, :, :225].view(np.uint32), ref[:, :, :225].view(np.uint32))
+
+
+@pytest.mark.parametrize("shape", [(300, 270, 8), (290, 290, 9), (283, 290, 24), (298, 280, 25), (281, 290, 56), (290, 281, 57),
+                                   (280, 281, 120), (281, 290, 121), (1200, 130, 1), (40, 129, 9)])
+def test_bricks_of_short_lines_equal_the_oracle(shape):
+    """Lines at the edges of the widths that 16 to 256 threads read, more rows of bricks than a wave (and
+    fewer), rows that do not fill a block."""
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import oracle
+    from paper_1709_05418_gb300 import api
+    rng = np.random.default_rng(sum(shape))
+    dens = (rng.random(shape) * 40.0 * (rng.random(shape) < 0.3)).astype(np.float32)
+    dens.flat[-1] = 41.0
+    ctx = api.Context()
+    v = ctx.load_volume(torch.from_numpy(dens).cuda())
+    ctx.build_mips(v)
+    gi = ctx.get_volume_info(v)
+    o = oracle.Volume(dens)
+    oi = o.stats()
+    for key in ("mean", "majorant", "nonzero"):
+        assert gi[key] == oi[key], key
+    assert np.array_equal(ctx.copy_brick_majorants(v).cpu().numpy(), o.brick_majorants())
+    o.close()
+    ctx.close()

@@ -23,6 +23,8 @@ int64_t t_slice(int64_t P) { return path_slice(P); }
 int64_t t_slice_smaller(int64_t n) { return path_slice_smaller(n); }
 int t_x_streams(int nx, int64_t rows, int levels) { return mip_x_streams(nx, rows, levels, 152); }
 int t_x_lines(int nx, int stream) { return mip_x_lines(nx, stream != 0); }
+int t_row_threads(int nx, int64_t rows) { return brick_row_threads(nx, rows, 152); }
+int t_brick_chunk(int w) { return brick_chunk(w); }
 // polls a wait makes until it gives up, or `total` if it does not; progress every `every` polls
 int64_t t_polls(uint32_t bound, int64_t total, int64_t every) {
     PollBound w{0, 0};
@@ -55,6 +57,8 @@ def rules(tmp_path_factory):
         f.argtypes, f.restype = [ctypes.c_int64], ctypes.c_int64
     L.t_x_streams.argtypes, L.t_x_streams.restype = [ctypes.c_int, ctypes.c_int64, ctypes.c_int], ctypes.c_int
     L.t_x_lines.argtypes, L.t_x_lines.restype = [ctypes.c_int, ctypes.c_int], ctypes.c_int
+    L.t_row_threads.argtypes, L.t_row_threads.restype = [ctypes.c_int, ctypes.c_int64], ctypes.c_int
+    L.t_brick_chunk.argtypes, L.t_brick_chunk.restype = [ctypes.c_int], ctypes.c_int
     L.t_polls.argtypes, L.t_polls.restype = [ctypes.c_uint32, ctypes.c_int64, ctypes.c_int64], ctypes.c_int64
     return L
 
@@ -152,3 +156,19 @@ def test_x_pass_streams_only_with_its_slots_filled(rules):
             assert 1 <= n <= most and n * (nx + 1) * 4 <= 72 * 1024
         if rules.t_x_streams(nx, 10 ** 6, 6):
             assert rules.t_x_lines(nx, 1) >= 27
+
+
+def test_brick_rows_take_no_more_threads_than_they_need(rules):
+    """Whole bricks a pass, each with its two neighbours inside the row's threads; where there are many
+    rows, short lines share a block (1 voxel: 16 rows of it)."""
+    many = 65536
+    for nx in range(1, 8193):
+        w = rules.t_row_threads(nx, many)
+        c = rules.t_brick_chunk(w)
+        assert w in (16, 32, 64, 128, 256) and c % 8 == 0 and 8 <= c <= w - 2
+        assert c >= nx or w == 256
+        assert w == 16 or rules.t_brick_chunk(w // 2) < nx
+        # a brick's last column, read from the row's own part of the shared buffer
+        assert 8 * (c // 8 - 1) + 9 < w
+        assert rules.t_row_threads(nx, 8 * 152) == 256
+    assert rules.t_row_threads(1, many) == 16 and rules.t_row_threads(249, many) == 256
