@@ -39,7 +39,8 @@ template <> __device__ __forceinline__ __nv_bfloat16 cvt_out<__nv_bfloat16>(floa
 // buffer, FP32 rows five levels at a time, and written with 16-byte stores.  Bound: one L1
 // wavefront per lookup inside the grid (a lane's 32-byte record is its own cache line; 73 % of
 // the L1 peak).  30,011 FP32 rows: 116 us (132 with each value stored directly, 25
-// consecutive ones per level and z-slice).
+// consecutive ones per level and z-slice).  Blended FP32 rows are stored directly: their two lookups
+// per value leave the stores room, and staging costs more than it saves (100,000 rows 620 us, 580 so).
 //
 // BATCH: the shading points of up to RPNN_MAX_BATCH renders, compacted: point j belongs
 // to the item i with off[i] <= j < off[i+1], reads its position and direction at
@@ -55,9 +56,10 @@ k_descriptor(const VolumeView v, const float* __restrict__ xs, const float* __re
     // row stride per level: 240 values (FP32, BF16) or 256 (E4M3: whole 32-byte K-steps)
     constexpr int DS = sizeof(OutT) == 1 ? 256 : RPNN_DESC_STRIDE;
     constexpr int ROW = RPNN_K * DS;
-    constexpr int PASSES = sizeof(OutT) == 4 ? 2 : 1, LEVELS = RPNN_K / PASSES;   // levels staged at a time
+    constexpr bool STAGE = !(BLEND && sizeof(OutT) == 4);
+    constexpr int PASSES = STAGE && sizeof(OutT) == 4 ? 2 : 1, LEVELS = RPNN_K / PASSES;   // levels staged at a time
     constexpr int NI = BATCH ? RPNN_MAX_BATCH : 1;
-    __shared__ __align__(16) OutT rowbuf[8][LEVELS * DS];
+    __shared__ __align__(16) OutT rowbuf[STAGE ? 8 : 1][STAGE ? LEVELS * DS : 8];
     __shared__ LevelK lk[NI][RPNN_K];
     __shared__ LevelB lb[BLEND ? NI : 1][RPNN_K];
     __shared__ int s_off[NI + 1];
@@ -101,8 +103,8 @@ k_descriptor(const VolumeView v, const float* __restrict__ xs, const float* __re
         const Frame F = make_frame(d, wl);
         const LevelK* lki = lk[it];
         const LevelB* lbi = lb[BLEND ? it : 0];
-        OutT* row = rowbuf[warp];
-        uint4* srow = reinterpret_cast<uint4*>(row);
+        OutT* row = STAGE ? rowbuf[warp] : out + qi * (int64_t)ROW;
+        const uint4* srow = reinterpret_cast<const uint4*>(row);
         constexpr int VEC = LEVELS * DS * (int)sizeof(OutT) / 16;
         for (int pass = 0; pass < PASSES; ++pass) {
             for (int task = lane; task < LEVELS * 25; task += 32) {
@@ -154,6 +156,7 @@ k_descriptor(const VolumeView v, const float* __restrict__ xs, const float* __re
                 const int kk = e / (DS - RPNN_S), j = e % (DS - RPNN_S);
                 row[kk * DS + RPNN_S + j] = cvt_out<OutT>(j == 0 ? F.gamma : 0.0f);
             }
+            if (!STAGE) continue;
             __syncwarp();
             uint4* gdst = reinterpret_cast<uint4*>(out + qi * (int64_t)ROW + pass * LEVELS * DS);
             for (int e = lane; e < VEC; e += 32) gdst[e] = srow[e];
