@@ -304,12 +304,13 @@ k_paths(const VolumeView v, const RenderArgs a, const float* __restrict__ qx, co
 // Training records (Sec. 5.1).  k_record_start, one thread per record, samples it: direction,
 // origin on the bounding sphere's cross-section, free flight by delta tracking with retries,
 // light direction (npaths = -1: no collision found in kRecordAttempts tries).
-__global__ void __launch_bounds__(32)
+__global__ void __launch_bounds__(128)
 k_record_start(const VolumeView v, int64_t first, int64_t n, uint64_t seed, float* __restrict__ xo,
                float* __restrict__ dout, float* __restrict__ wlo, float* __restrict__ label,
-               int* __restrict__ npaths, uint32_t* status) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
+               int* __restrict__ npaths, uint32_t* status, int lanes) {
+    const int lane = (int)threadIdx.x & 31;
+    const int64_t i = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * lanes + lane;
+    if (i >= n || lane >= lanes) return;
     const uint32_t rec = (uint32_t)(first + i);
     float3 x = f3(0.f, 0.f, 0.f), d = f3(0.f, 0.f, 1.f);
     int found = 0;
@@ -371,7 +372,7 @@ struct LabelPaths {
     uint64_t seed;
     uint32_t rec;
     float rel_ci;
-    int n_min, n_max;
+    int n_min, n_max, lanes;     // lanes of a warp that take paths
     uint32_t* status;
     int j;                       // this lane's path, -1: none
     KahanF S, Q;                 // warp 0: running sums of L and L^2
@@ -419,7 +420,7 @@ struct LabelPaths {
         const int lane = threadIdx.x & 31;
         volatile RecordRing& vr = r;
         if (threadIdx.x < 32 && !vr.done) rounds();
-        const bool claim = want && j < 0;
+        const bool claim = want && j < 0 && lane < lanes;
         const unsigned m = __ballot_sync(0xffffffffu, claim);
         int first = 0;
         if (m && lane == __ffs(m) - 1) first = atomicAdd(&r.next, __popc(m));
@@ -428,7 +429,7 @@ struct LabelPaths {
             j = first + __popc(m & ((1u << lane) - 1u));
             if (j < 0) j = 0x7fffffff;             // beyond the last path index
         }
-        if (!want || j >= n_max) return -1;
+        if (!want || j < 0 || j >= n_max) return -1;
         const int base = vr.base;
         __threadfence_block();
         if (j - base >= kRing) return 0;
@@ -466,7 +467,7 @@ struct LabelPaths {
 // (a warp per record in nested loops: 43 ms).
 __global__ void __launch_bounds__(128, 7)
 k_records(const VolumeView v, int64_t first, int64_t n, uint64_t seed, float rel_ci, int n_min,
-          int n_max, const float* __restrict__ xo, const float* __restrict__ dout, const float* __restrict__ wlo,
+          int n_max, int lanes, const float* __restrict__ xo, const float* __restrict__ dout, const float* __restrict__ wlo,
           float* __restrict__ label, int* __restrict__ npaths, uint32_t* status) {
     __shared__ RecordRing ring;
     for (int64_t i = blockIdx.x; i < n; i += gridDim.x) {
@@ -480,7 +481,7 @@ k_records(const VolumeView v, int64_t first, int64_t n, uint64_t seed, float rel
         if (threadIdx.x < 4) ring.wait[threadIdx.x] = PollBound{0, 0};
         __syncthreads();
         LabelPaths src{ring, f3(xo[3 * i], xo[3 * i + 1], xo[3 * i + 2]), f3(dout[3 * i], dout[3 * i + 1], dout[3 * i + 2]),
-                       seed, (uint32_t)(first + i), rel_ci, n_min, n_max, status, -1, KahanF(), KahanF(), 0.0f, 0};
+                       seed, (uint32_t)(first + i), rel_ci, n_min, n_max, lanes, status, -1, KahanF(), KahanF(), 0.0f, 0};
         trace_paths(v, f3(wlo[3 * i], wlo[3 * i + 1], wlo[3 * i + 2]), 1.0f, src);
         __syncthreads();                           // every warp has left the ring
         if (threadIdx.x == 0) {
@@ -662,16 +663,15 @@ rpnn_status launch_chunk_counts(Ctx& c, const int* count, int64_t rows, int n, i
 rpnn_status launch_records(Ctx& c, const VolumeView& vv, int64_t first, int64_t n, uint64_t seed,
                            float rel_ci, int n_min, int n_max, float* x, float* d, float* wl,
                            float* label, int* npaths, cudaStream_t s) {
-    k_record_start<<<(unsigned)((n + 31) / 32), 32, 0, s>>>(vv, first, n, seed, x, d, wl, label, npaths,
-                                                            c.status.as<uint32_t>());
+    const int start = record_start_lanes(n, c.num_sms);
+    k_record_start<<<(unsigned)((n + 4 * start - 1) / (4 * start)), 128, 0, s>>>(vv, first, n, seed, x, d, wl, label, npaths,
+                                                                                c.status.as<uint32_t>(), start);
     RPNN_CHECK_LAUNCH();
-    // a block per record (grid-stride beyond the grid limit); the fewer the records, the more
-    // warps each, so that the chip stays full until the last ones end (4,096 records: 12.9 ms
-    // with one warp each, 12.0 with two; 1,024: 5.8 with two, 4.4 with four)
-    const int64_t want = (int64_t)c.num_sms * 64;
-    const int warps = n >= want ? 1 : (n * 2 >= want ? 2 : 4);
+    // a block per record (grid-stride beyond the grid limit)
+    const int warps = record_warps(n, n_max, c.num_sms);
     k_records<<<(unsigned)std::min<int64_t>(n, 1 << 30), 32 * warps, 0, s>>>(
-        vv, first, n, seed, rel_ci, n_min, n_max, x, d, wl, label, npaths, c.status.as<uint32_t>());
+        vv, first, n, seed, rel_ci, n_min, n_max, record_lanes(n_max, warps), x, d, wl, label, npaths,
+        c.status.as<uint32_t>());
     RPNN_CHECK_LAUNCH();
     return RPNN_OK;
 }

@@ -96,4 +96,28 @@ RPNN_RULE int brick_row_threads(int nx, int64_t rows, int sms) {
     return w;
 }
 
+// Training records: how many of them one warp starts (each a delta track with retries, so lanes
+// of a warp wait for one another): one while the chip holds a warp for each.
+RPNN_RULE int record_start_lanes(int64_t n, int sms) {
+    int lanes = 1;
+    while (lanes < 32 && lanes * 64 * (int64_t)sms < n) lanes *= 2;
+    return lanes;
+}
+// Warps that share a record's paths: the fewer the records, the more, so that the chip stays full until
+// the last ones end (4,096 records: 12.9 ms with one each, 12.0 with two; 1,024: 5.8 with two,
+// 4.4 with four); but where the chip is full (28 warps an SM) none that would have fewer than 16
+// paths (4,000 records of 32 paths: 6.0 ms with four warps each, 3.5 with one).
+RPNN_RULE int record_warps(int64_t n, int n_max, int sms) {
+    const int64_t want = (int64_t)sms * 64;
+    int warps = n >= want ? 1 : (n * 2 >= want ? 2 : 4);
+    while (4 * n > 28 * (int64_t)sms && warps > 1 && 16 * warps >= n_max) warps /= 2;
+    return warps;
+}
+// ... and the lanes of each that take paths: the first warp to ask would leave none for the others
+// where the paths are few (152 records of 32 paths: 2.1 ms on one warp, 1.4 on eight lanes of four).
+RPNN_RULE int record_lanes(int n_max, int warps) {
+    const int64_t l = ((int64_t)n_max + warps - 1) / warps;
+    return l < 32 ? (int)l : 32;
+}
+
 }  // namespace rpnn

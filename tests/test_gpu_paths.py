@@ -93,3 +93,18 @@ def test_path_image_of_several_slices(env):
     tol = 1e-3 * np.maximum(np.abs(ref), 1e-3 * np.abs(ref).max()) + 1e-7
     assert (np.abs(got[pix] - ref) <= tol)[lit].mean() >= 0.9
     assert np.abs(got[pix][lit] / ref[lit] - 1.0).mean() <= 0.1
+
+
+@pytest.mark.parametrize("n_max", [1, 3, 30, 64, 100])
+def test_few_paths_give_the_same_labels_however_they_are_spread(env, n_max):
+    """8 lanes of four warps, all lanes of one, a start per warp or several: a record's values do not show it."""
+    _, ctx, vol, _, _ = env
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    n = 66 * sms
+    every = [t.cpu() for t in ctx.gen_records(vol, 5, n, 78, rel_ci=1e-7, n_min=1, n_max=n_max)]
+    for off, m in ((7, 1), (100, 7 * sms), (40, 7 * sms + 1), (9, 33 * sms)):
+        part = [t.cpu() for t in ctx.gen_records(vol, 5 + off, m, 78, rel_ci=1e-7, n_min=1, n_max=n_max)]
+        for a, b in zip(every, part):
+            assert torch.equal(a[off:off + m], b), (off, m)
+    ctx.sync_status()
+    assert int(every[4].max()) == n_max

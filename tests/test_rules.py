@@ -25,6 +25,9 @@ int t_x_streams(int nx, int64_t rows, int levels) { return mip_x_streams(nx, row
 int t_x_lines(int nx, int stream) { return mip_x_lines(nx, stream != 0); }
 int t_row_threads(int nx, int64_t rows) { return brick_row_threads(nx, rows, 152); }
 int t_brick_chunk(int w) { return brick_chunk(w); }
+int t_start_lanes(int64_t n) { return record_start_lanes(n, 152); }
+int t_warps(int64_t n, int n_max) { return record_warps(n, n_max, 152); }
+int t_lanes(int n_max, int warps) { return record_lanes(n_max, warps); }
 // polls a wait makes until it gives up, or `total` if it does not; progress every `every` polls
 int64_t t_polls(uint32_t bound, int64_t total, int64_t every) {
     PollBound w{0, 0};
@@ -59,6 +62,9 @@ def rules(tmp_path_factory):
     L.t_x_lines.argtypes, L.t_x_lines.restype = [ctypes.c_int, ctypes.c_int], ctypes.c_int
     L.t_row_threads.argtypes, L.t_row_threads.restype = [ctypes.c_int, ctypes.c_int64], ctypes.c_int
     L.t_brick_chunk.argtypes, L.t_brick_chunk.restype = [ctypes.c_int], ctypes.c_int
+    L.t_start_lanes.argtypes, L.t_start_lanes.restype = [ctypes.c_int64], ctypes.c_int
+    L.t_warps.argtypes, L.t_warps.restype = [ctypes.c_int64, ctypes.c_int], ctypes.c_int
+    L.t_lanes.argtypes, L.t_lanes.restype = [ctypes.c_int, ctypes.c_int], ctypes.c_int
     L.t_polls.argtypes, L.t_polls.restype = [ctypes.c_uint32, ctypes.c_int64, ctypes.c_int64], ctypes.c_int64
     return L
 
@@ -172,3 +178,23 @@ def test_brick_rows_take_no_more_threads_than_they_need(rules):
         assert 8 * (c // 8 - 1) + 9 < w
         assert rules.t_row_threads(nx, 8 * 152) == 256
     assert rules.t_row_threads(1, many) == 16 and rules.t_row_threads(249, many) == 256
+
+
+def test_few_paths_are_spread_over_a_records_warps(rules):
+    """Every warp that a record gets has paths to trace, few records start a warp each, and all paths
+    and records are reached whatever their number."""
+    for n in (1, 152, 1064, 1065, 4863, 4864, 9727, 9728, 9729, 2 ** 32):
+        lanes = rules.t_start_lanes(n)
+        assert lanes in (1, 2, 4, 8, 16, 32) and (lanes == 1) == (n <= 9728)
+        assert (n + 4 * lanes - 1) // (4 * lanes) <= 2 ** 31 - 1
+        for n_max in (1, 2, 16, 31, 32, 33, 64, 65, 127, 128, 1024, 2 ** 31 - 1):
+            warps = rules.t_warps(n, n_max)
+            per = rules.t_lanes(n_max, warps)
+            assert warps in (1, 2, 4) and 1 <= per <= 32
+            assert per * warps >= min(n_max, 32 * warps)
+            if n > 1064 and warps > 1:
+                assert n_max > 16 * warps
+            if n_max > 64:
+                assert warps == (1 if n >= 9728 else 2 if n >= 4864 else 4)
+            if n_max >= 128:
+                assert per == 32
