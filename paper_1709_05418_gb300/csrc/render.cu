@@ -74,10 +74,10 @@ k_primary(const VolumeView v_, const RenderArgs a_, int64_t P_, float* __restric
     const VolumeView& v = BATCH ? it.v : v_;
     const RenderArgs& a = BATCH ? it.a : a_;
     const int64_t P = BATCH ? it.P : P_;
-    const int wl = (int)threadIdx.x & 31;
+    const int warp_lane = (int)threadIdx.x & 31;
     const int64_t ps = BATCH ? (blockIdx.x - it.first_block) * (int64_t)blockDim.x + threadIdx.x
-                             : first + ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * lanes + wl;
-    const bool active = ps < P && (BATCH || wl < lanes);
+                             : first + ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * lanes + warp_lane;
+    const bool active = ps < P && (BATCH || warp_lane < lanes);
     int hit = 0;
     float3 x = f3(0.f, 0.f, 0.f), d = f3(0.f, 0.f, 1.f);
     float Ld = 0.0f;
