@@ -39,13 +39,13 @@ L2_FLUSH_BYTES = 256 << 20
 # summaries under profiles/ give the commands), with the SHA-256 prefixes of the sources the
 # captured build was compiled from.  A kernel whose sources changed since reports null.
 NCU_TRAFFIC = {
-    "descriptor": {"bytes_per_query": (795.742208e6 + 5.595392e6) / 178675,
-                   "sources": {"descriptor.cu": "3eeba11fdbbab198", "desc_lookup.cuh": "96d43ff4040f8e82",
+    "descriptor": {"bytes_per_query": (795.734528e6 + 5.623552e6) / 178675,
+                   "sources": {"descriptor.cu": "c2146dc776fc83e1", "desc_lookup.cuh": "96d43ff4040f8e82",
                                "volume.cu:k_pack": "375ff27268e0095e"}},
-    "network": {"bytes_per_query": (884.246528e6 + 0.669696e6) / 178675,
+    "network": {"bytes_per_query": (884.785152e6 + 3.582720e6) / 178675,
                 "sources": {"mlp_tc.cu": "fb9da248a167cbcd", "tc_ptx.cuh": "294268ada12e7cd2",
                             "tc_net.cuh": "84cfe3d7ca7bea66"}},
-    "network_fp8": {"bytes_per_query": (460.915200e6 + 1.886720e6) / 178675,
+    "network_fp8": {"bytes_per_query": (460.871936e6 + 1.793792e6) / 178675,
                     "sources": {"mlp_tc.cu": "fb9da248a167cbcd", "tc_ptx.cuh": "294268ada12e7cd2",
                                 "tc_net.cuh": "84cfe3d7ca7bea66"}},
 }

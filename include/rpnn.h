@@ -269,7 +269,8 @@ rpnn_status rpnn_render_env(rpnn_ctx* ctx, int32_t vol, const rpnn_render_desc* 
 /* Memory budget of rpnn_render (no counterpart in the paper): the descriptor and network
  * stages run over chunks of at most `rows` shading points (0 = the default 1,048,576
  * rows, i.e. 5 GB of BF16 descriptors; otherwise at least 128).  Results do not depend on
- * the chunking.  Errors: RPNN_ERR_ARG for 0 < rows < 128 or rows < 0. */
+ * the chunking.  (Path mode lists its shading points, 28 bytes each, for at most 2^24 samples at
+ * a time, fewer where that does not fit.)  Errors: RPNN_ERR_ARG for 0 < rows < 128 or rows < 0. */
 rpnn_status rpnn_set_render_chunk(rpnn_ctx* ctx, int64_t rows);
 /* Fused descriptor + network stages (off by default; Sec. 4.2 and 4.3 in one kernel, no
  * counterpart in the paper, which names descriptor construction as the bottleneck in
