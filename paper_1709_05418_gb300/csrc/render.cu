@@ -41,16 +41,19 @@ struct PrimaryItem {
 // RPNN_MAX_BATCH renders (items[i] from block first_block on); each block copies its item
 // into shared memory and works on that render's samples, writing into its region of the
 // per-sample buffers and appending its shading points to that region with its own count.
-// Not BATCH: samples first .. P - 1.  `lanes` (not BATCH): samples per warp.  A warp's rays diverge, so where the image has fewer
-// samples than the chip holds threads, fewer of them share a warp (64 x 64 samples, this pass alone: 118 us
-// with 32 per warp, 94 with 4, about 80 with 2).
-template <bool BATCH>
-__global__ void __launch_bounds__(128, BATCH ? 5 : 6)
+// PART: samples first .. P - 1, `lanes` of them per warp.  A warp's rays diverge, so where the image has
+// fewer samples than the chip holds threads, fewer of them share a warp (64 x 64 samples, this pass alone:
+// 118 us with 32 per warp, 94 with 4, about 80 with 2).  An instance of its own: with the two numbers as
+// arguments whole images of whole warps took 1 to 3 % longer (256 x 256 in a dense cloud 680 us, 658 without).
+enum PrimaryForm { kWhole, kPart, kBatched };
+template <PrimaryForm FORM>
+__global__ void __launch_bounds__(128, FORM == kBatched ? 5 : 6)
 k_primary(const VolumeView v_, const RenderArgs a_, int64_t P_, float* __restrict__ sample_val,
           float* __restrict__ qx, float* __restrict__ qd, uint32_t* __restrict__ qps,
           int* __restrict__ qcount, int* __restrict__ hit_out, float* __restrict__ x_out,
           float* __restrict__ d_out, float* __restrict__ Ld_out, uint32_t* status,
           const PrimaryItem* __restrict__ items, int n_items, int lanes, int64_t first) {
+    constexpr bool BATCH = FORM == kBatched;
     __shared__ __align__(16) PrimaryItem it;
     __shared__ int s_item;
     if (BATCH) {
@@ -75,9 +78,9 @@ k_primary(const VolumeView v_, const RenderArgs a_, int64_t P_, float* __restric
     const RenderArgs& a = BATCH ? it.a : a_;
     const int64_t P = BATCH ? it.P : P_;
     const int warp_lane = (int)threadIdx.x & 31;
-    const int64_t ps = BATCH ? (blockIdx.x - it.first_block) * (int64_t)blockDim.x + threadIdx.x
-                             : first + ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * lanes + warp_lane;
-    const bool active = ps < P && (BATCH || warp_lane < lanes);
+    const int64_t ps = FORM == kPart ? first + ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * lanes + warp_lane
+                                     : (blockIdx.x - (BATCH ? it.first_block : 0)) * (int64_t)blockDim.x + threadIdx.x;
+    const bool active = ps < P && (FORM != kPart || warp_lane < lanes);
     int hit = 0;
     float3 x = f3(0.f, 0.f, 0.f), d = f3(0.f, 0.f, 1.f);
     float Ld = 0.0f;
@@ -543,7 +546,7 @@ void batch_tables(const Ctx& c, const rpnn_batch_item* items, int n, const std::
 rpnn_status launch_primary_batch(Ctx& c, const void* tables, int n, int64_t blocks, float* sample_val, float* qx,
                                  float* qd, uint32_t* qps, int* qcount, cudaStream_t s) {
     const PrimaryItem* pi = static_cast<const PrimaryItem*>(tables);
-    k_primary<true><<<(unsigned)blocks, 128, 0, s>>>(VolumeView{}, RenderArgs{}, 0, sample_val, qx, qd, qps, qcount,
+    k_primary<kBatched><<<(unsigned)blocks, 128, 0, s>>>(VolumeView{}, RenderArgs{}, 0, sample_val, qx, qd, qps, qcount,
                                                      nullptr, nullptr, nullptr, nullptr, c.status.as<uint32_t>(), pi,
                                                      n, 32, 0);
     RPNN_CHECK_LAUNCH();
@@ -573,7 +576,8 @@ rpnn_status launch_primary(Ctx& c, const VolumeView& vv, const rpnn_render_desc&
     int lanes = 2;
     while (lanes < 32 && (int64_t)lanes * c.num_sms * 20 < P) lanes *= 2;
     const int64_t blocks = (P + 4 * lanes - 1) / (4 * lanes);
-    k_primary<false><<<(unsigned)blocks, 128, 0, s>>>(vv, make_args(rd), first + P, sample_val, qx, qd, qps, qcount, hit,
+    auto* const kernel = lanes == 32 && first == 0 ? k_primary<kWhole> : k_primary<kPart>;
+    kernel<<<(unsigned)blocks, 128, 0, s>>>(vv, make_args(rd), first + P, sample_val, qx, qd, qps, qcount, hit,
                                                       xo, dout, Ld, c.status.as<uint32_t>(), nullptr, 0, lanes, first);
     RPNN_CHECK_LAUNCH();
     return RPNN_OK;
