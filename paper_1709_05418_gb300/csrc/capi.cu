@@ -449,7 +449,11 @@ static rpnn_status render_impl(Ctx* c, int32_t vol, const rpnn_render_desc* desc
     rpnn_render_desc rd0 = *desc;                   // the primary pass carries light 0
     for (int a = 0; a < 3; ++a) rd0.light_dir[a] = lights[a];
     rd0.light_E = lights[3 * nl];
-    const bool path = desc->mode == RPNN_MODE_PATH;
+    const VolumeView vv = v->view();
+    const bool in_primary = desc->mode == RPNN_MODE_PATH &&
+                            path_in_primary((int64_t)desc->width * desc->height * desc->spp, vv.albedo_c,
+                                            vv.majorant * vv.dscale, c->num_sms);
+    const bool path = desc->mode == RPNN_MODE_PATH && !in_primary;     // paths are a launch of their own
     const bool queries = net || path || nl > 1;     // shading points are listed for the network, paths or extra lights
     const int64_t P = (int64_t)desc->width * desc->height * desc->spp;
     const bool f32 = desc->precision == RPNN_F32;
@@ -481,7 +485,6 @@ static rpnn_status render_impl(Ctx* c, int32_t vol, const rpnn_render_desc* desc
         if (!st) st = ensure_rows(c, CH, f32);
     }
     if (st) return st;
-    const VolumeView vv = v->view();
     int* qc = c->q_count.as<int>();
     cudaEvent_t* ev = nullptr;
     if (c->profiling) {
@@ -503,6 +506,11 @@ static rpnn_status render_impl(Ctx* c, int32_t vol, const rpnn_render_desc* desc
     for (int64_t first = 0; first < P; first += slice) {
         NvtxRange stage("primary");
         RPNN_CUDA_TRY(cudaMemsetAsync(qc, 0, 2 * sizeof(int), s));
+        if (in_primary) {
+            st = launch_primary_paths(*c, vv, rd0, c->sample_val.as<float>(), s);
+            if (st) return st;
+            break;
+        }
         st = launch_primary(*c, vv, rd0, c->sample_val.as<float>(), queries ? c->q_x.as<float>() : nullptr,
                             queries ? c->q_d.as<float>() : nullptr, queries ? c->q_ps.as<uint32_t>() : nullptr,
                             queries ? qc : nullptr, nullptr, nullptr, nullptr, nullptr, s, first,

@@ -293,6 +293,9 @@ rpnn_status launch_scatter_composite(Ctx& c, const rpnn_render_desc& rd, float a
                                      float* sample_val, float* image, bool with_g,
                                      cudaStream_t s, const int* g_off = nullptr,
                                      const int* g_total = nullptr);
+// Path mode in one pass: sample = albedo (L_d + L_i), the path traced by its own lane.
+rpnn_status launch_primary_paths(Ctx& c, const VolumeView& vv, const rpnn_render_desc& rd, float* sample_val,
+                                 cudaStream_t s);
 // Path mode: adds the path-traced L_i of the *qcount shading points to their samples (which hold
 // L_d) and multiplies by the albedo; *next: the work counter, zero before the launch.
 rpnn_status launch_paths(Ctx& c, const VolumeView& vv, const rpnn_render_desc& rd, const float* qx, const float* qd,

@@ -172,4 +172,62 @@ __device__ __forceinline__ void trace_paths(const VolumeView& v, const float3 wl
     }
 }
 
+// One path by itself, in nested loops: the same draws and the same rounding sequence as trace_paths,
+// so the same estimate.  For a lane of the primary pass, where paths are so short that listing
+// them for a second launch costs more than its shared steps save (path_in_primary).
+__device__ __forceinline__ float trace_path(const VolumeView& v, float3 x, float3 d, const float3 wl, const float E,
+                                            const Rng& rng, bool& capped) {
+    const float maj_s = v.majorant * v.dscale;
+    uint32_t ctr = 0;
+    float L = 0.0f;
+    for (int b = 0; b < kBounceCap; ++b) {
+        float4 xi = rng.draw(ctr++);
+        d = phase_sample(v, b == 0 ? v.lm : v.lmc, d, xi.x, xi.y);
+        float t, t1;
+        if (!(v.majorant > 0.0f) || !box_clip(v.ext, x, d, t, t1)) return L;
+        for (uint32_t n = 0;;) {
+            xi = rng.draw(ctr++);
+            t -= logf(1.0f - xi.x) / maj_s;
+            if (!(t < t1)) return L;
+            const float3 p = f3(__fmaf_rn(t, d.x, x.x), __fmaf_rn(t, d.y, x.y), __fmaf_rn(t, d.z, x.z));
+            if (xi.y * v.majorant < raw_density(v, p)) { x = p; break; }
+            if (++n >= v.track_cap) { capped = true; return L; }
+        }
+        xi = rng.draw(ctr++);
+        if (!(xi.x < v.albedo_c)) return L;
+        // next-event estimate: ratio tracking towards the light
+        float T = 1.0f;
+        if (box_clip(v.ext, x, wl, t, t1)) {
+            BrickWalk w;
+            walk_init(v, x, wl, t, w);
+            float tau = -1.0f;
+            for (uint32_t n = 0;;) {
+                const float te = walk_exit(w, t1), mu_b = walk_majorant(v, w);
+                if (mu_b > 0.0f) {
+                    if (tau < 0.0f) tau = -logf(1.0f - rng.draw(ctr++).x);
+                    const float mu_s = mu_b * v.dscale;
+                    const float seg = __fmul_rn(mu_s, __fsub_rn(te, t));
+                    if (tau < seg) {
+                        t += tau / mu_s;
+                        const float3 p = f3(__fmaf_rn(t, wl.x, x.x), __fmaf_rn(t, wl.y, x.y), __fmaf_rn(t, wl.z, x.z));
+                        T *= 1.0f - raw_density(v, p) / mu_b;
+                        tau = -1.0f;
+                        if (++n >= v.track_cap) { capped = true; break; }
+                        continue;
+                    }
+                    tau = __fsub_rn(tau, seg);
+                }
+                if (te >= t1) break;
+                t = te;
+                if (!walk_step(v, w)) break;
+                if (++n >= v.track_cap) { capped = true; break; }
+            }
+        }
+        const float ct = __fmaf_rn(d.z, wl.z, __fmaf_rn(d.x, wl.x, __fmul_rn(d.y, wl.y)));
+        L = __fmaf_rn(__fmul_rn(E, phase_eval(v, v.lmc, ct)), T, L);
+    }
+    capped = true;
+    return L;
+}
+
 }  // namespace rpnn

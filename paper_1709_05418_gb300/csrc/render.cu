@@ -5,7 +5,8 @@
 // tracking to the first real collision (the visible point), next-event estimation of
 // the direct in-scattering with a ratio-tracked shadow ray, and an appended shading query
 // for the descriptor + network stages (RPNN mode) or for k_paths, which adds a path-traced
-// estimate of the indirect part (path mode).  Queries are compacted with one atomic per
+// estimate of the indirect part (path mode).  Short paths of middle-sized images are traced
+// here (kWithPaths).  Queries are compacted with one atomic per
 // warp so the list stays in pixel order within a warp.
 #include <vector>
 
@@ -45,7 +46,7 @@ struct PrimaryItem {
 // fewer samples than the chip holds threads, fewer of them share a warp (64 x 64 samples, this pass alone:
 // 118 us with 32 per warp, 94 with 4, about 80 with 2).  An instance of its own: with the two numbers as
 // arguments whole images of whole warps took 1 to 3 % longer (256 x 256 in a dense cloud 680 us, 658 without).
-enum PrimaryForm { kWhole, kPart, kBatched };
+enum PrimaryForm { kWhole, kPart, kBatched, kWithPaths };
 template <PrimaryForm FORM>
 __global__ void __launch_bounds__(128, FORM == kBatched ? 5 : 6)
 k_primary(const VolumeView v_, const RenderArgs a_, int64_t P_, float* __restrict__ sample_val,
@@ -104,8 +105,9 @@ k_primary(const VolumeView v_, const RenderArgs a_, int64_t P_, float* __restric
             const float3 wl = f3(a.wl[0], a.wl[1], a.wl[2]);
             uint32_t c2 = 0;
             Ld = nee(v, true, x, d, wl, a.E, make_rng(a.seed, pixel, s, kDomShadow), c2, capped);
+            if (FORM == kWithPaths) val = v.albedo * (Ld + trace_path(v, x, d, wl, a.E, make_rng(a.seed, pixel, s, kDomPath), capped));
             // path mode: k_paths adds L_i and multiplies by the albedo
-            val = a.mode == RPNN_MODE_PATH ? Ld : v.albedo * Ld;
+            else val = a.mode == RPNN_MODE_PATH ? Ld : v.albedo * Ld;
         }
         if (capped) raise_status(status, kStatIterLimit);
         if (sample_val) sample_val[ps] = val;
@@ -595,6 +597,16 @@ rpnn_status launch_scatter_composite(Ctx& c, const rpnn_render_desc& rd, float a
     int64_t b = (npix + 255) / 256;
     if (b > c.num_sms * 16) b = c.num_sms * 16;
     k_composite<<<(unsigned)b, 256, 0, s>>>(sample_val, npix, rd.spp, image);
+    RPNN_CHECK_LAUNCH();
+    return RPNN_OK;
+}
+
+rpnn_status launch_primary_paths(Ctx& c, const VolumeView& vv, const rpnn_render_desc& rd, float* sample_val,
+                                 cudaStream_t s) {
+    const int64_t P = (int64_t)rd.width * rd.height * rd.spp;
+    k_primary<kWithPaths><<<(unsigned)((P + 127) / 128), 128, 0, s>>>(vv, make_args(rd), P, sample_val, nullptr, nullptr,
+                                                                     nullptr, nullptr, nullptr, nullptr, nullptr, nullptr,
+                                                                     c.status.as<uint32_t>(), nullptr, 0, 32, 0);
     RPNN_CHECK_LAUNCH();
     return RPNN_OK;
 }

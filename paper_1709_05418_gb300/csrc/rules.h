@@ -120,4 +120,17 @@ RPNN_RULE int record_lanes(int n_max, int warps) {
     return l < 32 ? (int)l : 32;
 }
 
+// Path-traced renders: whether each sample's lane of the primary pass traces its path too, instead of
+// listing it for a launch that deals the paths to lanes as they get free.  That launch wins by a
+// third where paths are long or many; between the sizes at which the chip is half empty and several
+// times full, short paths (little survives a collision, or few collisions lie across the cloud:
+// `depth`, the majorant's optical depth of the unit box) are over before it has paid for itself.  Time
+// of the second launch against the lane's own, 128^3 fBm and 64^3 blobs, 160^2 to 400^2: depth 5, any
+// albedo 1.10-1.39; 10: 0.98-1.34; 20: 0.90-1.14 (160^2: 0.90-1.07); 50: 0.76-1.06 at albedo 0.9 and above,
+// 0.86-1.13 at 0.7, 0.95-1.24 at 0.3.  512^2 x 2: 0.63-0.91 everywhere; 64^2: 0.55-1.1 above depth 2.
+RPNN_RULE bool path_in_primary(int64_t samples, float albedo, float depth, int sms) {
+    const int least = depth <= 6.0f ? 100 : (depth <= 12.0f || albedo <= 0.5f ? 160 : 240);   // samples per SM
+    return (albedo <= 0.5f || depth <= 20.0f) && samples >= least * (int64_t)sms && samples <= 1300 * (int64_t)sms;
+}
+
 }  // namespace rpnn

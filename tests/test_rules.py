@@ -28,6 +28,7 @@ int t_brick_chunk(int w) { return brick_chunk(w); }
 int t_start_lanes(int64_t n) { return record_start_lanes(n, 152); }
 int t_warps(int64_t n, int n_max) { return record_warps(n, n_max, 152); }
 int t_lanes(int n_max, int warps) { return record_lanes(n_max, warps); }
+int t_path_in_primary(int64_t P, float a, float depth) { return path_in_primary(P, a, depth, 152); }
 // polls a wait makes until it gives up, or `total` if it does not; progress every `every` polls
 int64_t t_polls(uint32_t bound, int64_t total, int64_t every) {
     PollBound w{0, 0};
@@ -65,6 +66,7 @@ def rules(tmp_path_factory):
     L.t_start_lanes.argtypes, L.t_start_lanes.restype = [ctypes.c_int64], ctypes.c_int
     L.t_warps.argtypes, L.t_warps.restype = [ctypes.c_int64, ctypes.c_int], ctypes.c_int
     L.t_lanes.argtypes, L.t_lanes.restype = [ctypes.c_int, ctypes.c_int], ctypes.c_int
+    L.t_path_in_primary.argtypes, L.t_path_in_primary.restype = [ctypes.c_int64, ctypes.c_float, ctypes.c_float], ctypes.c_int
     L.t_polls.argtypes, L.t_polls.restype = [ctypes.c_uint32, ctypes.c_int64, ctypes.c_int64], ctypes.c_int64
     return L
 
@@ -198,3 +200,16 @@ def test_few_paths_are_spread_over_a_records_warps(rules):
                 assert warps == (1 if n >= 9728 else 2 if n >= 4864 else 4)
             if n_max >= 128:
                 assert per == 32
+
+
+def test_short_paths_of_middle_sized_images_stay_in_the_primary_pass(rules):
+    """Long paths, thumbnails and large images (and with them every image of several slices) are dealt
+    to lanes by a launch of their own."""
+    for a, depth in ((0.99, 5.0), (0.9, 12.0), (0.3, 50.0), (0.5, 400.0)):
+        for side, there in ((64, 0), (160, 1), (256, 1), (400, 1), (512, 0)):
+            assert rules.t_path_in_primary(side * side, a, depth) == there, (a, depth, side)
+        assert not rules.t_path_in_primary(2 ** 24, a, depth)
+    for a, depth in ((0.99, 50.0), (0.51, 20.5), (1.0, 1000.0)):
+        assert not any(rules.t_path_in_primary(P, a, depth) for P in (1, 25600, 65536, 160000, 2 ** 31 - 1))
+    assert rules.t_path_in_primary(200 * 200, 0.99, 20.0) and not rules.t_path_in_primary(160 * 160, 0.99, 20.0)
+    assert rules.t_path_in_primary(128 * 128, 0.99, 5.0) and not rules.t_path_in_primary(128 * 128, 0.99, 10.0)
