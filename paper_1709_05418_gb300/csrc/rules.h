@@ -74,10 +74,12 @@ RPNN_RULE int64_t path_slice_smaller(int64_t slice) { return slice / 2 > kMinPat
 // fit beside one another), for `levels` of `rows` lines of nx voxels; otherwise each output is a task.
 // Streaming halves the arithmetic, but a line that does not fit is an idle slot and a block has a
 // warp per level.  Streamed and by task, nx x ny x nz: 256^3 123 and 180 us; 640 x 256^2 528 and 627;
-// 768 x 256^2 (23 lines fit) 687 and 652; 64^3 18.4 and 13.0 (64 blocks, fewer than SMs); one level
-// of 1,024 x 128 x 256, with the call around it, 612 and 262; lines under 96: within 5 % either way.
+// 768 x 256^2 (23 lines fit) 687 and 652; 160 to 384 x 5,250 lines 0.76 to 0.99 of the time by task,
+// x 4,096 lines (64 blocks or fewer, on 152 SMs) 0.86 to 1.21, 64^3 18.4 and 13.0; 96 and 128 x 10,000
+// 20.1 and 18.6, 27.9 and 26.7, x 16,384 0.89 and 0.83 of it; one level of 1,024 x 128 x 256, with the call
+// around it, 612 and 262.
 RPNN_RULE bool mip_x_streams(int nx, int64_t rows, int levels, int sms) {
-    return levels > 1 && nx >= 96 && nx <= 680 && rows >= 64 * (int64_t)sms;
+    return levels > 1 && nx >= 96 && nx <= 680 && rows >= (nx < 144 ? 100 : 33) * (int64_t)sms;
 }
 RPNN_RULE int mip_x_lines(int nx, bool stream) {
     const int most = stream ? 64 : 32, fit = (stream ? 72 : 64) * 1024 / ((nx + 1) * 4);

@@ -154,9 +154,9 @@ def test_path_renders_list_a_bounded_slice(rules):
 def test_x_pass_streams_only_with_its_slots_filled(rules):
     """Long lines, single levels and small grids keep the form whose tasks fill every lane; staged
     lines fit the shared memory the launches ask for, whatever the length."""
-    assert rules.t_x_streams(256, 256 * 256, 6) and rules.t_x_streams(96, 9728, 2)
+    assert rules.t_x_streams(256, 256 * 256, 6) and rules.t_x_streams(96, 15200, 2) and rules.t_x_streams(144, 5016, 2)
     for nx, rows, levels in ((768, 65536, 6), (1024, 2 ** 20, 8), (8192, 10 ** 6, 9), (256, 65536, 1), (64, 4096, 5),
-                             (256, 9727, 6)):
+                             (256, 5015, 6), (143, 15199, 6)):
         assert not rules.t_x_streams(nx, rows, levels), (nx, rows, levels)
     for nx in range(1, 8193):
         for stream, most in ((0, 32), (1, 64)):
