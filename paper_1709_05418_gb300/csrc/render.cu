@@ -42,11 +42,12 @@ struct PrimaryItem {
 // RPNN_MAX_BATCH renders (items[i] from block first_block on); each block copies its item
 // into shared memory and works on that render's samples, writing into its region of the
 // per-sample buffers and appending its shading points to that region with its own count.
-// PART: samples first .. P - 1, `lanes` of them per warp.  A warp's rays diverge, so where the image has
-// fewer samples than the chip holds threads, fewer of them share a warp (64 x 64 samples, this pass alone:
-// 118 us with 32 per warp, 94 with 4, about 80 with 2).  An instance of its own: with the two numbers as
-// arguments whole images of whole warps took 1 to 3 % longer (256 x 256 in a dense cloud 680 us, 658 without).
-enum PrimaryForm { kWhole, kPart, kBatched, kWithPaths };
+// kPart: `lanes` samples per warp.  A warp's rays diverge, so where the image has fewer samples than the
+// chip holds threads, fewer of them share a warp (64 x 64 samples, this pass alone: 118 us with 32 per warp,
+// 94 with 4, about 80 with 2).  kSlice: from sample `first` on, too.  Instances of their own: with the two
+// numbers as arguments whole images of whole warps took 1 to 3 % longer (256 x 256 in a dense cloud 680 us,
+// 658 without), and parts 2 % with `first`.
+enum PrimaryForm { kWhole, kPart, kSlice, kBatched, kWithPaths };
 template <PrimaryForm FORM>
 __global__ void __launch_bounds__(128, FORM == kBatched ? 5 : 6)
 k_primary(const VolumeView v_, const RenderArgs a_, int64_t P_, float* __restrict__ sample_val,
@@ -79,9 +80,10 @@ k_primary(const VolumeView v_, const RenderArgs a_, int64_t P_, float* __restric
     const RenderArgs& a = BATCH ? it.a : a_;
     const int64_t P = BATCH ? it.P : P_;
     const int warp_lane = (int)threadIdx.x & 31;
-    const int64_t ps = FORM == kPart ? first + ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * lanes + warp_lane
-                                     : (blockIdx.x - (BATCH ? it.first_block : 0)) * (int64_t)blockDim.x + threadIdx.x;
-    const bool active = ps < P && (FORM != kPart || warp_lane < lanes);
+    constexpr bool PART = FORM == kPart || FORM == kSlice;
+    const int64_t ps = PART ? ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * lanes + warp_lane + (FORM == kSlice ? first : 0)
+                            : (blockIdx.x - (BATCH ? it.first_block : 0)) * (int64_t)blockDim.x + threadIdx.x;
+    const bool active = ps < P && (!PART || warp_lane < lanes);
     int hit = 0;
     float3 x = f3(0.f, 0.f, 0.f), d = f3(0.f, 0.f, 1.f);
     float Ld = 0.0f;
@@ -578,7 +580,7 @@ rpnn_status launch_primary(Ctx& c, const VolumeView& vv, const rpnn_render_desc&
     int lanes = 2;
     while (lanes < 32 && (int64_t)lanes * c.num_sms * 20 < P) lanes *= 2;
     const int64_t blocks = (P + 4 * lanes - 1) / (4 * lanes);
-    auto* const kernel = lanes == 32 && first == 0 ? k_primary<kWhole> : k_primary<kPart>;
+    auto* const kernel = first > 0 ? k_primary<kSlice> : (lanes == 32 ? k_primary<kWhole> : k_primary<kPart>);
     kernel<<<(unsigned)blocks, 128, 0, s>>>(vv, make_args(rd), first + P, sample_val, qx, qd, qps, qcount, hit,
                                                       xo, dout, Ld, c.status.as<uint32_t>(), nullptr, 0, lanes, first);
     RPNN_CHECK_LAUNCH();
