@@ -72,14 +72,16 @@ RPNN_RULE int64_t path_slice_smaller(int64_t slice) { return slice / 2 > kMinPat
 
 // x pass of the pyramid build: whether its warps stream along lines (64 slots a warp, as many lines as
 // fit beside one another), for `levels` of `rows` lines of nx voxels; otherwise each output is a task.
-// Streaming halves the arithmetic, but a line that does not fit is an idle slot and a block has a
-// warp per level.  Streamed and by task, nx x ny x nz: 256^3 123 and 180 us; 640 x 256^2 528 and 627;
-// 768 x 256^2 (23 lines fit) 687 and 652; 160 to 384 x 5,250 lines 0.76 to 0.99 of the time by task,
-// x 4,096 lines (64 blocks or fewer, on 152 SMs) 0.86 to 1.21, 64^3 18.4 and 13.0; 96 and 128 x 10,000
-// 20.1 and 18.6, 27.9 and 26.7, x 16,384 0.89 and 0.83 of it; one level of 1,024 x 128 x 256, with the call
-// around it, 612 and 262.
+// Streaming halves the arithmetic, and a thread's chain over a long line serves all its outputs; but a
+// line that does not fit is an idle slot and a block has a warp per level.  Streamed against by task,
+// all levels together, nx x lines: 256 x 65,536 123 and 180 us; 160 to 640 x 5,250 0.76-1.0 of the time, x
+// 4,096 (64 blocks) 0.86-1.21; 96 and 128 x 10,000 1.08 and 1.04, x 16,384 0.89 and 0.83; 704 to 1,024 (25 to
+// 17 lines fit) x 65,536 0.91-1.11, x 262,144 0.91-1.06, x 6,400 1.0-1.5; 1,100 to 8,192 x 4,096 and more
+// 0.64-1.0 (1,536 x 4,096 1.19), x 256 0.88-1.1.  One level of 1,024 x 32,768, with the call around it, 612
+// and 262 us.
 RPNN_RULE bool mip_x_streams(int nx, int64_t rows, int levels, int sms) {
-    return levels > 1 && nx >= 96 && nx <= 680 && rows >= (nx < 144 ? 100 : 33) * (int64_t)sms;
+    const int least = nx < 144 ? 100 : (nx <= 680 ? 33 : (nx < 1088 ? 400 : 0));       // lines per SM
+    return levels > 1 && nx >= 96 && rows >= least * (int64_t)sms;
 }
 RPNN_RULE int mip_x_lines(int nx, bool stream) {
     const int most = stream ? 64 : 32, fit = (stream ? 72 : 64) * 1024 / ((nx + 1) * 4);

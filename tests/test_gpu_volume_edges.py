@@ -38,9 +38,9 @@ def test_stats_bricks_and_levels_equal_the_oracle(shape):
 
 
 @pytest.mark.parametrize("shape", [(124, 124, 97), (80, 124, 97), (76, 129, 287), (51, 100, 288), (76, 128, 640), (76, 128, 681),
-                                   (70, 139, 95)])
+                                   (70, 139, 95), (16, 19, 1100), (17, 19, 2500)])
 def test_levels_built_together_equal_the_oracle(shape):
-    """Enough lines for the streaming x pass (5,016 up to 680 voxels, 15,200 below 144) and just outside its range: the
+    """Enough lines for the streaming x pass (5,016 up to 680 voxels, 15,200 below 144, any from 1,088) and just outside its range: the
     levels a descriptor reads are built together, so its values are the oracle's bit for bit."""
     if not torch.cuda.is_available():
         pytest.skip("no GPU")

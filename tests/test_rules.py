@@ -151,19 +151,19 @@ def test_path_renders_list_a_bounded_slice(rules):
     assert "slice = path ? path_slice(P) : P;" in body and "q_x.reserve(slice * 3" in body
 
 
-def test_x_pass_streams_only_with_its_slots_filled(rules):
-    """Long lines, single levels and small grids keep the form whose tasks fill every lane; staged
-    lines fit the shared memory the launches ask for, whatever the length."""
-    assert rules.t_x_streams(256, 256 * 256, 6) and rules.t_x_streams(96, 15200, 2) and rules.t_x_streams(144, 5016, 2)
-    for nx, rows, levels in ((768, 65536, 6), (1024, 2 ** 20, 8), (8192, 10 ** 6, 9), (256, 65536, 1), (64, 4096, 5),
-                             (256, 5015, 6), (143, 15199, 6)):
-        assert not rules.t_x_streams(nx, rows, levels), (nx, rows, levels)
+def test_x_pass_streams_where_that_was_measured_to_pay(rules):
+    """Single levels, small grids and middling lines on few rows keep the form whose tasks fill every lane;
+    staged lines fit the shared memory the launches ask for, whatever the length."""
+    for nx, rows in ((96, 15200), (144, 5016), (256, 65536), (680, 5016), (681, 60800), (1024, 2 ** 20), (1088, 1),
+                     (8192, 10 ** 6)):
+        assert rules.t_x_streams(nx, rows, 2) and rules.t_x_streams(nx, rows, 9), (nx, rows)
+        assert not rules.t_x_streams(nx, rows, 1)
+    for nx, rows in ((64, 4096), (95, 10 ** 6), (143, 15199), (256, 5015), (768, 32768), (1024, 4096), (1087, 60799)):
+        assert not rules.t_x_streams(nx, rows, 6), (nx, rows)
     for nx in range(1, 8193):
         for stream, most in ((0, 32), (1, 64)):
             n = rules.t_x_lines(nx, stream)
             assert 1 <= n <= most and n * (nx + 1) * 4 <= 72 * 1024
-        if rules.t_x_streams(nx, 10 ** 6, 6):
-            assert rules.t_x_lines(nx, 1) >= 27
 
 
 def test_brick_rows_take_no_more_threads_than_they_need(rules):
